@@ -149,6 +149,8 @@ xt_status get_work(xt_ctx* ctx, int32_t n, Work* w, Batch** desc) {
   const size_t o_sb = off; off = align_up(off + 4 * (size_t)(kNumClasses * kNumJ));
   const size_t o_se = off; off = align_up(off + 4 * (size_t)(kNumClasses * kNumJ));
   const size_t o_heads = off; off = align_up(off + 4 * (size_t)kMaxLaunches);
+  const size_t o_left = off; off = align_up(off + 4 * (size_t)kNearBins);
+  const size_t o_tmp = off; off = align_up(off + 4 * (size_t)n);
   void* old = ctx->work;
   xt_status s = dev_alloc(ctx, &ctx->work, &ctx->work_bytes, off);
   if (s != XT_OK) return s;
@@ -162,6 +164,8 @@ xt_status get_work(xt_ctx* ctx, int32_t n, Work* w, Batch** desc) {
   w->seg_begin = (int32_t*)(base + o_sb);
   w->seg_end = (int32_t*)(base + o_se);
   w->heads = (int32_t*)(base + o_heads);
+  w->near_left = (int32_t*)(base + o_left);
+  w->near_tmp = (int32_t*)(base + o_tmp);
   return XT_OK;
 }
 
@@ -173,6 +177,8 @@ struct Plan {
   bool any_huge = false;
   int64_t slab = 0;
   bool pool_serial = true;  // global-ring launches share one pool region, in order
+  int32_t near_pairs = 0;   // pairs of the NEAR class (k_near runs when there are any)
+  int near_grid = 0;
 };
 
 int64_t next_pow2(int64_t x) { return (int64_t)1 << log2_ceil(x); }
@@ -265,8 +271,8 @@ bool lane_launch(xt_ctx* ctx, const Score& sc, int cls, int j, bool allow_gring,
   int R = ctx->forced_P == 1 ? ctx->forced_R : (t && t->P == 1 ? t->R : lane_default_R(j));
   // the packed engine's 16-row strips need more registers than it has (they
   // spill); its long buckets, and those with 4-bit row-key tags, keep 8
-  if (cls == CLS_PACKED && R > 8 && (ctx->forced_P != 1 || packed_tag_bits(j) == 4)) R = 8;
-  const int rows = cls == CLS_PACKED ? 2 * R : R;
+  if (packed_class(cls) && R > 8 && (ctx->forced_P != 1 || packed_tag_bits(j) == 4)) R = 8;
+  const int rows = packed_class(cls) ? 2 * R : R;
   const int64_t need = std::min<int64_t>((int64_t)1 << j, next_pow2(rows + 2 * (int64_t)sc.w + 2));
   const int lg = log2_ceil(need);
   const size_t ring = (size_t)kLaneThreads * lane_ring_bytes(cls, lg);
@@ -274,14 +280,14 @@ bool lane_launch(xt_ctx* ctx, const Score& sc, int cls, int j, bool allow_gring,
   if (gring && !allow_gring) return false;
   L->cls = cls; L->j_lo = j; L->j_hi = j; L->lane = true; L->P = 1; L->R = R;
   L->rs_log2 = lg; L->global_ring = gring; L->slab = gring ? ((int64_t)1 << lg) : 0;
-  const size_t smem = (gring ? 0 : ring) + (cls == CLS_PACKED ? lane_stage_bytes(j) : 0) +
+  const size_t smem = (gring ? 0 : ring) + (packed_class(cls) ? lane_stage_bytes(j) : 0) +
                       lane_pipe_bytes(cls, gring);
   const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(4, (size_t)(220 * 1024) / (smem + 1024)));
   L->grid = ctx->num_sms * per_sm;
   int k = 0;
   while ((1 << k) < ctx->match + 1) ++k;
   // packed: the anchoring shift and, above it, the row keys' step-tag bits
-  L->mparam = cls == CLS_PACKED ? (k | packed_tag_bits(j) << 8) : ctx->match + 1;
+  L->mparam = packed_class(cls) ? (k | packed_tag_bits(j) << 8) : ctx->match + 1;
   return true;
 }
 
@@ -342,6 +348,7 @@ void plan_batched(xt_ctx* ctx, const Score& sc, Plan* pl, bool allow_gring = tru
 // ---- count-aware planning (the batched path): classify runs first with
 // per-bucket flags that do not depend on the counts, then every non-empty
 // bucket is planned from its own pair count.
+constexpr int kNearLeft = 3;             // one NEAR pair in so many is left for the engines
 constexpr int32_t kBucketSmall = XT_SMALL_BUCKET;  // fewer pairs: a bucket cannot fill the GPU
 constexpr int32_t kLaneSlots = 77824;    // one-lane thread slots of a full GPU (152 x 4 x 128)
 // Built-in rule: the fewest pairs of a bucket for one lane per pair.  A pair's
@@ -418,9 +425,16 @@ Launch queue_launch(const xt_ctx* ctx, int cls, int j, int P, int R, int lg) {
 // empty buckets get no launch; a bucket too small to fill the GPU takes its
 // small-batch schedule, or by default a group schedule with enough lanes per
 // pair to fill it; larger buckets take the throughput schedule.
-void plan_counts(xt_ctx* ctx, const Score& sc, const int32_t (*cnt)[kNumJ], const JFlags& jf,
+void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFlags& jf,
                  const bool* lane_ok, Plan* pl) {
   pl->jf = jf;
+  // the NEAR class is planned for the pairs k_near is expected to leave
+  for (int j = 0; j < kNumJ; ++j) {
+    int32_t& c = cnt[CLS_NEAR][j];
+    pl->near_pairs += c;
+    c = (c + kNearLeft - 1) / kNearLeft;
+  }
+  pl->near_grid = near_grid(pl->near_pairs, ctx->num_sms);
   const bool saved = ctx->plan_small;
   // the call's estimated cells: each bucket's pairs at a query length three
   // quarters of the way up the bucket
@@ -440,7 +454,7 @@ void plan_counts(xt_ctx* ctx, const Score& sc, const int32_t (*cnt)[kNumJ], cons
       if (lane_ok[j]) long_pairs += cnt[cls][j];
   const bool long_lanes = long_pairs >= 2 * (int64_t)kLaneSlots;
   auto min_pairs = [&](int jj) { return jj >= kLongJ && long_lanes ? 0 : lane_min_pairs(jj); };
-  for (int cls = CLS_PACKED; cls <= CLS_WIDE; ++cls) {
+  for (int cls : {CLS_PACKED, CLS_NARROW, CLS_WIDE, CLS_NEAR}) {
     int prev = -1;
     for (int j = kJMax; j >= 0; --j) {
       const int32_t c = cnt[cls][j];
@@ -517,11 +531,15 @@ void plan_counts(xt_ctx* ctx, const Score& sc, const int32_t (*cnt)[kNumJ], cons
     }
   }
   ctx->plan_small = saved;
+  // the NEAR class, which waits for k_near, after the others; within each,
   // longest queries first: their pairs set the call's critical path, and the
   // launches after them fill the slots they leave (c5-mix call of 1M pairs:
   // 21.6 ms in class order, 19.7 ms in this order, both with the rings apart)
   std::stable_sort(pl->launch, pl->launch + pl->n_launch,
-                   [](const Launch& a, const Launch& b) { return a.j_hi > b.j_hi; });
+                   [](const Launch& a, const Launch& b) {
+                     const bool na = a.cls == CLS_NEAR, nb = b.cls == CLS_NEAR;
+                     return na != nb ? nb : a.j_hi > b.j_hi;
+                   });
   int32_t huge_pairs = 0;
   for (int j = 0; j < kNumJ; ++j) huge_pairs += cnt[CLS_HUGE][j];
   if (huge_pairs > 0) {
@@ -640,11 +658,14 @@ xt_status check_args(xt_ctx* ctx, const void* q_seq, int64_t q_bytes, const void
 }
 
 // The front of a call: reset counters, classify, order the queue.
-cudaError_t enqueue_front(const JFlags& jf, const Score& sc, int32_t match, const Work& w,
-                          const Batch* desc, int32_t n_cap, cudaStream_t stream) {
+cudaError_t enqueue_front(const JFlags& jf, const Score& sc, int32_t match, bool diag, bool near,
+                          const Work& w, const Batch* desc, int32_t n_cap, cudaStream_t stream) {
   cudaError_t e = cudaMemsetAsync(w.counts, 0, 4 * (size_t)kNumBuckets, stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(w.heads, 0, 4 * (size_t)kMaxLaunches, stream);
-  if (e == cudaSuccess) e = launch_classify(desc, n_cap, sc, match, jf, w, stream);
+  // the queue heads and, next to them, the counters of pairs k_near leaves
+  const size_t zero = (size_t)((const char*)(w.near_left + kNearBins) - (const char*)w.heads);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.heads, 0, zero, stream);
+  if (e == cudaSuccess && diag) e = launch_diag(desc, n_cap, sc, match, near, w, stream);
+  if (e == cudaSuccess) e = launch_classify(desc, n_cap, sc, match, jf, diag, w, stream);
   if (e == cudaSuccess) e = launch_order(desc, n_cap, w, stream);
   return e;
 }
@@ -671,15 +692,27 @@ cudaError_t enqueue_dp(xt_ctx* ctx, bool plain, const Plan& pl, int plain_rs, co
   // launch's start, and small batches fill the GPU.  Global-ring launches
   // with regions of their own fork too; sharing one region (a plan whose
   // rings exceed the pool cap or the budget) they stay in order on branch 0.
-  const int nb = std::min(ctx->branches, pl.n_launch);
+  // The near pass goes first on branch 0, and the launches of the pairs it
+  // leaves wait for it on theirs.
+  const bool near = pl.near_pairs > 0;
+  const int nb = std::min(ctx->branches, pl.n_launch + (near ? 1 : 0));
   if (e == cudaSuccess && nb > 1) {
     e = cudaEventRecord(ctx->fork_ev, stream);
     for (int b = 0; e == cudaSuccess && b < nb; ++b) e = cudaStreamWaitEvent(ctx->aux[b], ctx->fork_ev, 0);
   }
-  for (int i = 0, rr = 0; e == cudaSuccess && i < pl.n_launch; ++i) {
+  int rr = 0;
+  if (e == cudaSuccess && near) {
+    cudaStream_t st = nb > 1 ? ctx->aux[rr++] : stream;
+    e = launch_near(desc, sc, ctx->match, pl.near_grid, w, kMaxLaunches - 1, st);
+    if (e == cudaSuccess && nb > 1) e = cudaEventRecord(ctx->near_ev, st);
+    dp += 2;
+  }
+  for (int i = 0; e == cudaSuccess && i < pl.n_launch; ++i) {
     const Launch& L = pl.launch[i];
     cudaStream_t st = stream;
     if (nb > 1) st = ctx->aux[L.global_ring && pl.pool_serial ? 0 : (rr++ % nb)];
+    if (L.cls == CLS_NEAR && nb > 1) e = cudaStreamWaitEvent(st, ctx->near_ev, 0);
+    if (e != cudaSuccess) break;
     void* gring = L.global_ring ? static_cast<void*>(reinterpret_cast<char*>(ctx->pool) + L.pool_off)
                                 : nullptr;
     e = L.lane ? launch_lane(desc, sc, w, L, i, gring, st)
@@ -724,14 +757,17 @@ uint64_t plan_signature(const Plan& pl) {
     mix(L.global_ring); mix(L.slab); mix(L.grid); mix(L.mparam); mix((int64_t)L.pool_off);
   }
   mix(pl.pool_serial);
+  mix(pl.near_grid);
   for (int j = 0; j < kNumJ; ++j) mix(pl.jf.f[j]);
   return h;
 }
 
 // The first half of a call: checks, workspace, descriptor, and for the
 // batched path the classify pass and the copy of its bucket counts.  The
-// call's state waits in ctx->pending for run_finish.
-xt_status run_begin(xt_ctx* ctx, bool plain, const uint8_t* q_seq, int64_t q_bytes,
+// call's state waits in ctx->pending for run_finish.  early: the caller may
+// still be filling the sequence buffers until _finish, so only the lengths are
+// read here (no diagonal pass).
+xt_status run_begin(xt_ctx* ctx, bool plain, bool early, const uint8_t* q_seq, int64_t q_bytes,
                     const int64_t* q_off, const int32_t* q_len, const uint8_t* t_seq,
                     int64_t t_bytes, const int64_t* t_off, const int32_t* t_len,
                     const int32_t* h0, int32_t n, const xt_scoring* scr, xt_result* out,
@@ -778,7 +814,13 @@ xt_status run_begin(xt_ctx* ctx, bool plain, const uint8_t* q_seq, int64_t q_byt
     // classify and order with count-independent bucket flags, then bring the
     // pair count of every (class, bucket) back for the plan
     batched_flags(ctx, pc.sc, n, &pc.jf, pc.lane_ok);
-    e = enqueue_front(pc.jf, pc.sc, scr->match, pc.w, pc.desc, pc.n_cap, stream);
+    // a forced schedule puts every pair on that schedule's engine.  The
+    // diagonal bounds need a gap to cost something; the narrow band must lie
+    // inside the call's, and its padded columns need alpha < 128
+    const bool diag = pc.diag = ctx->near_first && !early && n >= kNearMinPairs && !ctx->forced_P &&
+                      pc.sc.alpha >= 1;
+    const bool near = diag && pc.sc.alpha <= 127 && pc.sc.w >= kNearHalf;
+    e = enqueue_front(pc.jf, pc.sc, scr->match, diag, near, pc.w, pc.desc, pc.n_cap, stream);
     const size_t seg_bytes =
         (size_t)((const char*)(pc.w.seg_end + kNumClasses * kNumJ) - (const char*)pc.w.seg_begin);
     if (e == cudaSuccess)
@@ -830,7 +872,7 @@ xt_status run_finish(xt_ctx* ctx) {
   // replay as one graph once a call with the same key has been seen
   auto body = [&](cudaStream_t st, int* dp) -> cudaError_t {
     cudaError_t r = cudaSuccess;
-    if (plain) r = enqueue_front(pl.jf, sc, pc.scr.match, w, pc.desc, pc.n_cap, st);
+    if (plain) r = enqueue_front(pl.jf, sc, pc.scr.match, false, false, w, pc.desc, pc.n_cap, st);
     if (r == cudaSuccess) r = enqueue_dp(ctx, plain, pl, plain_rs, sc, w, pc.desc, pc.n_cap, st, dp);
     return r;
   };
@@ -879,14 +921,15 @@ xt_status run_finish(xt_ctx* ctx) {
   if (ge && ge->exec) {
     e = cudaGraphLaunch(ge->exec, pc.stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
-    dp = plain ? 1 + pl.n_launch : pl.n_launch;
+    dp = (plain ? 1 : 0) + (pl.near_pairs > 0 ? 2 : 0) + pl.n_launch;
   } else {
     ctx->launch_error.clear();
     e = body(pc.stream, &dp);
     if (e != cudaSuccess) return cuda_fail(ctx, e, ("launch " + ctx->launch_error).c_str());
   }
   ctx->calls += 1;
-  ctx->launches += 4 + dp;  // descriptor, classify, scan, scatter + DP kernels
+  // descriptor, (diagonals,) classify, scan, scatter + DP kernels
+  ctx->launches += 4 + (pc.diag ? 1 : 0) + dp;
   ctx->dp_launches += dp;
   return XT_OK;
 }
@@ -895,7 +938,7 @@ xt_status run(xt_ctx* ctx, bool plain, const uint8_t* q_seq, int64_t q_bytes, co
               const int32_t* q_len, const uint8_t* t_seq, int64_t t_bytes, const int64_t* t_off,
               const int32_t* t_len, const int32_t* h0, int32_t n, const xt_scoring* scr,
               xt_result* out, int64_t* cells, cudaStream_t stream) {
-  xt_status s = run_begin(ctx, plain, q_seq, q_bytes, q_off, q_len, t_seq, t_bytes, t_off, t_len,
+  xt_status s = run_begin(ctx, plain, false, q_seq, q_bytes, q_off, q_len, t_seq, t_bytes, t_off, t_len,
                           h0, n, scr, out, cells, stream);
   if (s != XT_OK) {
     if (s != XT_EBUSY) ctx->pending.active = false;
@@ -935,6 +978,7 @@ xt_status xt_ctx_create(xt_ctx** out, int device, size_t mem_budget_bytes) {
   ok = ok && cudaHostAlloc((void**)&c->seg_host, 4 * kSegHostWords, cudaHostAllocDefault) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&c->seg_ev, cudaEventDisableTiming) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming) == cudaSuccess;
+  ok = ok && cudaEventCreateWithFlags(&c->near_ev, cudaEventDisableTiming) == cudaSuccess;
   for (int b = 0; ok && b < kMaxBranches; ++b) {
     ok = cudaStreamCreateWithFlags(&c->aux[b], cudaStreamNonBlocking) == cudaSuccess &&
          cudaEventCreateWithFlags(&c->join_ev[b], cudaEventDisableTiming) == cudaSuccess;
@@ -975,6 +1019,7 @@ xt_status xt_ctx_destroy(xt_ctx* ctx) {
   if (ctx->seg_host) cudaFreeHost(ctx->seg_host);
   if (ctx->seg_ev) cudaEventDestroy(ctx->seg_ev);
   if (ctx->fork_ev) cudaEventDestroy(ctx->fork_ev);
+  if (ctx->near_ev) cudaEventDestroy(ctx->near_ev);
   if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
   for (auto& ev : ctx->stage_ev)
     if (ev) cudaEventDestroy(ev);
@@ -1011,8 +1056,9 @@ xt_status xt_extend_batch_begin(xt_ctx* ctx, const uint8_t* q_seq, int64_t q_byt
                                 xt_result* out, int64_t* cells_out, void* stream) {
   if (!ctx) return XT_EINVAL;
   std::lock_guard<std::mutex> lk(ctx->mu);
-  const xt_status s = run_begin(ctx, false, q_seq, q_bytes, q_off, q_len, t_seq, t_bytes, t_off,
-                                t_len, h0, n_pairs, sc, out, cells_out, (cudaStream_t)stream);
+  const xt_status s = run_begin(ctx, false, true, q_seq, q_bytes, q_off, q_len, t_seq, t_bytes,
+                                t_off, t_len, h0, n_pairs, sc, out, cells_out,
+                                (cudaStream_t)stream);
   if (s != XT_OK && s != XT_EBUSY) ctx->pending.active = false;
   return s;
 }
@@ -1175,6 +1221,7 @@ xt_status chunk_contexts(xt_ctx* ctx) {
     c->forced_R = ctx->forced_R;
     c->branches = ctx->branches;
     c->graphs = ctx->graphs;
+    c->near_first = ctx->near_first;
     c->alphabet = XT_ALPHABET_CODES;
   }
   return XT_OK;
@@ -1317,9 +1364,8 @@ xt_status xt_extend_batch_host(xt_ctx* ctx, const uint8_t* q_seq, int64_t q_byte
   const uint8_t* cq = (const uint8_t*)(d + (packed ? o_qc : o_q));
   const uint8_t* ct = (const uint8_t*)(d + (packed ? o_tc : o_t));
   // Without a memory budget the chunks alternate between two contexts of
-  // their own (workspace, ring pool, streams): chunk k classifies as soon as
-  // the metadata is on the device, and its extension kernels wait only for
-  // its own bytes, so they take the slots that chunk k-1's kernels leave as
+  // their own (workspace, ring pool, streams): chunk k waits only for its own
+  // bytes, so its kernels take the slots that chunk k-1's kernels leave as
   // they drain.  Chunk k+2 reuses chunk k's context after it in stream order.
   const bool apart = ctx->budget == 0 && !ctx->timing;
   if (apart) {
@@ -1346,17 +1392,11 @@ xt_status xt_extend_batch_host(xt_ctx* ctx, const uint8_t* q_seq, int64_t q_byte
     cudaStream_t cst = apart ? cc->copy_stream : st;
     if (apart) {
       e = cudaStreamWaitEvent(cst, ev[1], 0);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(cst, ev[2 + k], 0);
       if (e != cudaSuccess) break;
-      s = run_begin(cc, false, cq, qn, dqo + p0, dql + p0, ct, tn, dto + p0, dtl + p0, dh0 + p0,
-                    p1 - p0, sc, dout + p0, dcells ? dcells + p0 : nullptr, cst);
-      if (s == XT_OK) {
-        e = cudaStreamWaitEvent(cst, ev[2 + k], 0);
-        s = e == cudaSuccess ? run_finish(cc) : cuda_fail(cc, e, "chunk bytes");
-      }
-      if (s != XT_OK) {
-        cc->pending.active = false;
-        ctx->last_error = cc->last_error;
-      }
+      s = run(cc, false, cq, qn, dqo + p0, dql + p0, ct, tn, dto + p0, dtl + p0, dh0 + p0,
+              p1 - p0, sc, dout + p0, dcells ? dcells + p0 : nullptr, cst);
+      if (s != XT_OK) ctx->last_error = cc->last_error;
     } else {
       e = cudaStreamWaitEvent(st, ev[2 + k], 0);
       if (e != cudaSuccess) break;
@@ -1589,6 +1629,8 @@ bool carve_static(void* base_ptr, int32_t n, Work* w, Batch** desc) {
   w->seg_begin = (int32_t*)(base + o_sb);
   w->seg_end = (int32_t*)(base + o_se);
   w->heads = (int32_t*)(base + o_heads);
+  w->near_left = nullptr;  // no near pass on this path
+  w->near_tmp = nullptr;
   *desc = (Batch*)(base + o_desc);
   return true;
 }
@@ -1641,7 +1683,7 @@ extern "C" xt_status xt_extend_batch_static(const uint8_t* q_seq, int64_t q_byte
   // are rewritten; everything else is written before it is read
   if (e == cudaSuccess) e = cudaMemsetAsync(w.counts, 0, 4 * (size_t)kNumBuckets, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(w.heads, 0, 4 * (size_t)kMaxLaunches, st);
-  if (e == cudaSuccess) e = launch_classify(desc, n_pairs, sc, scr->match, pl.jf, w, st);
+  if (e == cudaSuccess) e = launch_classify(desc, n_pairs, sc, scr->match, pl.jf, false, w, st);
   if (e == cudaSuccess) e = launch_order(desc, n_pairs, w, st);
   for (int i = 0; e == cudaSuccess && i < pl.n_launch; ++i) {
     const Launch& L = pl.launch[i];

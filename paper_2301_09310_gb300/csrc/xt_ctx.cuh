@@ -111,6 +111,7 @@ struct PendingCall {
   bool has_cells = false;
   cudaStream_t stream = nullptr;
   JFlags jf{};
+  bool diag = false;            // the diagonal pass ran
   bool lane_ok[kNumJ] = {};
 };
 
@@ -161,6 +162,8 @@ struct xt_ctx {
   int branches = xt::kMaxBranches;
   cudaStream_t aux[xt::kMaxBranches] = {};
   cudaEvent_t fork_ev = nullptr;
+  cudaEvent_t near_ev = nullptr;  // the near pass is done (its class's launches wait for it)
+  bool near_first = true;         // the near passes run (the autotuner times the engines without)
   cudaEvent_t join_ev[xt::kMaxBranches] = {};
   std::vector<xt::GraphEntry> graph_cache;
   int match = 1;                 // scoring of the call being planned

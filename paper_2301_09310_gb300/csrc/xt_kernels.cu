@@ -11,27 +11,6 @@
 
 namespace xt {
 
-__device__ __forceinline__ int ceil_log2(uint32_t x) {  // x >= 1
-  return x <= 1 ? 0 : 32 - __clz(x - 1);
-}
-
-// Length bucket j (qlen + 2 <= 2^j, at least kJMin) and sub-bucket: the exact
-// query length while a bucket spans at most kNumSub lengths, else its top bits.
-__device__ __forceinline__ void bucket_of(int32_t ql, int* j_out, int* sub_out) {
-  int j = ceil_log2((uint32_t)ql + 2u);
-  if (j < kJMin) j = kJMin;
-  int sub;
-  if (j == kJMin) {
-    sub = ql;
-  } else {
-    const int32_t off = ql + 2 - (1 << (j - 1));
-    sub = j <= 9 ? off : (off >> (j - 9));
-  }
-  sub = sub < 0 ? 0 : (sub >= kNumSub ? kNumSub - 1 : sub);
-  *j_out = j;
-  *sub_out = sub;
-}
-
 // ---------------------------------------------------------------- classify
 // Validates every pair, writes the results of invalid and degenerate pairs
 // directly, and assigns the others a class and a (bucket, sub-bucket) by
@@ -51,7 +30,8 @@ __device__ __forceinline__ void hist_clear(int32_t* s_hist) {
 // Class of pair k (CLS_DONE after writing the result of an invalid or
 // degenerate pair) and its histogram bin.
 __device__ __forceinline__ int classify_pair(const Batch& b, int32_t k, int32_t match,
-                                             int32_t mshift, const uint8_t* s_jf, int* bin) {
+                                             int32_t mshift, const uint8_t* s_jf, bool near,
+                                             int* bin) {
   const int64_t qo = b.q_off[k], to = b.t_off[k];
   const int32_t ql = b.q_len[k], tl = b.t_len[k], h0 = b.h0[k];
   const bool ok = h0 >= 1 && h0 <= XT_MAX_H0 && ql >= 0 && tl >= 0 && ql <= XT_MAX_LEN &&
@@ -81,13 +61,14 @@ __device__ __forceinline__ int classify_pair(const Batch& b, int32_t k, int32_t 
       bound * tag + tag - 1 <= 32767)
     cls = CLS_PACKED;
   if ((jf & kJHuge) || (cls == CLS_WIDE && (jf & kJHugeWide))) cls = CLS_HUGE;
-  *bin = (cls * kNumJ + j) * kNumSub + sub;
+  if (near && cls == CLS_PACKED) cls = CLS_NEAR;
+  *bin = bin_of(cls, j, sub);
   return cls;
 }
 
 __global__ void __launch_bounds__(kOrdThreads) k_classify(const Batch* __restrict__ bd, Score sc,
                                                           int32_t match, int32_t mshift,
-                                                          JFlags jfl, Work w) {
+                                                          JFlags jfl, bool after_diag, Work w) {
   extern __shared__ int32_t s_hist[];  // [kNumBuckets]
   // the bucket flags, indexed by a runtime bucket: shared memory, not a
   // local copy of the by-value argument
@@ -102,8 +83,10 @@ __global__ void __launch_bounds__(kOrdThreads) k_classify(const Batch* __restric
     const int64_t kk = base + r * kOrdThreads + threadIdx.x;
     if (kk < b.n) {
       const int32_t k = (int32_t)kk;
+      const uint8_t mark = after_diag ? w.pclass[k] : kRest;
+      if (mark == CLS_DONE) continue;
       int bin = 0;
-      const int cls = classify_pair(b, k, match, mshift, s_jf, &bin);
+      const int cls = classify_pair(b, k, match, mshift, s_jf, mark == CLS_NEAR, &bin);
       w.pclass[k] = (uint8_t)cls;
       if (cls < kNumClasses) atomicAdd(&s_hist[bin], 1);
     }
@@ -122,12 +105,12 @@ constexpr int kScanThreads = 1024;
 constexpr int kScanPer = (kNumBuckets + kScanThreads - 1) / kScanThreads;
 
 __device__ __forceinline__ int scan_index(int L) {  // queue position -> counter index
-  const int per_cls = kNumJ * kNumSub;
+  const int per_cls = kJSpan * kNumSub;
   const int cls = L / per_cls;
   const int rem = L - cls * per_cls;
   const int j = kJMax - rem / kNumSub;
   const int sub = kNumSub - 1 - rem % kNumSub;
-  return (cls * kNumJ + j) * kNumSub + sub;
+  return bin_of(cls, j, sub);
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan(Work w) {
@@ -167,12 +150,18 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(Work w) {
     const int L = t * kScanPer + k;
     if (L < kNumBuckets) {
       const int idx = scan_index(L);
-      const int cj = idx / kNumSub;  // cls * kNumJ + j
+      const int cls = idx / (kJSpan * kNumSub);
+      const int j = kJMin + idx / kNumSub % kJSpan;
       const int sub = idx % kNumSub;
       w.cursor[idx] = acc;
-      if (sub == kNumSub - 1) w.seg_begin[cj] = acc;
+      if (sub == kNumSub - 1) w.seg_begin[cls * kNumJ + j] = acc;
       acc += vals[k];
-      if (sub == 0) w.seg_end[cj] = acc;
+      if (sub == 0) w.seg_end[cls * kNumJ + j] = acc;
+      if (sub == 0 && j == kJMin)  // no pairs below the shortest bucket
+        for (int u = 0; u < kJMin; ++u) {
+          w.seg_begin[cls * kNumJ + u] = acc;
+          w.seg_end[cls * kNumJ + u] = acc;
+        }
     }
   }
 }
@@ -198,7 +187,7 @@ __global__ void __launch_bounds__(kOrdThreads) k_scatter(const Batch* __restrict
       if (cls < kNumClasses) {
         int j, sub;
         bucket_of(q_len[kk], &j, &sub);
-        bin[r] = (cls * kNumJ + j) * kNumSub + sub;
+        bin[r] = bin_of(cls, j, sub);
         rank[r] = atomicAdd(&s_hist[bin[r]], 1);
       }
     }
@@ -659,14 +648,15 @@ cudaError_t raise_smem_limit(K kern, size_t smem) {
 constexpr size_t kHistBytes = sizeof(int32_t) * (size_t)kNumBuckets;
 
 cudaError_t launch_classify(const Batch* bd, int32_t n_cap, const Score& sc, int32_t match,
-                            const JFlags& jf, const Work& w, cudaStream_t stream) {
+                            const JFlags& jf, bool after_diag, const Work& w,
+                            cudaStream_t stream) {
   if (n_cap == 0) return cudaSuccess;
   int mshift = 0;
   while ((1 << mshift) < match + 1) ++mshift;
   cudaError_t e = raise_smem_limit(k_classify, kHistBytes);
   if (e != cudaSuccess) return e;
   const int grid = (int)(((int64_t)n_cap + kOrdPairs - 1) / kOrdPairs);
-  k_classify<<<grid, kOrdThreads, kHistBytes, stream>>>(bd, sc, match, mshift, jf, w);
+  k_classify<<<grid, kOrdThreads, kHistBytes, stream>>>(bd, sc, match, mshift, jf, after_diag, w);
   return cudaGetLastError();
 }
 
@@ -714,13 +704,13 @@ cudaError_t launch_queue(const Batch* b, const Score& sc, const Work& w, const L
                          int head_id, int2* gring, cudaStream_t stream) {
   // packed pairs (score bound B <= 2047) fit the 32-bit row key H * 65536 + j
   // as NARROW pairs do; WIDE and HUGE pairs keep the explicit (max, column)
-  if (L.cls == CLS_NARROW || L.cls == CLS_PACKED)
+  if (L.cls == CLS_NARROW || packed_class(L.cls))
     return launch_queue_w<false>(b, sc, w, L, head_id, gring, stream);
   return launch_queue_w<true>(b, sc, w, L, head_id, gring, stream);
 }
 
 size_t lane_ring_bytes(int cls, int rs_log2) {
-  return ((size_t)1 << rs_log2) * (cls == CLS_PACKED ? sizeof(uint32_t) : sizeof(int2));
+  return ((size_t)1 << rs_log2) * (packed_class(cls) ? sizeof(uint32_t) : sizeof(int2));
 }
 
 size_t lane_stage_bytes(int j_hi) {
@@ -728,7 +718,7 @@ size_t lane_stage_bytes(int j_hi) {
 }
 
 size_t lane_pipe_bytes(int cls, bool global_ring) {
-  return (global_ring && cls != CLS_PACKED) ? (size_t)kLaneThreads * kPipeD * sizeof(int2) : 0;
+  return (global_ring && !packed_class(cls)) ? (size_t)kLaneThreads * kPipeD * sizeof(int2) : 0;
 }
 
 template <int R, bool PACKED, bool GRING, bool QSTAGE, int TB = 6>
@@ -746,7 +736,7 @@ static cudaError_t launch_lane_t(const Batch* b, const Score& sc, const Work& w,
 
 cudaError_t launch_lane(const Batch* b, const Score& sc, const Work& w, const Launch& L,
                         int head_id, void* gring, cudaStream_t stream) {
-  const bool packed = L.cls == CLS_PACKED;
+  const bool packed = packed_class(L.cls);
   const bool stage = packed && lane_stage_bytes(L.j_hi) > 0;
   // packed long buckets (no query stage): row keys with 4-bit step tags
   if (packed && (L.mparam >> 8) == 4) {

@@ -13,8 +13,13 @@ namespace xt {
 //   NARROW: 32-bit, row key H*65536 + j (h0 + match*min(qlen,tlen) <= 32767)
 //   WIDE:   32-bit with an explicit (max, column) pair per row
 //   HUGE:   band ring too large for shared memory (global slab per group)
-enum PairClass : uint8_t { CLS_PACKED = 0, CLS_NARROW = 1, CLS_WIDE = 2, CLS_HUGE = 3, CLS_DONE = 4 };
-constexpr int kNumClasses = 4;           // classes that need a DP kernel
+//   NEAR:   PACKED pairs that k_near tries on a narrow band first
+enum PairClass : uint8_t {
+  CLS_PACKED = 0, CLS_NARROW = 1, CLS_WIDE = 2, CLS_HUGE = 3, CLS_NEAR = 4, CLS_DONE = 5
+};
+constexpr int kNumClasses = 5;           // classes that need a DP kernel
+constexpr uint8_t kRest = 0xFF;          // seen by k_diag, class still to be found
+constexpr bool packed_class(int cls) { return cls == CLS_PACKED || cls == CLS_NEAR; }
 // per-bucket flags (Work::jflags)
 constexpr uint8_t kJHuge = 1;            // bucket's pairs go to the HUGE class
 constexpr uint8_t kJPacked = 2;          // bucket runs the one-lane engine: packed pairs allowed
@@ -35,7 +40,18 @@ constexpr int kJMin = 5;                 // length buckets j: qlen + 2 <= 2^j
 constexpr int kJMax = 21;
 constexpr int kNumJ = kJMax + 1;
 constexpr int kNumSub = 256;             // sub-buckets per bucket: exact query length up to 2^9
-constexpr int kNumBuckets = kNumClasses * kNumJ * kNumSub;
+constexpr int kJSpan = kJMax - kJMin + 1;
+constexpr int kNumBuckets = kNumClasses * kJSpan * kNumSub;
+// Calls of fewer pairs skip the near passes: their time is launches and one
+// pair's latency, which the passes add to (1,000 pairs of 100 bases 147 ->
+// 223 us; 5,000 of 64 bases 180 -> 164 us).
+constexpr int32_t kNearMinPairs = 4096;
+// k_near's narrow band: diagonals |i - j| <= kNearHalf; queries it takes, and
+// the calls' scoring it holds for (see xt_near.cuh)
+constexpr int kNearHalf = 15;
+constexpr int kNearJMax = 9;
+constexpr int kNearMaxQ = (1 << kNearJMax) - 2;
+constexpr int kNearBins = (kNearJMax - kJMin + 1) * kNumSub;
 constexpr int kQueueThreads = 128;       // threads per CTA of the queue kernels
 constexpr int kMaxLaunches = 64;         // queue-kernel launches per call (heads)
 
@@ -48,6 +64,8 @@ struct Work {
   int32_t* seg_begin;   // [kNumClasses * kNumJ]
   int32_t* seg_end;     // [kNumClasses * kNumJ]
   int32_t* heads;       // [kMaxLaunches]
+  int32_t* near_left;   // [kNearBins] pairs k_near left, per exact length
+  int32_t* near_tmp;    // [n] those pairs, each length's run where its queue run was
 };
 
 constexpr int kLaneThreads = 128;        // threads per CTA of the one-lane kernels
@@ -75,8 +93,18 @@ struct JFlags {
 };
 // Kernels read the batch arguments from a device copy (bd) so that one
 // captured graph serves every call; n_cap sizes the per-pair grids (>= n).
+// after_diag: launch_diag ran before on the same stream (w.pclass holds its marks).
 cudaError_t launch_classify(const Batch* bd, int32_t n_cap, const Score& sc, int32_t match,
-                            const JFlags& jf, const Work& w, cudaStream_t stream);
+                            const JFlags& jf, bool after_diag, const Work& w, cudaStream_t stream);
+// Settle the pairs whose diagonal alone decides; mark the others for classify
+// (near: CLS_NEAR where k_near may settle them).
+cudaError_t launch_diag(const Batch* bd, int32_t n_cap, const Score& sc, int32_t match, bool near,
+                        const Work& w, cudaStream_t stream);
+// The NEAR class on its narrow band; its segment table and queue region then
+// hold the pairs left, longest first.
+int near_grid(int32_t pairs, int num_sms);
+cudaError_t launch_near(const Batch* bd, const Score& sc, int32_t match, int grid, const Work& w,
+                        int head_id, cudaStream_t stream);
 cudaError_t launch_order(const Batch* bd, int32_t n_cap, const Work& w, cudaStream_t stream);
 cudaError_t launch_queue(const Batch* bd, const Score& sc, const Work& w, const Launch& L,
                          int head_id, int2* gring, cudaStream_t stream);
@@ -123,5 +151,34 @@ size_t lane_stage_bytes(int j_hi);
 // Ring-feed slot bytes per CTA of a one-lane launch (global rings of 32-bit pairs).
 size_t lane_pipe_bytes(int cls, bool global_ring);
 int max_smem_per_block_optin(int device);
+
+__device__ __forceinline__ int ceil_log2(uint32_t x) {  // x >= 1
+  return x <= 1 ? 0 : 32 - __clz(x - 1);
+}
+
+// Length bucket j (qlen + 2 <= 2^j, at least kJMin) and sub-bucket: the exact
+// query length while a bucket spans at most kNumSub lengths, else its top bits.
+__device__ __forceinline__ void bucket_of(int32_t ql, int* j_out, int* sub_out) {
+  int j = ceil_log2((uint32_t)ql + 2u);
+  if (j < kJMin) j = kJMin;
+  int sub;
+  if (j == kJMin) {
+    sub = ql;
+  } else {
+    const int32_t off = ql + 2 - (1 << (j - 1));
+    sub = j <= 9 ? off : (off >> (j - 9));
+  }
+  sub = sub < 0 ? 0 : (sub >= kNumSub ? kNumSub - 1 : sub);
+  *j_out = j;
+  *sub_out = sub;
+}
+
+// Counter of a (class, bucket, sub-bucket), and of a NEAR pair k_near left.
+__host__ __device__ __forceinline__ int bin_of(int cls, int j, int sub) {
+  return (cls * kJSpan + j - kJMin) * kNumSub + sub;
+}
+__host__ __device__ __forceinline__ int near_bin(int j, int sub) {
+  return (j - kJMin) * kNumSub + sub;
+}
 
 }  // namespace xt

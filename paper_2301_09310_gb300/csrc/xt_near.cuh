@@ -1,0 +1,95 @@
+// xt_near.cuh -- the bounds under which a pair whose query nearly matches its
+// target is extended without its whole band.
+//
+// Notation: a = match, o = gap_open, e = gap_extend, P_k = h0 + a (k + 1).
+// No cell (i, j) exceeds P_min(i,j) (every base a match, no gap), and a path
+// that opens a gap and moves d diagonals away from the seed's has paid at
+// least o + e d of that.  Cells on the diagonals |i - j| <= c are extended
+// exactly (c = 0: base by base; c > 0: a band of 2c + 1 diagonals), giving
+// lower bounds H' <= H; every path that leaves those diagonals is worth at
+// most P - Q, Q = o + e (c + 1).  So, with best_i the running best of the
+// near rows:
+//   (1) P_min(i, qlen-1) - best_i < Q on every row i: no cell outside raises
+//       the best or ties the row maximum of a row that does, so score, qle,
+//       tle and max_off are the near ones;
+//   (2) the near end-to-end score g > 0 and P_(qlen-1) - g < Q: gscore and
+//       gtle are the near ones.  Rows from qlen on hold at most
+//       P_(qlen-1) - o - e (i - qlen + 1), so once that is <= g no later row
+//       changes anything;
+//   (3) z-drop: a row's true maximum is at least the near one, so best_i -
+//       m'_i <= zdrop excludes a stop on the rows extended.  Later rows hold
+//       the deletion run from the end cell (row r, column qlen-1), and their
+//       drop is at most best - g + o + e (d_best - d_end), d the diagonal
+//       i - j of the best and of the end cell;
+//   (4) the last live row (the cells output counts rows up to it): the
+//       deletion run from the end cell reaches the last row of the band or of
+//       the target; or no path can live longer: a path's last row is at most
+//       qlen-1 + (Y - o - 1) / e with Y the largest H(i,j) + e (i - j), and Y
+//       is at most max(best, P_(qlen-1) - o, g + e d_end) -- when the last
+//       is the largest, the run itself attains the bound.
+// A pair that fails any of these is extended over its whole band as before.
+#pragma once
+#include <cstdint>
+
+#include "xt_common.cuh"
+
+namespace xt {
+
+// Bases of one sequence, eight per step, read as aligned 8-byte words of the
+// caller's buffer [lo, hi); a word that is not wholly inside it is put
+// together from its bytes that are.
+struct ByteStream {
+  const uint8_t* lo;
+  const uint8_t* hi;
+  const uint8_t* at;  // the aligned word after cur
+  uint64_t cur;
+  int sh;
+  __device__ __forceinline__ uint64_t word(const uint8_t* p) const {
+    if (p >= lo && p + 8 <= hi) return __ldg(reinterpret_cast<const unsigned long long*>(p));
+    uint64_t v = 0;
+    if (p + 8 > lo && p < hi)
+      for (int k = 0; k < 8; ++k)
+        if (p + k >= lo && p + k < hi) v |= (uint64_t)__ldg(p + k) << (8 * k);
+    return v;
+  }
+  __device__ __forceinline__ void init(const uint8_t* buf, int64_t bytes, const uint8_t* p) {
+    lo = buf;
+    hi = buf + bytes;
+    const uint8_t* a = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)7);
+    sh = (int)(reinterpret_cast<uintptr_t>(p) & 7) * 8;
+    cur = word(a);
+    at = a + 8;
+  }
+  // the next eight bytes (those outside the buffer 0)
+  __device__ __forceinline__ uint64_t next() {
+    const uint64_t n = word(at);
+    at += 8;
+    const uint64_t v = sh ? (cur >> sh) | (n << (64 - sh)) : cur;
+    cur = n;
+    return v;
+  }
+};
+
+// What the near part of a pair found; diagonals are i - j.
+struct NearEnd {
+  int32_t best, d_best;  // local best and its diagonal
+  int32_t g, row;        // end-to-end score and its row
+};
+
+// Conditions (3), after the rows extended, and (4): the last live row, or -1
+// when it is not known.
+__device__ __forceinline__ int32_t near_last_row(const NearEnd& n, int32_t qlen, int32_t tlen,
+                                                 int32_t h0, int32_t match, const Score& sc) {
+  const int64_t e = sc.beta, o = sc.alpha - sc.beta;
+  const int64_t d_end = n.row - (qlen - 1);
+  if (sc.zdrop > 0 && n.best - n.g + o + e * (n.d_best - d_end) > sc.zdrop) return -1;
+  const int64_t cap = min((int64_t)tlen - 1, (int64_t)qlen - 1 + sc.w);
+  if (cap <= n.row || e * (cap - n.row) <= (int64_t)n.g - o - 1) return (int32_t)cap;
+  const int64_t y = n.g + e * d_end;
+  const int64_t p = h0 + (int64_t)match * qlen;
+  if (e == 0 || d_end < 0 || y < n.best || p - y > o) return -1;
+  const int64_t k = y - o - 1 >= 0 ? (y - o - 1) / e : 0;
+  return (int32_t)min(cap, max((int64_t)n.row, qlen - 1 + k));
+}
+
+}  // namespace xt

@@ -474,6 +474,21 @@ xt_status xt_autotune(xt_ctx* ctx, const xt_scoring* sc, int j_max, double cells
     }
   }
   if (cudaSetDevice(ctx->device) != cudaSuccess) return XT_ECUDA;
+  // the trials time the engines: without the near passes, which would settle
+  // most trial pairs before any engine saw them
+  struct EnginesOnly {
+    xt_ctx* c;
+    bool saved;
+    explicit EnginesOnly(xt_ctx* ctx) : c(ctx) {
+      std::lock_guard<std::mutex> lk(c->mu);
+      saved = c->near_first;
+      c->near_first = false;
+    }
+    ~EnginesOnly() {
+      std::lock_guard<std::mutex> lk(c->mu);
+      c->near_first = saved;
+    }
+  } engines_only(ctx);
   Entry entry;
   entry.device = device_name(ctx->device);
   entry.sms = ctx->num_sms;
