@@ -198,6 +198,13 @@ const BucketSched* tuned(const xt_ctx* ctx, int w, int j) {
   return nullptr;
 }
 
+// Whether bucket j has a tuned schedule for band w in either size class.
+bool tuned_any(const xt_ctx* ctx, int w, int j) {
+  for (const auto& t : ctx->tuning)
+    if (t.w == w && (t.small[j].P > 0 || t.b[j].P > 0)) return true;
+  return false;
+}
+
 // Ring entries (log2) of a group-engine pair of bucket j under band w.
 int queue_ring_log2(int j, int w, int P, int R) {
   return log2_ceil(std::min<int64_t>((int64_t)1 << j, next_pow2((int64_t)P * R + 2 * (int64_t)w + 2)));
@@ -292,7 +299,7 @@ bool lane_launch(xt_ctx* ctx, const Score& sc, int cls, int j, bool allow_gring,
 }
 
 bool same_config(const Launch& a, const Launch& b) {
-  return a.cls == b.cls && a.lane == b.lane && a.P == b.P && a.R == b.R &&
+  return a.cls == b.cls && a.lane == b.lane && a.band == b.band && a.P == b.P && a.R == b.R &&
          a.rs_log2 == b.rs_log2 && a.global_ring == b.global_ring && a.grid == b.grid &&
          a.mparam == b.mparam;
 }
@@ -373,6 +380,8 @@ inline double band_cells_est(double q, int w) {
 void batched_flags(xt_ctx* ctx, const Score& sc, int32_t n, JFlags* jf, bool* lane_ok) {
   *jf = JFlags{};
   for (int j = 0; j < kNumJ; ++j) lane_ok[j] = false;
+  int bP, bK;
+  const bool band = ctx->near_first && !ctx->forced_P && band_shape(sc, ctx->match, &bP, &bK);
   const bool saved = ctx->plan_small;
   for (int j = kJMin; j <= kJMax; ++j) {
     Launch L;
@@ -391,8 +400,11 @@ void batched_flags(xt_ctx* ctx, const Score& sc, int32_t n, JFlags* jf, bool* la
     }
     lane_ok[j] = want && lane_launch(ctx, sc, CLS_PACKED, j, true, &L) &&
                  lane_launch(ctx, sc, CLS_NARROW, j, true, &L);
+    const bool banded = band && j >= kBandJMin && !tuned_any(ctx, sc.w, j);
+    if (banded) jf->f[j] |= kJBand;
     if (lane_ok[j])
-      jf->f[j] |= kJPacked | (packed_tag_bits(j) == 4 && n >= kTag4MinPairs ? kJTag4 : 0);
+      jf->f[j] |= kJPacked |
+                  (packed_tag_bits(j) == 4 && n >= kTag4MinPairs && !banded ? kJTag4 : 0);
     // the default rule's answer (tuned group schedules always fit, see
     // bucket_sched_ok, but a bucket's class must not depend on its count)
     const int fP = ctx->forced_P;
@@ -454,7 +466,10 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
       if (lane_ok[j]) long_pairs += cnt[cls][j];
   const bool long_lanes = long_pairs >= 2 * (int64_t)kLaneSlots;
   auto min_pairs = [&](int jj) { return jj >= kLongJ && long_lanes ? 0 : lane_min_pairs(jj); };
-  for (int cls : {CLS_PACKED, CLS_NARROW, CLS_WIDE, CLS_NEAR}) {
+  // one launch takes the BAND class, longest queries first
+  int32_t band_pairs = 0;
+  for (int j = 0; j < kNumJ; ++j) band_pairs += cnt[CLS_BAND][j];
+  for (int cls : {CLS_PACKED, CLS_NARROW, CLS_WIDE, CLS_NEAR, CLS_BAND}) {
     int prev = -1;
     for (int j = kJMax; j >= 0; --j) {
       const int32_t c = cnt[cls][j];
@@ -462,8 +477,12 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
       const int jj = j < kJMin ? kJMin : j;   // classify clamps short queries into kJMin
       ctx->plan_small = c < kBucketSmall;
       Launch L;
-      bool lane = false;
-      if (cls != CLS_WIDE && lane_ok[jj]) {
+      bool lane = false, band = false;
+      if (cls == CLS_BAND) {
+        band = true;  // classify gives the class to buckets the band engine takes
+        band_shape(sc, ctx->match, &L.P, &L.R);
+        L.cls = cls; L.band = true; L.grid = band_grid(L.P, band_pairs, ctx->num_sms);
+      } else if (cls != CLS_WIDE && lane_ok[jj]) {
         lane = true;
         if (ctx->forced_P > 1) {
           lane = false;
@@ -481,7 +500,8 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
                                            (double)kLaneSlots <= est_cells;
         }
       }
-      if (lane) {
+      if (band) {
+      } else if (lane) {
         lane_launch(ctx, sc, cls, jj, true, &L);
       } else {
         int P = 0, R = 8, lg = 0;
@@ -715,8 +735,9 @@ cudaError_t enqueue_dp(xt_ctx* ctx, bool plain, const Plan& pl, int plain_rs, co
     if (e != cudaSuccess) break;
     void* gring = L.global_ring ? static_cast<void*>(reinterpret_cast<char*>(ctx->pool) + L.pool_off)
                                 : nullptr;
-    e = L.lane ? launch_lane(desc, sc, w, L, i, gring, st)
-               : launch_queue(desc, sc, w, L, i, static_cast<int2*>(gring), st);
+    e = L.band   ? launch_band(desc, sc, ctx->match, w, L, i, ctx->num_sms, st)
+        : L.lane ? launch_lane(desc, sc, w, L, i, gring, st)
+                 : launch_queue(desc, sc, w, L, i, static_cast<int2*>(gring), st);
     if (e != cudaSuccess) {
       char buf[192];
       std::snprintf(buf, sizeof(buf),
@@ -753,7 +774,7 @@ uint64_t plan_signature(const Plan& pl) {
   mix(pl.n_launch);
   for (int i = 0; i < pl.n_launch; ++i) {
     const Launch& L = pl.launch[i];
-    mix(L.cls); mix(L.j_lo); mix(L.j_hi); mix(L.lane); mix(L.P); mix(L.R); mix(L.rs_log2);
+    mix(L.cls); mix(L.j_lo); mix(L.j_hi); mix(L.lane); mix(L.band); mix(L.P); mix(L.R); mix(L.rs_log2);
     mix(L.global_ring); mix(L.slab); mix(L.grid); mix(L.mparam); mix((int64_t)L.pool_off);
   }
   mix(pl.pool_serial);

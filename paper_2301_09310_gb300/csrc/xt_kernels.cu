@@ -60,6 +60,7 @@ __device__ __forceinline__ int classify_pair(const Batch& b, int32_t k, int32_t 
   if (!wide && (jf & kJPacked) && ((bound + 1) << mshift) <= 32767 &&
       bound * tag + tag - 1 <= 32767)
     cls = CLS_PACKED;
+  if (cls == CLS_NARROW && (jf & kJBand) && ((bound + 1) << mshift) <= 32767) cls = CLS_BAND;
   if ((jf & kJHuge) || (cls == CLS_WIDE && (jf & kJHugeWide))) cls = CLS_HUGE;
   if (near && cls == CLS_PACKED) cls = CLS_NEAR;
   *bin = bin_of(cls, j, sub);
@@ -704,7 +705,7 @@ cudaError_t launch_queue(const Batch* b, const Score& sc, const Work& w, const L
                          int head_id, int2* gring, cudaStream_t stream) {
   // packed pairs (score bound B <= 2047) fit the 32-bit row key H * 65536 + j
   // as NARROW pairs do; WIDE and HUGE pairs keep the explicit (max, column)
-  if (L.cls == CLS_NARROW || packed_class(L.cls))
+  if (L.cls == CLS_NARROW || L.cls == CLS_BAND || packed_class(L.cls))
     return launch_queue_w<false>(b, sc, w, L, head_id, gring, stream);
   return launch_queue_w<true>(b, sc, w, L, head_id, gring, stream);
 }

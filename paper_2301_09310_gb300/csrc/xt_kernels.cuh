@@ -14,10 +14,13 @@ namespace xt {
 //   WIDE:   32-bit with an explicit (max, column) pair per row
 //   HUGE:   band ring too large for shared memory (global slab per group)
 //   NEAR:   PACKED pairs that k_near tries on a narrow band first
+//   BAND:   NARROW pairs whose scores fit 16 bits under the anchoring
+//           multiplier, in buckets the band engine takes
 enum PairClass : uint8_t {
-  CLS_PACKED = 0, CLS_NARROW = 1, CLS_WIDE = 2, CLS_HUGE = 3, CLS_NEAR = 4, CLS_DONE = 5
+  CLS_PACKED = 0, CLS_NARROW = 1, CLS_WIDE = 2, CLS_HUGE = 3, CLS_NEAR = 4, CLS_BAND = 5,
+  CLS_DONE = 6
 };
-constexpr int kNumClasses = 5;           // classes that need a DP kernel
+constexpr int kNumClasses = 6;           // classes that need a DP kernel
 constexpr uint8_t kRest = 0xFF;          // seen by k_diag, class still to be found
 constexpr bool packed_class(int cls) { return cls == CLS_PACKED || cls == CLS_NEAR; }
 // per-bucket flags (Work::jflags)
@@ -25,6 +28,7 @@ constexpr uint8_t kJHuge = 1;            // bucket's pairs go to the HUGE class
 constexpr uint8_t kJPacked = 2;          // bucket runs the one-lane engine: packed pairs allowed
 constexpr uint8_t kJHugeWide = 4;        // the bucket's WIDE pairs (group engine only) are HUGE
 constexpr uint8_t kJTag4 = 8;            // packed row keys of the bucket carry 4-bit step tags
+constexpr uint8_t kJBand = 16;           // bucket's NARROW pairs may go to the BAND class
 // Step-tag bits of the packed row keys (H * 2^bits + step in 16 bits) in
 // bucket j: 6 (H <= 511) up to queries of 510 bases, 4 (H <= 2047, folded
 // every 16 steps) beyond, where a pair's score bound grows past 511.
@@ -40,6 +44,9 @@ constexpr int kJMin = 5;                 // length buckets j: qlen + 2 <= 2^j
 constexpr int kJMax = 21;
 constexpr int kNumJ = kJMax + 1;
 constexpr int kNumSub = 256;             // sub-buckets per bucket: exact query length up to 2^9
+// buckets the band engine takes: queries of 511 bases and longer (streams of
+// 55k / 885k pairs 2.71 / 14.1 -> 1.62 / 9.9 ms)
+constexpr int kBandJMin = 10;
 constexpr int kJSpan = kJMax - kJMin + 1;
 constexpr int kNumBuckets = kNumClasses * kJSpan * kNumSub;
 // Calls of fewer pairs skip the near passes: their time is launches and one
@@ -77,6 +84,7 @@ constexpr int kLaneStageJMax = 9;        // one-lane kernels stage queries up to
 struct Launch {
   int cls = 0, j_lo = 0, j_hi = 0;
   bool lane = false;         // one-lane engine (k_lane) instead of the group engine (k_queue)
+  bool band = false;         // band engine (k_band): P lanes of R slots
   int P = 1, R = 8;          // lanes per pair, rows per lane-strip (per half when packed)
   int rs_log2 = 0;           // ring entries per group = 1 << rs_log2
   bool global_ring = false;  // ring in a global slab per group instead of shared memory
@@ -112,6 +120,12 @@ cudaError_t launch_plain(const Batch* bd, int32_t n_cap, const Score& sc, const 
                          int rs_log2, cudaStream_t stream);
 cudaError_t launch_lane(const Batch* bd, const Score& sc, const Work& w, const Launch& L,
                         int head_id, void* gring, cudaStream_t stream);
+// The band engine's lanes per pair and slots per lane for a scoring; false
+// where it does not hold the band or the scoring's row keys.
+bool band_shape(const Score& sc, int32_t match, int* P, int* K);
+int band_grid(int P, int32_t pairs, int num_sms);
+cudaError_t launch_band(const Batch* bd, const Score& sc, int32_t match, const Work& w,
+                        const Launch& L, int head_id, int num_sms, cudaStream_t stream);
 // ASCII letters to base codes (A/C/G/T either case -> 0..3, else 4), n bytes.
 cudaError_t launch_ascii_codes(const uint8_t* in, uint8_t* out, int64_t n, int num_sms,
                                cudaStream_t stream);

@@ -24,11 +24,12 @@ __device__ __forceinline__ bool diag_scan(const Batch& b, const Pair& pr, const 
   const int32_t loss_n = match - (int32_t)(int8_t)(sc.nnnn & 0xFF);
   const int32_t limit = sc.alpha - 1;
   ByteStream qs, ts;
-  qs.init(b.q_seq, b.q_bytes, pr.q);
-  ts.init(b.t_seq, b.t_bytes, pr.t);
+  const uint8_t *qe = b.q_seq + b.q_bytes, *te = b.t_seq + b.t_bytes;
+  qs.init(b.q_seq, qe, pr.q);
+  ts.init(b.t_seq, te, pr.t);
   int32_t g = pr.h0, best = pr.h0, at = -1, lost = 0, pos = 0;
   for (int32_t c = 0; c < pr.qlen; c += 8) {
-    const uint64_t x = qs.next(), y = ts.next();
+    const uint64_t x = qs.next(b.q_seq, qe), y = ts.next(b.t_seq, te);
     const uint64_t any_n = (x | y) & 0xFCFCFCFCFCFCFCFCull;  // a code of 4 or more
     const uint64_t z = (x ^ y) | any_n;
     uint64_t bad = (((z & 0x7F7F7F7F7F7F7F7Full) + 0x7F7F7F7F7F7F7F7Full) | z) & 0x8080808080808080ull;
@@ -117,25 +118,6 @@ constexpr int kC = kNearHalf;
 constexpr int kSlots = 2 * kC + 1;
 constexpr int kKeyBits = 5;
 static_assert(kSlots < (1 << kKeyBits) && kSlots <= 32, "slot index fits the row key");
-constexpr uint32_t kPadCode = 5u;  // columns past the query: score kPadScore
-constexpr uint32_t kPadScore = 0x80u;
-
-// Eight base codes (bytes) as nibbles, codes above 4 as 4, those at positions
-// left.. as kPadCode.
-__device__ __forceinline__ uint32_t nibbles(uint64_t v, int32_t left) {
-  uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32);
-  if (((lo + 0x7B7B7B7Bu) | lo | (hi + 0x7B7B7B7Bu) | hi) & 0x80808080u) {  // some byte above 4
-    lo = __vminu4(lo, 0x04040404u);
-    hi = __vminu4(hi, 0x04040404u);
-  }
-  uint32_t w = prmt(lo | (lo >> 4), hi | (hi >> 4), 0x6420u);
-  if (left < 8) {
-    const uint32_t keep = left <= 0 ? 0u : (1u << (4 * left)) - 1u;
-    w = (w & keep) | (0x11111111u * kPadCode & ~keep);
-  }
-  return w;
-}
-
 // Two pairs per lane, one in each 16-bit half of every register.  A row's
 // kSlots cells sit in registers by diagonal: slot s of row i is column
 // i - kC + s, so the diagonal neighbour of the row above has the same slot
@@ -155,8 +137,8 @@ __device__ __forceinline__ uint32_t nibbles(uint64_t v, int32_t left) {
 // 31 diagonals are what two pairs' cells, with 16 bits each, leave of 168
 // registers; they admit a loss of 21 against a perfect match.
 __global__ void __launch_bounds__(kNearThreads, kNearBlocks)
-    k_near(const Batch* __restrict__ bd, Score sc, Work w, int32_t match, int32_t mshift,
-           int head_id) {
+    k_near(const Batch* __restrict__ bd, Score sc, Work w, int32_t match, uint32_t mcm,
+           uint32_t kmul, int head_id) {
   __shared__ Batch s_b;
   __shared__ uint32_t s_tbl[8];
   __shared__ uint32_t s_row[kSlots][kNearThreads];
@@ -174,7 +156,6 @@ __global__ void __launch_bounds__(kNearThreads, kNearBlocks)
   const int32_t alpha = sc.alpha, beta = sc.beta, gopen = alpha - beta;
   const uint32_t na2 = pack16(-alpha, -alpha), nb2 = pack16(-beta, -beta);
   const uint32_t nn = (sc.nnnn & 0xFFu) | (kPadScore << 8);
-  const uint32_t mcm = 1u << mshift;
   const uint32_t a2 = pack16(match, match);
   const int32_t qbound = gopen + beta * (kC + 1);  // Q
   for (;;) {
@@ -195,8 +176,8 @@ __global__ void __launch_bounds__(kNearThreads, kNearBlocks)
       tl[h] = k >= 0 ? b.t_len[k] : 1;
       h0[h] = k >= 0 ? b.h0[k] : 1;
       rmax[h] = k >= 0 ? min(tl[h] - 1, ql[h] - 1 + kC) : -1;
-      qs[h].init(b.q_seq, b.q_bytes, b.q_seq + (k >= 0 ? b.q_off[k] : 0) - kC);
-      ts[h].init(b.t_seq, b.t_bytes, b.t_seq + (k >= 0 ? b.t_off[k] : 0));
+      qs[h].init(b.q_seq, b.q_seq + b.q_bytes, b.q_seq + (k >= 0 ? b.q_off[k] : 0) - kC);
+      ts[h].init(b.t_seq, b.t_seq + b.t_bytes, b.t_seq + (k >= 0 ? b.t_off[k] : 0));
       if (k >= 0) act |= 0xFFFFu << (16 * h);
     }
     const int32_t rows = __reduce_max_sync(0xffffffffu, max(rmax[0], rmax[1])) + 1;
@@ -224,11 +205,11 @@ __global__ void __launch_bounds__(kNearThreads, kNearBlocks)
 #pragma unroll
     for (int u = 0; u < 5; ++u, qpos += 8)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) win[h][u] = nibbles(qs[h].next(), ql[h] - qpos);
+      for (int h = 0; h < 2; ++h) win[h][u] = nibbles(qs[h].next(b.q_seq, b.q_seq + b.q_bytes), ql[h] - qpos);
     for (int32_t i8 = 0; i8 < rows; i8 += 8) {
       uint32_t tw[2];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) tw[h] = nibbles(ts[h].next(), 8);
+      for (int h = 0; h < 2; ++h) tw[h] = nibbles(ts[h].next(b.t_seq, b.t_seq + b.t_bytes), 8);
       const int32_t i_end = min(i8 + 8, rows);
 #pragma unroll 1
       for (int32_t i = i8; i < i_end; ++i) {
@@ -258,9 +239,7 @@ __global__ void __launch_bounds__(kNearThreads, kNearBlocks)
           const uint32_t f = F[s];
           const uint32_t h2 = __vimax3_s16x2(M, E, f);
           HA = add16x2(h2, na2);
-          asm("max.s16x2 %0, %0, %1;"
-              : "+r"(key)
-              : "r"(h2 * (1u << kKeyBits) + (uint32_t)s * 0x00010001u));
+          key = __viaddmax_s16x2(h2 * kmul, (uint32_t)s * 0x00010001u, key);
           if (s) F[s - 1] = __viaddmax_s16x2_relu(f, nb2, HA);
           H[s] = h2;
         }
@@ -325,7 +304,7 @@ __global__ void __launch_bounds__(kNearThreads, kNearBlocks)
       for (int h = 0; h < 2; ++h) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) win[h][u] = win[h][u + 1];
-        win[h][4] = nibbles(qs[h].next(), ql[h] - qpos);
+        win[h][4] = nibbles(qs[h].next(b.q_seq, b.q_seq + b.q_bytes), ql[h] - qpos);
       }
       qpos += 8;
     }
@@ -421,7 +400,7 @@ cudaError_t launch_near(const Batch* bd, const Score& sc, int32_t match, int gri
   if (grid <= 0) return cudaSuccess;
   int mshift = 0;
   while ((1 << mshift) < match + 1) ++mshift;
-  k_near<<<grid, kNearThreads, 0, stream>>>(bd, sc, w, match, mshift, head_id);
+  k_near<<<grid, kNearThreads, 0, stream>>>(bd, sc, w, match, 1u << mshift, 1u << kKeyBits, head_id);
   k_near_gather<<<64, kGatherThreads, 0, stream>>>(w);
   return cudaGetLastError();
 }
