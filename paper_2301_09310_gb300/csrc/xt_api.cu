@@ -677,14 +677,12 @@ xt_status check_args(xt_ctx* ctx, const void* q_seq, int64_t q_bytes, const void
   return XT_OK;
 }
 
-// The front of a call: reset counters, classify, order the queue.
+// The front of a call: classify, order the queue (launch_store_desc ran before
+// and reset the counters).
 cudaError_t enqueue_front(const JFlags& jf, const Score& sc, int32_t match, bool diag, bool near,
                           const Work& w, const Batch* desc, int32_t n_cap, cudaStream_t stream) {
-  cudaError_t e = cudaMemsetAsync(w.counts, 0, 4 * (size_t)kNumBuckets, stream);
-  // the queue heads and, next to them, the counters of pairs k_near leaves
-  const size_t zero = (size_t)((const char*)(w.near_left + kNearBins) - (const char*)w.heads);
-  if (e == cudaSuccess) e = cudaMemsetAsync(w.heads, 0, zero, stream);
-  if (e == cudaSuccess && diag) e = launch_diag(desc, n_cap, sc, match, near, w, stream);
+  cudaError_t e = cudaSuccess;
+  if (diag) e = launch_diag(desc, n_cap, sc, match, near, w, stream);
   if (e == cudaSuccess) e = launch_classify(desc, n_cap, sc, match, jf, diag, w, stream);
   if (e == cudaSuccess) e = launch_order(desc, n_cap, w, stream);
   return e;
@@ -829,7 +827,7 @@ xt_status run_begin(xt_ctx* ctx, bool plain, bool early, const uint8_t* q_seq, i
   hb.q_seq = q_seq; hb.t_seq = t_seq; hb.q_off = q_off; hb.t_off = t_off; hb.q_len = q_len;
   hb.t_len = t_len; hb.h0 = h0; hb.q_bytes = q_bytes; hb.t_bytes = t_bytes; hb.n = n;
   hb.out = out; hb.cells = cells;
-  e = launch_store_desc(pc.desc, hb, stream);
+  e = launch_store_desc(pc.desc, hb, pc.w, stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "descriptor");
   if (!plain) {
     // classify and order with count-independent bucket flags, then bring the
@@ -1699,11 +1697,9 @@ extern "C" xt_status xt_extend_batch_static(const uint8_t* q_seq, int64_t q_byte
   // the descriptor travels to its device slot as a kernel parameter: no
   // host buffer has to outlive the call, and no copy waits behind bulk
   // copies that other streams queued on the copy engine
-  cudaError_t e = launch_store_desc(desc, b, st);
-  // counters and queue heads start at zero on every call; the bucket flags
-  // are rewritten; everything else is written before it is read
-  if (e == cudaSuccess) e = cudaMemsetAsync(w.counts, 0, 4 * (size_t)kNumBuckets, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(w.heads, 0, 4 * (size_t)kMaxLaunches, st);
+  cudaError_t e = launch_store_desc(desc, b, w, st);
+  // (it zeroes the counters and queue heads; everything else is written before
+  // it is read)
   if (e == cudaSuccess) e = launch_classify(desc, n_pairs, sc, scr->match, pl.jf, false, w, st);
   if (e == cudaSuccess) e = launch_order(desc, n_pairs, w, st);
   for (int i = 0; e == cudaSuccess && i < pl.n_launch; ++i) {

@@ -89,9 +89,9 @@ struct ChunkStarts {
 };
 // ends[2k], ends[2k+1]: how far chunk k's pairs read into the query and the
 // target buffer (see xt_stage.cu); ends must be zeroed first.
-// Store a call's batch descriptor into device memory (one thread; the
-// descriptor travels as a kernel parameter).
-cudaError_t launch_store_desc(Batch* dst, const Batch& b, cudaStream_t stream);
+// Store a call's batch descriptor into device memory (it travels as a kernel
+// parameter) and zero the bin counts, queue heads and near counters.
+cudaError_t launch_store_desc(Batch* dst, const Batch& b, const Work& w, cudaStream_t stream);
 cudaError_t launch_chunk_ends(const int64_t* q_off, const int32_t* q_len, const int64_t* t_off,
                               const int32_t* t_len, int32_t n, const ChunkStarts& cb,
                               int64_t q_bytes, int64_t t_bytes, unsigned long long* ends,

@@ -43,12 +43,17 @@ constexpr int32_t kTag4MinPairs = 1 << 19;
 constexpr int kJMin = 5;                 // length buckets j: qlen + 2 <= 2^j
 constexpr int kJMax = 21;
 constexpr int kNumJ = kJMax + 1;
-constexpr int kNumSub = 256;             // sub-buckets per bucket: exact query length up to 2^9
+// Bins the queue is ordered by, within a class: one per exact query length in
+// the buckets up to kExactJ, kLongSub of equal width in each longer one (bins
+// of 1.6% of the length; a one-block scan reads them all in every call).
+constexpr int kExactJ = 9;
+constexpr int kLongSub = 64;
+constexpr int kExactBins = 1 << kExactJ;
+constexpr int kClassBins = kExactBins + kLongSub * (kJMax - kExactJ);
 // buckets the band engine takes: queries of 511 bases and longer (streams of
 // 55k / 885k pairs 2.71 / 14.1 -> 1.62 / 9.9 ms)
 constexpr int kBandJMin = 10;
-constexpr int kJSpan = kJMax - kJMin + 1;
-constexpr int kNumBuckets = kNumClasses * kJSpan * kNumSub;
+constexpr int kNumBuckets = kNumClasses * kClassBins;
 // Calls of fewer pairs skip the near passes: their time is launches and one
 // pair's latency, which the passes add to (1,000 pairs of 100 bases 147 ->
 // 223 us; 5,000 of 64 bases 180 -> 164 us).
@@ -58,7 +63,8 @@ constexpr int32_t kNearMinPairs = 4096;
 constexpr int kNearHalf = 15;
 constexpr int kNearJMax = 9;
 constexpr int kNearMaxQ = (1 << kNearJMax) - 2;
-constexpr int kNearBins = (kNearJMax - kJMin + 1) * kNumSub;
+static_assert(kNearJMax <= kExactJ, "one bin per length");
+constexpr int kNearBins = 1 << kNearJMax;
 constexpr int kQueueThreads = 128;       // threads per CTA of the queue kernels
 constexpr int kMaxLaunches = 64;         // queue-kernel launches per call (heads)
 
@@ -170,29 +176,35 @@ __device__ __forceinline__ int ceil_log2(uint32_t x) {  // x >= 1
   return x <= 1 ? 0 : 32 - __clz(x - 1);
 }
 
-// Length bucket j (qlen + 2 <= 2^j, at least kJMin) and sub-bucket: the exact
-// query length while a bucket spans at most kNumSub lengths, else its top bits.
-__device__ __forceinline__ void bucket_of(int32_t ql, int* j_out, int* sub_out) {
-  int j = ceil_log2((uint32_t)ql + 2u);
-  if (j < kJMin) j = kJMin;
-  int sub;
-  if (j == kJMin) {
-    sub = ql;
-  } else {
-    const int32_t off = ql + 2 - (1 << (j - 1));
-    sub = j <= 9 ? off : (off >> (j - 9));
-  }
-  sub = sub < 0 ? 0 : (sub >= kNumSub ? kNumSub - 1 : sub);
-  *j_out = j;
-  *sub_out = sub;
+// Length bucket j of a query: qlen + 2 <= 2^j, at least kJMin.
+__device__ __forceinline__ int bucket_of(int32_t ql) {
+  const int j = ceil_log2((uint32_t)ql + 2u);
+  return j < kJMin ? kJMin : j;
 }
 
-// Counter of a (class, bucket, sub-bucket), and of a NEAR pair k_near left.
-__host__ __device__ __forceinline__ int bin_of(int cls, int j, int sub) {
-  return (cls * kJSpan + j - kJMin) * kNumSub + sub;
+// Bin of a query length: bucket j <= kExactJ is the bins 2^(j-1) .. 2^j - 1
+// (kJMin: from 0), one per length; the buckets after it kLongSub bins each.
+__device__ __forceinline__ int bin_of_len(int32_t ql) {
+  if (ql + 2 <= kExactBins) return ql + 1;
+  const int j = bucket_of(ql);
+  const int sub = (ql + 1 - (1 << (j - 1))) >> (j - 7);  // 2^(j-1) lengths, 64 bins
+  return kExactBins + (j - kExactJ - 1) * kLongSub + (sub < kLongSub ? sub : kLongSub - 1);
 }
-__host__ __device__ __forceinline__ int near_bin(int j, int sub) {
-  return (j - kJMin) * kNumSub + sub;
+static_assert(kLongSub == 64, "bin_of_len's shift");
+
+// Bucket of a bin, and whether the bin is its bucket's longest or shortest.
+__device__ __forceinline__ int bucket_of_bin(int bin) {
+  if (bin >= kExactBins) return kExactJ + 1 + (bin - kExactBins) / kLongSub;
+  const int j = 32 - __clz(bin);
+  return j < kJMin ? kJMin : j;
+}
+__device__ __forceinline__ bool longest_bin(int bin) {
+  return bin >= kExactBins ? bin % kLongSub == kLongSub - 1
+                           : bin == (1 << bucket_of_bin(bin)) - 1;
+}
+__device__ __forceinline__ bool shortest_bin(int bin) {
+  if (bin >= kExactBins) return bin % kLongSub == 0;
+  return bin == 0 || (bin >= 1 << kJMin && (bin & (bin - 1)) == 0);
 }
 
 }  // namespace xt

@@ -325,10 +325,8 @@ __global__ void __launch_bounds__(kNearThreads, kNearBlocks)
         write_result(b, kk[h], n.best, brow[h] - n.d_best + 1, brow[h] + 1, n.g, n.row + 1, off[h],
                      XT_OK, band_cells_upto(last, ql[h], sc.w));
       } else {
-        int j, sub;
-        bucket_of(ql[h], &j, &sub);
-        const int bin = bin_of(CLS_NEAR, j, sub);
-        const int32_t at = w.cursor[bin] - w.counts[bin] + atomicAdd(&w.near_left[near_bin(j, sub)], 1);
+        const int nb = bin_of_len(ql[h]), bin = CLS_NEAR * kClassBins + nb;
+        const int32_t at = w.cursor[bin] - w.counts[bin] + atomicAdd(&w.near_left[nb], 1);
         w.near_tmp[at] = kk[h];
       }
     }
@@ -338,16 +336,15 @@ __global__ void __launch_bounds__(kNearThreads, kNearBlocks)
 // Pairs left by k_near, from their length's run in near_tmp to one run in the
 // queue at the class's place (longest first, as every segment); the class's
 // segment table then covers the pairs left.
-constexpr int kGatherThreads = 640;
-static_assert(kNearBins == 2 * kGatherThreads, "two bins per thread");
+constexpr int kGatherThreads = kNearBins;  // a thread per bin
 
 __global__ void __launch_bounds__(kGatherThreads) k_near_gather(Work w) {
   __shared__ int32_t s_pre[kNearBins];  // in queue order
   __shared__ int32_t s_warp[kGatherThreads / 32];
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-  // queue position u -> bin kNearBins - 1 - u (longest bucket, longest length first)
-  const int32_t c0 = w.near_left[kNearBins - 1 - 2 * t], c1 = w.near_left[kNearBins - 2 - 2 * t];
-  int32_t inc = c0 + c1;
+  // queue position u -> bin kNearBins - 1 - u (longest length first)
+  const int32_t c0 = w.near_left[kNearBins - 1 - t];
+  int32_t inc = c0;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const int32_t v = __shfl_up_sync(0xffffffffu, inc, d);
@@ -355,10 +352,9 @@ __global__ void __launch_bounds__(kGatherThreads) k_near_gather(Work w) {
   }
   if (lane == 31) s_warp[wid] = inc;
   __syncthreads();
-  int32_t before = inc - c0 - c1;
+  int32_t before = inc - c0;
   for (int u = 0; u < wid; ++u) before += s_warp[u];
-  s_pre[2 * t] = before;
-  s_pre[2 * t + 1] = before + c0;
+  s_pre[t] = before;
   __syncthreads();
   const int32_t region = w.seg_begin[CLS_NEAR * kNumJ + kJMax];  // never rewritten below
   const int warps = gridDim.x * (kGatherThreads / 32);
@@ -366,17 +362,14 @@ __global__ void __launch_bounds__(kGatherThreads) k_near_gather(Work w) {
     const int nb = kNearBins - 1 - u;
     const int32_t c = w.near_left[nb];
     if (c == 0) continue;
-    const int bin = bin_of(CLS_NEAR, kJMin + nb / kNumSub, nb % kNumSub);
+    const int bin = CLS_NEAR * kClassBins + nb;
     const int32_t src = w.cursor[bin] - w.counts[bin], dst = region + s_pre[u];
     for (int32_t k = lane; k < c; k += 32) w.order[dst + k] = w.near_tmp[src + k];
   }
-  if (blockIdx.x == 0 && t <= kNearJMax - kJMin) {
-    const int j = kNearJMax - t;  // bucket j's bins in queue order: [256 t, 256 t + 256)
-    const int32_t lo = s_pre[kNumSub * t];
-    const int last = kNumSub * t + kNumSub - 1;
-    const int32_t hi = s_pre[last] + w.near_left[kNearBins - 1 - last];
-    w.seg_begin[CLS_NEAR * kNumJ + j] = region + lo;
-    w.seg_end[CLS_NEAR * kNumJ + j] = region + hi;
+  if (blockIdx.x == 0) {
+    const int bin = kNearBins - 1 - t;
+    if (longest_bin(bin)) w.seg_begin[CLS_NEAR * kNumJ + bucket_of_bin(bin)] = region + before;
+    if (shortest_bin(bin)) w.seg_end[CLS_NEAR * kNumJ + bucket_of_bin(bin)] = region + before + c0;
   }
 }
 

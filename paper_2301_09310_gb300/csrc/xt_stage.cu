@@ -59,12 +59,27 @@ k_chunk_ends(const int64_t* __restrict__ q_off, const int32_t* __restrict__ q_le
   }
 }
 
-__global__ void k_store_desc(Batch* dst, Batch b) { *dst = b; }
+// The call's descriptor, and the counters a batched call starts at zero: one
+// block, in the place of two memsets (a launch each on the call's critical path).
+constexpr int kDescThreads = 1024;
+static_assert(kNumBuckets % 4 == 0 && kNearBins % 4 == 0 && kMaxLaunches % 4 == 0, "int4 stores");
+
+__global__ void __launch_bounds__(kDescThreads) k_store_desc(Batch* dst, Batch b, Work w) {
+  const int4 z = make_int4(0, 0, 0, 0);
+  if (threadIdx.x == 0) *dst = b;
+  if (w.counts)
+    for (int i = threadIdx.x; i < kNumBuckets / 4; i += kDescThreads)
+      reinterpret_cast<int4*>(w.counts)[i] = z;
+  if (w.heads && threadIdx.x < kMaxLaunches / 4) reinterpret_cast<int4*>(w.heads)[threadIdx.x] = z;
+  if (w.near_left)
+    for (int i = threadIdx.x; i < kNearBins / 4; i += kDescThreads)
+      reinterpret_cast<int4*>(w.near_left)[i] = z;
+}
 
 }  // namespace
 
-cudaError_t launch_store_desc(Batch* dst, const Batch& b, cudaStream_t stream) {
-  k_store_desc<<<1, 1, 0, stream>>>(dst, b);
+cudaError_t launch_store_desc(Batch* dst, const Batch& b, const Work& w, cudaStream_t stream) {
+  k_store_desc<<<1, kDescThreads, 0, stream>>>(dst, b, w);
   return cudaGetLastError();
 }
 
