@@ -149,7 +149,7 @@ xt_status get_work(xt_ctx* ctx, int32_t n, Work* w, Batch** desc) {
   const size_t o_sb = off; off = align_up(off + 4 * (size_t)(kNumClasses * kNumJ));
   const size_t o_se = off; off = align_up(off + 4 * (size_t)(kNumClasses * kNumJ));
   const size_t o_heads = off; off = align_up(off + 4 * (size_t)kMaxLaunches);
-  const size_t o_left = off; off = align_up(off + 4 * (size_t)kNearBins);
+  const size_t o_left = off; off = align_up(off + 4 * (size_t)(kNearBins + kBandLeft));
   const size_t o_tmp = off; off = align_up(off + 4 * (size_t)n);
   void* old = ctx->work;
   xt_status s = dev_alloc(ctx, &ctx->work, &ctx->work_bytes, off);
@@ -165,6 +165,7 @@ xt_status get_work(xt_ctx* ctx, int32_t n, Work* w, Batch** desc) {
   w->seg_end = (int32_t*)(base + o_se);
   w->heads = (int32_t*)(base + o_heads);
   w->near_left = (int32_t*)(base + o_left);
+  w->band_left = w->near_left + kNearBins;
   w->near_tmp = (int32_t*)(base + o_tmp);
   return XT_OK;
 }
@@ -179,6 +180,7 @@ struct Plan {
   bool pool_serial = true;  // global-ring launches share one pool region, in order
   int32_t near_pairs = 0;   // pairs of the NEAR class (k_near runs when there are any)
   int near_grid = 0;
+  int band_near = 0;        // narrow band launches (each gathers the pairs it left)
 };
 
 int64_t next_pow2(int64_t x) { return (int64_t)1 << log2_ceil(x); }
@@ -251,7 +253,7 @@ void bucket_schedule(const xt_ctx* ctx, int j, int w, int* P, int* R, int* rs_lo
   *P = 32; *R = 8; *rs_log2 = 0; *huge = true;
 }
 
-void add_huge_launch(xt_ctx* ctx, const Score& sc, Plan* pl) {
+Launch huge_launch(const xt_ctx* ctx, const Score& sc, Plan* pl) {
   // global slabs: ring of min(qlen, 256 + 2w) + 2 entries, qlen <= XT_MAX_LEN
   const int64_t need = std::min<int64_t>(XT_MAX_LEN, 256 + 2 * (int64_t)sc.w) + 2;
   pl->slab = next_pow2(need);
@@ -259,10 +261,14 @@ void add_huge_launch(xt_ctx* ctx, const Score& sc, Plan* pl) {
   int64_t grid = (int64_t)kPoolCap / per_cta;
   if (grid > 2 * ctx->num_sms) grid = 2 * ctx->num_sms;
   if (grid < 1) grid = 1;
-  Launch& L = pl->launch[pl->n_launch++];
-  L = Launch();
+  Launch L;
   L.cls = CLS_HUGE; L.j_lo = 0; L.j_hi = kJMax; L.lane = false; L.P = 32; L.R = 8;
   L.rs_log2 = 0; L.global_ring = true; L.slab = pl->slab; L.grid = (int)grid; L.mparam = 0;
+  return L;
+}
+
+void add_huge_launch(const xt_ctx* ctx, const Score& sc, Plan* pl) {
+  pl->launch[pl->n_launch++] = huge_launch(ctx, sc, pl);
 }
 
 constexpr int kLaneJMax = 9;           // single-phase plan: one-lane engine up to 2^9 - 2 bases
@@ -300,6 +306,7 @@ bool lane_launch(xt_ctx* ctx, const Score& sc, int cls, int j, bool allow_gring,
 
 bool same_config(const Launch& a, const Launch& b) {
   return a.cls == b.cls && a.lane == b.lane && a.band == b.band && a.P == b.P && a.R == b.R &&
+         !a.near_hw && !b.near_hw && !a.after_prev && !b.after_prev &&
          a.rs_log2 == b.rs_log2 && a.global_ring == b.global_ring && a.grid == b.grid &&
          a.mparam == b.mparam;
 }
@@ -380,8 +387,9 @@ inline double band_cells_est(double q, int w) {
 void batched_flags(xt_ctx* ctx, const Score& sc, int32_t n, JFlags* jf, bool* lane_ok) {
   *jf = JFlags{};
   for (int j = 0; j < kNumJ; ++j) lane_ok[j] = false;
-  int bP, bK;
-  const bool band = ctx->near_first && !ctx->forced_P && band_shape(sc, ctx->match, &bP, &bK);
+  int bP, bK, bhw;
+  const bool may_band = ctx->near_first && !ctx->forced_P;
+  const bool band = may_band && band_shape(sc, ctx->match, 0, &bP, &bK);
   const bool saved = ctx->plan_small;
   for (int j = kJMin; j <= kJMax; ++j) {
     Launch L;
@@ -400,7 +408,8 @@ void batched_flags(xt_ctx* ctx, const Score& sc, int32_t n, JFlags* jf, bool* la
     }
     lane_ok[j] = want && lane_launch(ctx, sc, CLS_PACKED, j, true, &L) &&
                  lane_launch(ctx, sc, CLS_NARROW, j, true, &L);
-    const bool banded = band && j >= kBandJMin && !tuned_any(ctx, sc.w, j);
+    const bool banded = may_band && !tuned_any(ctx, sc.w, j) &&
+                        (band || band_near_shape(sc, ctx->match, j, &bP, &bK, &bhw));
     if (banded) jf->f[j] |= kJBand;
     if (lane_ok[j])
       jf->f[j] |= kJPacked |
@@ -466,9 +475,11 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
       if (lane_ok[j]) long_pairs += cnt[cls][j];
   const bool long_lanes = long_pairs >= 2 * (int64_t)kLaneSlots;
   auto min_pairs = [&](int jj) { return jj >= kLongJ && long_lanes ? 0 : lane_min_pairs(jj); };
-  // one launch takes the BAND class, longest queries first
-  int32_t band_pairs = 0;
-  for (int j = 0; j < kNumJ; ++j) band_pairs += cnt[CLS_BAND][j];
+  // the band engine, where it holds the band
+  int bP = 0, bK = 0, bhw = 0;
+  const bool band_ok = ctx->near_first && !ctx->forced_P && band_shape(sc, ctx->match, 0, &bP, &bK);
+  // pairs of each launch
+  int32_t pairs_of[kMaxLaunches] = {};
   for (int cls : {CLS_PACKED, CLS_NARROW, CLS_WIDE, CLS_NEAR, CLS_BAND}) {
     int prev = -1;
     for (int j = kJMax; j >= 0; --j) {
@@ -478,10 +489,29 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
       ctx->plan_small = c < kBucketSmall;
       Launch L;
       bool lane = false, band = false;
+      if (cls == CLS_BAND && !band_ok) {
+        // a narrow band first, then the group engine for the pairs it leaves
+        if (pl->n_launch >= kMaxLaunches - 2 ||
+            !band_near_shape(sc, ctx->match, jj, &L.P, &L.R, &L.near_hw)) {
+          pl->bad = true;
+          continue;
+        }
+        L.cls = cls; L.band = true; L.j_lo = L.j_hi = j;
+        pairs_of[pl->n_launch] = c;
+        pl->launch[pl->n_launch++] = L;
+        pl->band_near++;
+        int P, R, lg;
+        bool huge;
+        bucket_schedule(ctx, jj, sc.w, &P, &R, &lg, &huge, true);
+        L = huge ? huge_launch(ctx, sc, pl) : queue_launch(ctx, cls, jj, P, R, lg);
+        L.cls = cls; L.j_lo = L.j_hi = j; L.after_prev = true;
+        pairs_of[pl->n_launch] = (c + kNearLeft - 1) / kNearLeft;
+        pl->launch[pl->n_launch++] = L;
+        prev = -1;
+        continue;
+      }
       if (cls == CLS_BAND) {
-        band = true;  // classify gives the class to buckets the band engine takes
-        band_shape(sc, ctx->match, &L.P, &L.R);
-        L.cls = cls; L.band = true; L.grid = band_grid(L.P, band_pairs, ctx->num_sms);
+        band = true;
       } else if (cls != CLS_WIDE && lane_ok[jj]) {
         lane = true;
         if (ctx->forced_P > 1) {
@@ -500,7 +530,12 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
                                            (double)kLaneSlots <= est_cells;
         }
       }
+      // too few pairs for one lane each: groups of the band engine, whose rows
+      // stop at the query's end and which work in 16 bits
+      if (!lane && band_ok && packed_class(cls) && !tuned(ctx, sc.w, jj)) band = true;
       if (band) {
+        band_shape(sc, ctx->match, c, &L.P, &L.R);
+        L.cls = cls; L.band = true;
       } else if (lane) {
         lane_launch(ctx, sc, cls, jj, true, &L);
       } else {
@@ -540,17 +575,30 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
       L.j_hi = j;
       if (prev >= 0 && same_config(pl->launch[prev], L)) {
         pl->launch[prev].j_lo = j;
+        pairs_of[prev] += c;
         continue;
       }
-      if (pl->n_launch >= kMaxLaunches - 1) {  // 3 classes x 17 buckets + 1 stay below
+      if (pl->n_launch >= kMaxLaunches - 2) {  // the last heads: HUGE and the near pass
         pl->bad = true;
         continue;
       }
+      pairs_of[pl->n_launch] = c;
       pl->launch[pl->n_launch] = L;
       prev = pl->n_launch++;
     }
   }
   ctx->plan_small = saved;
+  // no more CTAs than the pairs need (group launches in powers of two, so that
+  // calls of like size share a graph)
+  for (int i = 0; i < pl->n_launch; ++i) {
+    Launch& L = pl->launch[i];
+    if (L.band) {
+      L.grid = band_grid(L.P, L.R, pairs_of[i], ctx->num_sms);
+    } else if (!L.lane) {
+      const int64_t per_cta = kQueueThreads / L.P;
+      L.grid = (int)std::min<int64_t>(L.grid, next_pow2((pairs_of[i] + per_cta - 1) / per_cta));
+    }
+  }
   // the NEAR class, which waits for k_near, after the others; within each,
   // longest queries first: their pairs set the call's critical path, and the
   // launches after them fill the slots they leave (c5-mix call of 1M pairs:
@@ -725,10 +773,13 @@ cudaError_t enqueue_dp(xt_ctx* ctx, bool plain, const Plan& pl, int plain_rs, co
     if (e == cudaSuccess && nb > 1) e = cudaEventRecord(ctx->near_ev, st);
     dp += 2;
   }
+  cudaStream_t st = stream;
   for (int i = 0; e == cudaSuccess && i < pl.n_launch; ++i) {
     const Launch& L = pl.launch[i];
-    cudaStream_t st = stream;
-    if (nb > 1) st = ctx->aux[L.global_ring && pl.pool_serial ? 0 : (rr++ % nb)];
+    // a launch that takes what the one before it left follows on its stream
+    const bool leads = i + 1 < pl.n_launch && pl.launch[i + 1].after_prev;
+    const bool ring = L.global_ring || (leads && pl.launch[i + 1].global_ring);
+    if (!L.after_prev) st = nb > 1 ? ctx->aux[ring && pl.pool_serial ? 0 : (rr++ % nb)] : stream;
     if (L.cls == CLS_NEAR && nb > 1) e = cudaStreamWaitEvent(st, ctx->near_ev, 0);
     if (e != cudaSuccess) break;
     void* gring = L.global_ring ? static_cast<void*>(reinterpret_cast<char*>(ctx->pool) + L.pool_off)
@@ -740,11 +791,11 @@ cudaError_t enqueue_dp(xt_ctx* ctx, bool plain, const Plan& pl, int plain_rs, co
       char buf[192];
       std::snprintf(buf, sizeof(buf),
                     "launch %d of %d (%s cls %d buckets %d..%d P %d R %d ring 2^%d %s grid %d): ", i,
-                    pl.n_launch, L.lane ? "one-lane" : "group", L.cls, L.j_lo, L.j_hi, L.P, L.R,
+                    pl.n_launch, L.band ? "band" : (L.lane ? "one-lane" : "group"), L.cls, L.j_lo, L.j_hi, L.P, L.R,
                     L.rs_log2, L.global_ring ? "global" : "shared", L.grid);
       ctx->launch_error = buf;
     }
-    ++dp;
+    dp += L.near_hw > 0 ? 2 : 1;
   }
   if (e == cudaSuccess && nb > 1) {
     for (int b = 0; e == cudaSuccess && b < nb; ++b) {
@@ -773,7 +824,7 @@ uint64_t plan_signature(const Plan& pl) {
   for (int i = 0; i < pl.n_launch; ++i) {
     const Launch& L = pl.launch[i];
     mix(L.cls); mix(L.j_lo); mix(L.j_hi); mix(L.lane); mix(L.band); mix(L.P); mix(L.R); mix(L.rs_log2);
-    mix(L.global_ring); mix(L.slab); mix(L.grid); mix(L.mparam); mix((int64_t)L.pool_off);
+    mix(L.near_hw); mix(L.after_prev); mix(L.global_ring); mix(L.slab); mix(L.grid); mix(L.mparam); mix((int64_t)L.pool_off);
   }
   mix(pl.pool_serial);
   mix(pl.near_grid);
@@ -940,7 +991,7 @@ xt_status run_finish(xt_ctx* ctx) {
   if (ge && ge->exec) {
     e = cudaGraphLaunch(ge->exec, pc.stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
-    dp = (plain ? 1 : 0) + (pl.near_pairs > 0 ? 2 : 0) + pl.n_launch;
+    dp = (plain ? 1 : 0) + (pl.near_pairs > 0 ? 2 : 0) + pl.band_near + pl.n_launch;
   } else {
     ctx->launch_error.clear();
     e = body(pc.stream, &dp);
@@ -1649,6 +1700,7 @@ bool carve_static(void* base_ptr, int32_t n, Work* w, Batch** desc) {
   w->seg_end = (int32_t*)(base + o_se);
   w->heads = (int32_t*)(base + o_heads);
   w->near_left = nullptr;  // no near pass on this path
+  w->band_left = nullptr;
   w->near_tmp = nullptr;
   *desc = (Batch*)(base + o_desc);
   return true;

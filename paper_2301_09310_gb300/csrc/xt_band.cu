@@ -39,7 +39,8 @@ namespace xt {
 namespace {
 
 constexpr int kBandThreads = 128;
-constexpr int kBandBlocks = 3;  // per SM: up to 168 registers
+// CTAs per SM: 32 slots take up to 168 registers a thread, fewer slots less.
+__host__ __device__ constexpr int band_blocks(int K) { return K <= 14 ? 4 : 3; }
 constexpr int kKeyBits = 5;     // slots of a lane
 constexpr int kBaseSteps = 8;   // steps between two bases
 
@@ -50,11 +51,15 @@ constexpr int32_t kNoKey = 16383;
 // Rows between the row a base was taken from and the last one it is used for.
 __host__ __device__ constexpr int base_age(int P) { return P + kBaseSteps; }
 
-template <int P, int K>
-__global__ void __launch_bounds__(kBandThreads, kBandBlocks)
+// NEAR: the P * K slots hold diagonals |i - j| <= hw of a wider band (hw <
+// sc.w); a pair is settled only where the bounds of xt_near.cuh prove its
+// outputs, and the others go to near_tmp at their bucket's place in the queue
+// (counted in band_left).
+template <int P, int K, bool NEAR>
+__global__ void __launch_bounds__(kBandThreads, band_blocks(K))
     k_band(const Batch* __restrict__ bd, Score sc, Work w, int cls, int j_lo, int j_hi,
            int head_id, int32_t match, uint32_t mcm, uint32_t kmul, int32_t fall,
-           int sms) {
+           int sms, const int32_t hw) {
   static_assert(K % 2 == 0 && K <= 32 && P <= 32, "slot index fits the key");
   constexpr int kWords = (K + 7) / 8;          // window words a row's slots span
   constexpr int kWin = (K + 7 + 7) / 8;        // and over the eight rows of a reload
@@ -76,7 +81,7 @@ __global__ void __launch_bounds__(kBandThreads, kBandBlocks)
   const int32_t begin = w.seg_begin[cls * kNumJ + j_hi];
   const int32_t end = w.seg_end[cls * kNumJ + j_lo];
   int32_t* head = w.heads + head_id;
-  const int32_t alpha = sc.alpha, beta = sc.beta, hw = sc.w;
+  const int32_t alpha = sc.alpha, beta = sc.beta;
   const int32_t pad = P * K - (2 * hw + 1);    // dead slots before the band's first
   const int32_t u0 = p * K;                    // slot u of the group: column i - hw - pad + u
   const uint32_t na2 = pack16(-alpha, -alpha), nb2 = pack16(-beta, -beta);
@@ -149,12 +154,27 @@ __global__ void __launch_bounds__(kBandThreads, kBandBlocks)
     }
     const int32_t ends_from = __reduce_min_sync(full, min(ql[0], ql[1])) - 1 - hw;
     auto half = [](uint32_t v, int h) -> int32_t { return h ? hi16(v) : lo16(v); };
+    // NEAR: whether the cells off the narrow band leave the results alone, row i
+    // the last one seen (the rows since was_best was taken against that best,
+    // those to come against the last); a failed pair is left
+    int32_t was_best[2] = {h0[0], h0[1]};
+    auto leave = [&](int h) {
+      act[h] = false;
+      const int j = bucket_of(ql[h]);
+      w.near_tmp[w.seg_begin[cls * kNumJ + j] + atomicAdd(&w.band_left[j], 1)] = kk[h];
+    };
+    auto settled = [&](int h, int32_t i) -> bool {
+      const int32_t top = half(best2, h), cap = min(tl[h] - 1, ql[h] - 1 + sc.w);
+      return g[h] > 0 && near_row_ok(i, ql[h], h0[h], match, hw, was_best[h], sc) &&
+             near_row_ok(cap, ql[h], h0[h], match, hw, top, sc) &&
+             near_end_ok(g[h], ql[h], tl[h], h0[h], match, hw, sc);
+    };
     auto finish = [&](int h, int32_t last) {
       act[h] = false;
       const int32_t d = mid - half(bu2, h);  // diagonal of the best
       write_result(b, kk[h], half(best2, h), brow[h] - d + 1, brow[h] + 1, g[h],
                    g[h] > 0 ? grow[h] + 1 : 0, half(off2, h), XT_OK,
-                   band_cells_upto(last, ql[h], hw));
+                   band_cells_upto(last, ql[h], sc.w));
     };
     uint32_t win[2][kWin], tw[2] = {0, 0};
     int32_t qpos = qpos0;
@@ -331,6 +351,21 @@ __global__ void __launch_bounds__(kBandThreads, kBandBlocks)
             if (!act[h]) continue;
             const int32_t m = half(M2, h), top = half(best2, h);
             bool stop = i >= row_end[h];
+            if (NEAR) {
+              // a dead row or one far below the best: only the whole band
+              // tells whether the extension stops there
+              if (m == 0 || (sc.zdrop > 0 && top - m > sc.zdrop)) {
+                leave(h);
+              } else if (stop) {
+                int32_t last = -1;
+                if (settled(h, i)) {
+                  const NearEnd n = {top, mid - half(bu2, h), g[h], grow[h]};
+                  last = near_last_row(n, ql[h], tl[h], h0[h], match, sc);
+                }
+                if (last >= 0) finish(h, last); else leave(h);
+              }
+              continue;
+            }
             if (m == 0) {
               if (dead_row[h] != i - 1) live_row[h] = i - 1;
               dead_row[h] = i;
@@ -370,15 +405,22 @@ __global__ void __launch_bounds__(kBandThreads, kBandBlocks)
 #pragma unroll
             for (int o = P / 2; o > 0; o >>= 1) top[h] = max(top[h], __shfl_xor_sync(full, top[h], o, P));
           if (p == P - 1 && act[h] && g[h] > 0 && bound[h] <= g[h]) {
-            NearEnd n;
-            n.best = half(best2, h);
-            n.d_best = mid - half(bu2, h);
-            n.g = g[h];
-            n.row = grow[h];
+            const NearEnd n = {half(best2, h), mid - half(bu2, h), g[h], grow[h]};
             const int32_t last = near_last_row(n, ql[h], tl[h], h0[h], match, sc);
-            if (last >= 0) finish(h, last);
+            if (NEAR && (last < 0 || !settled(h, i)))
+              leave(h);
+            else if (last >= 0)
+              finish(h, last);
           }
           bound[h] = top[h];
+        }
+      }
+      // the rows of the last eight steps against the best before them
+      if (NEAR && p == P - 1 && i >= 0) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (act[h] && !near_row_ok(i, ql[h], h0[h], match, hw, was_best[h], sc)) leave(h);
+          was_best[h] = half(best2, h);
         }
       }
       more = __any_sync(full, p == P - 1 && (act[0] || act[1]));
@@ -393,60 +435,95 @@ __global__ void __launch_bounds__(kBandThreads, kBandBlocks)
   }
 }
 
-// The lane counts and slots compiled, narrowest first.
+// The pairs the NEAR launch of bucket j left, from near_tmp to the front of the
+// bucket's run in the queue.
+__global__ void k_band_gather(Work w, int cls, int j) {
+  const int32_t at = w.seg_begin[cls * kNumJ + j], n = w.band_left[j];
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    w.order[at + i] = w.near_tmp[at + i];
+  if (blockIdx.x == 0 && threadIdx.x == 0) w.seg_end[cls * kNumJ + j] = at + n;
+}
+
+// The lane counts and slots compiled: per lane count, fewest slots first.
 struct BandShape {
   int P, K;
 };
-constexpr BandShape kBandShapes[] = {{2, 32},  {4, 32},  {8, 26},  {8, 32},
-                                     {16, 26}, {16, 32}, {32, 26}, {32, 32}};
+constexpr BandShape kBandShapes[] = {{2, 32},  {4, 32},  {8, 26},  {8, 32},  {16, 14}, {16, 26},
+                                     {16, 32}, {32, 8},  {32, 14}, {32, 26}, {32, 32}};
 
-int32_t band_fall(const Score& sc, int32_t match) {
+int32_t band_fall(const Score& sc) {
   // the most a row's maximum can fall below the one before it
   int32_t d = sc.alpha;
   d = std::max(d, -(int32_t)(int8_t)((sc.prof[0] >> 8) & 0xFF));
   d = std::max(d, -(int32_t)(int8_t)(sc.nnnn & 0xFF));
-  (void)match;
   return d;
 }
 
-}  // namespace
-
-bool band_shape(const Score& sc, int32_t match, int* P, int* K) {
+// Whether the engine takes the scoring with P lanes a pair.
+bool band_scoring(const Score& sc, int32_t match, int P) {
   if (sc.w < 8 || sc.alpha < 1 || sc.alpha > 127) return false;
-  for (const BandShape& s : kBandShapes) {
-    if (s.P * s.K < 2 * sc.w + 1) continue;
-    const int32_t fall = band_fall(sc, match);
-    // H - base of a row's maximum, and of the column before the query, within the key
-    if (base_age(s.P) * (fall + match) + fall + match + 2 > (32767 >> kKeyBits) - 1)
-      return false;
-    *P = s.P;
-    *K = s.K;
-    return true;
-  }
-  return false;
+  const int32_t fall = band_fall(sc);
+  // H - base of a row's maximum, and of the column before the query, within the key
+  return base_age(P) * (fall + match) + fall + match + 2 <= (32767 >> kKeyBits) - 1;
 }
 
-int band_grid(int P, int32_t pairs, int num_sms) {
+// A launch with fewer warps than this leaves schedulers idle.
+constexpr int64_t kBandWarps = 608;
+
+}  // namespace
+
+// Lanes per pair: the fewest that hold the band, whose rows cost the least in
+// all; while the launch's warps then leave schedulers idle, more lanes with
+// fewer slots each, which shorten the time of a row (a row costs a warp about
+// 20 cycles a slot and 300 besides).
+bool band_shape(const Score& sc, int32_t match, int32_t pairs, int* P, int* K) {
+  *P = 0;
+  for (const BandShape& s : kBandShapes) {
+    if (s.P * s.K < 2 * (int64_t)sc.w + 1 || s.P == *P || !band_scoring(sc, match, s.P)) continue;
+    if (*P && (int64_t)pairs * s.P > kBandWarps * 64) break;
+    *P = s.P;
+    *K = s.K;
+  }
+  return *P > 0;
+}
+
+// The narrow band tried first on the pairs of bucket j where the whole band is
+// too wide for the engine: diagonals up to an eighth to a quarter of the
+// query's length to each side.  A read with 2% substitutions loses about a tenth
+// of its length against a perfect match, and a pair is settled while it loses
+// less than the half width.
+bool band_near_shape(const Score& sc, int32_t match, int j, int* P, int* K, int* hw) {
+  if (j < kBandNearJMin) return false;
+  *P = j <= 10 ? 8 : (j == 11 ? 16 : 32);
+  *K = 32;
+  *hw = *P * *K / 2 - 1;
+  return *hw < sc.w && band_scoring(sc, match, *P);
+}
+
+int band_grid(int P, int K, int32_t pairs, int num_sms) {
   const int64_t per_cta = 2 * (int64_t)kBandThreads / P;
   const int64_t want = ((int64_t)pairs + per_cta - 1) / per_cta;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms * kBandBlocks));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms * band_blocks(K)));
 }
 
 cudaError_t launch_band(const Batch* bd, const Score& sc, int32_t match, const Work& w,
                         const Launch& L, int head_id, int num_sms, cudaStream_t stream) {
   int mshift = 0;
   while ((1 << mshift) < match + 1) ++mshift;
-  const int32_t fall = band_fall(sc, match);
-#define XT_B(PP, KK)                                                                           \
-  if (L.P == PP && L.R == KK) {                                                                \
-    k_band<PP, KK><<<L.grid, kBandThreads, 0, stream>>>(bd, sc, w, L.cls, L.j_lo, L.j_hi,      \
-                                                        head_id, match, 1u << mshift, 1u << kKeyBits, fall,   \
-                                                        num_sms);         \
+  const int32_t fall = band_fall(sc);
+#define XT_BL(PP, KK, NN)                                                                      \
+  if (L.P == PP && L.R == KK && (L.near_hw > 0) == NN) {                                       \
+    k_band<PP, KK, NN><<<L.grid, kBandThreads, 0, stream>>>(                                   \
+        bd, sc, w, L.cls, L.j_lo, L.j_hi, head_id, match, 1u << mshift, 1u << kKeyBits, fall,  \
+        num_sms, NN ? L.near_hw : sc.w);                                                       \
+    if (NN) k_band_gather<<<16, 256, 0, stream>>>(w, L.cls, L.j_lo);                           \
     return cudaGetLastError();                                                                 \
   }
-  XT_B(2, 32) XT_B(4, 32) XT_B(8, 26) XT_B(8, 32) XT_B(16, 26) XT_B(16, 32) XT_B(32, 26)
-  XT_B(32, 32)
-#undef XT_B
+  XT_BL(2, 32, false) XT_BL(4, 32, false) XT_BL(8, 26, false) XT_BL(8, 32, false)
+  XT_BL(16, 14, false) XT_BL(16, 26, false) XT_BL(16, 32, false) XT_BL(32, 8, false)
+  XT_BL(32, 14, false) XT_BL(32, 26, false) XT_BL(32, 32, false)
+  XT_BL(8, 32, true) XT_BL(16, 32, true) XT_BL(32, 32, true)
+#undef XT_BL
   return cudaErrorInvalidValue;
 }
 

@@ -63,7 +63,7 @@ __device__ __forceinline__ int classify_pair(const Batch& b, int32_t k, int32_t 
       bound * tag + tag - 1 <= 32767)
     cls = CLS_PACKED;
   if (cls == CLS_NARROW && (jf & kJBand) && ((bound + 1) << mshift) <= 32767) cls = CLS_BAND;
-  if ((jf & kJHuge) || (cls == CLS_WIDE && (jf & kJHugeWide))) cls = CLS_HUGE;
+  if (cls != CLS_BAND && ((jf & kJHuge) || (cls == CLS_WIDE && (jf & kJHugeWide)))) cls = CLS_HUGE;
   if (near && cls == CLS_PACKED) cls = CLS_NEAR;
   *bin = cls * kClassBins + bin_of_len(ql);
   return cls;

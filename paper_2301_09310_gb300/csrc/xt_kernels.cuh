@@ -15,7 +15,7 @@ namespace xt {
 //   HUGE:   band ring too large for shared memory (global slab per group)
 //   NEAR:   PACKED pairs that k_near tries on a narrow band first
 //   BAND:   NARROW pairs whose scores fit 16 bits under the anchoring
-//           multiplier, in buckets the band engine takes
+//           multiplier, where the band engine holds the band or a narrower one
 enum PairClass : uint8_t {
   CLS_PACKED = 0, CLS_NARROW = 1, CLS_WIDE = 2, CLS_HUGE = 3, CLS_NEAR = 4, CLS_BAND = 5,
   CLS_DONE = 6
@@ -50,9 +50,9 @@ constexpr int kExactJ = 9;
 constexpr int kLongSub = 64;
 constexpr int kExactBins = 1 << kExactJ;
 constexpr int kClassBins = kExactBins + kLongSub * (kJMax - kExactJ);
-// buckets the band engine takes: queries of 511 bases and longer (streams of
-// 55k / 885k pairs 2.71 / 14.1 -> 1.62 / 9.9 ms)
-constexpr int kBandJMin = 10;
+// buckets (queries of 511 bases and longer) the band engine tries on a narrow
+// band where the whole band is too wide for it
+constexpr int kBandNearJMin = 10;
 constexpr int kNumBuckets = kNumClasses * kClassBins;
 // Calls of fewer pairs skip the near passes: their time is launches and one
 // pair's latency, which the passes add to (1,000 pairs of 100 bases 147 ->
@@ -65,6 +65,7 @@ constexpr int kNearJMax = 9;
 constexpr int kNearMaxQ = (1 << kNearJMax) - 2;
 static_assert(kNearJMax <= kExactJ, "one bin per length");
 constexpr int kNearBins = 1 << kNearJMax;
+constexpr int kBandLeft = (kNumJ + 3) / 4 * 4;
 constexpr int kQueueThreads = 128;       // threads per CTA of the queue kernels
 constexpr int kMaxLaunches = 64;         // queue-kernel launches per call (heads)
 
@@ -78,7 +79,8 @@ struct Work {
   int32_t* seg_end;     // [kNumClasses * kNumJ]
   int32_t* heads;       // [kMaxLaunches]
   int32_t* near_left;   // [kNearBins] pairs k_near left, per exact length
-  int32_t* near_tmp;    // [n] those pairs, each length's run where its queue run was
+  int32_t* band_left;   // [kBandLeft] pairs a narrow band launch left, per bucket
+  int32_t* near_tmp;    // [n] those pairs, each length's (bucket's) run where its queue run was
 };
 
 constexpr int kLaneThreads = 128;        // threads per CTA of the one-lane kernels
@@ -91,6 +93,8 @@ struct Launch {
   int cls = 0, j_lo = 0, j_hi = 0;
   bool lane = false;         // one-lane engine (k_lane) instead of the group engine (k_queue)
   bool band = false;         // band engine (k_band): P lanes of R slots
+  int near_hw = 0;           // > 0: on a narrower band of this half width
+  bool after_prev = false;   // takes the pairs the launch before it left, on its stream
   int P = 1, R = 8;          // lanes per pair, rows per lane-strip (per half when packed)
   int rs_log2 = 0;           // ring entries per group = 1 << rs_log2
   bool global_ring = false;  // ring in a global slab per group instead of shared memory
@@ -126,10 +130,13 @@ cudaError_t launch_plain(const Batch* bd, int32_t n_cap, const Score& sc, const 
                          int rs_log2, cudaStream_t stream);
 cudaError_t launch_lane(const Batch* bd, const Score& sc, const Work& w, const Launch& L,
                         int head_id, void* gring, cudaStream_t stream);
-// The band engine's lanes per pair and slots per lane for a scoring; false
-// where it does not hold the band or the scoring's row keys.
-bool band_shape(const Score& sc, int32_t match, int* P, int* K);
-int band_grid(int P, int32_t pairs, int num_sms);
+// The band engine's lanes per pair and slots per lane for a scoring and a
+// launch of so many pairs; false where it does not hold the band or the
+// scoring's row keys.
+bool band_shape(const Score& sc, int32_t match, int32_t pairs, int* P, int* K);
+// The narrow band (half width hw) for bucket j's pairs of a wider band.
+bool band_near_shape(const Score& sc, int32_t match, int j, int* P, int* K, int* hw);
+int band_grid(int P, int K, int32_t pairs, int num_sms);
 cudaError_t launch_band(const Batch* bd, const Score& sc, int32_t match, const Work& w,
                         const Launch& L, int head_id, int num_sms, cudaStream_t stream);
 // ASCII letters to base codes (A/C/G/T either case -> 0..3, else 4), n bytes.

@@ -28,6 +28,21 @@
 //       is at most max(best, P_(qlen-1) - o, g + e d_end) -- when the last
 //       is the largest, the run itself attains the bound.
 // A pair that fails any of these is extended over its whole band as before.
+//
+// For a band of half width c that is a good part of the query (xt_band.cu) (1)
+// and (2) count what an excursion to diagonal +-(c + 1) costs in matches too.
+// A path to (i, j) with I query and D target bases in gaps makes j + 1 - I =
+// i + 1 - D matches at most.
+//   (1') A cell of row i that an excursion reaches, outside the band or back
+//        inside, is worth at most h0 + a f(i) - Q, f(i) = min(i + 1, max(qlen -
+//        c - 1, min(i - c, qlen))): an insertion excursion has I > c and at
+//        most min(i + 1, qlen - c - 1) matches (outside the band j > i + c; back
+//        inside it pays a deletion too), a deletion excursion has D > c and at
+//        most min(i - c, qlen).
+//   (2') The last column: an insertion excursion loses c + 1 matches besides Q.
+//        A deletion excursion that ends in row qlen - 1 + d, d <= c, inserts
+//        c + 1 - d bases at least, which cost o + (a + e)(c + 1 - d); if the
+//        target has rows beyond qlen - 1 + c, one that ends there costs Q alone.
 #pragma once
 #include <cstdint>
 
@@ -107,6 +122,23 @@ __device__ __forceinline__ int32_t near_last_row(const NearEnd& n, int32_t qlen,
   if (e == 0 || d_end < 0 || y < n.best || p - y > o) return -1;
   const int64_t k = y - o - 1 >= 0 ? (y - o - 1) / e : 0;
   return (int32_t)min(cap, max((int64_t)n.row, qlen - 1 + k));
+}
+
+// (1') on row i with best the running best of the row or a lower one.
+__device__ __forceinline__ bool near_row_ok(int32_t i, int32_t qlen, int32_t h0, int32_t match,
+                                            int32_t c, int32_t best, const Score& sc) {
+  const int64_t q = sc.alpha - sc.beta + (int64_t)sc.beta * (c + 1);
+  const int32_t f = min(i + 1, max(qlen - c - 1, min(i - c, qlen)));
+  return h0 + (int64_t)match * f - best < q;
+}
+
+// (2') for the end-to-end score g.
+__device__ __forceinline__ bool near_end_ok(int32_t g, int32_t qlen, int32_t tlen, int32_t h0,
+                                            int32_t match, int32_t c, const Score& sc) {
+  const int64_t a = match, e = sc.beta, o = sc.alpha - e;
+  const int64_t d = max(tlen - qlen, 0);
+  const int64_t more = d > c ? 0 : min(a * (c + 1), o + (a + e) * (c + 1 - d));
+  return h0 + a * qlen - g < o + e * (c + 1) + more;
 }
 
 }  // namespace xt
