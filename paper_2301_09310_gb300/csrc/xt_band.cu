@@ -52,7 +52,7 @@ constexpr int32_t kNoKey = 16383;
 __host__ __device__ constexpr int base_age(int P) { return P + kBaseSteps; }
 
 // NEAR: the P * K slots hold diagonals |i - j| <= hw of a wider band (hw <
-// sc.w); a pair is settled only where the bounds of xt_near.cuh prove its
+// sc.w); a pair is settled only where the bounds of xt_bounds.cuh prove its
 // outputs, and the others go to near_tmp at their bucket's place in the queue
 // (counted in band_left).
 template <int P, int K, bool NEAR>
@@ -66,9 +66,12 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
   constexpr int kGroups = 32 / P;              // per warp
   constexpr int kCheck = P < 8 ? 8 : P;        // steps between two looks at the end
   constexpr int kAge = base_age(P);
+  // few slots: selects instead of branches and shared memory (with 32 slots the
+  // code they add cost 3,001 long pairs 8.2 -> 9.8 ms)
+  constexpr bool kFew = K <= 14;
   __shared__ Batch s_b;
   __shared__ uint32_t s_tbl[8];
-  __shared__ uint32_t s_row[K][kBandThreads];
+  __shared__ uint32_t s_row[K][kBandThreads];  // a lane's row, to take a slot by its number
   if (threadIdx.x == 0) {
     s_b = *bd;
 #pragma unroll
@@ -260,13 +263,19 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
         for (int s = 1; s < K; ++s) slot(s);
         Eout = __viaddmax_s16x2_relu(E, nb2, HA);
         // F must not leave the band on its left
-        switch (kill_s) {
+        if constexpr (kFew) {
+#pragma unroll
+          for (int n = 0; n < K - 1; n += 2)
+            if (kill_s == n) F[n] &= kill;
+        } else {
+          switch (kill_s) {
 #define XT_KILL(n) case n: if (n < K - 1) F[n < K ? n : 0] &= kill; break;
           XT_KILL(0) XT_KILL(2) XT_KILL(4) XT_KILL(6) XT_KILL(8) XT_KILL(10) XT_KILL(12)
           XT_KILL(14) XT_KILL(16) XT_KILL(18) XT_KILL(20) XT_KILL(22) XT_KILL(24) XT_KILL(26)
           XT_KILL(28) XT_KILL(30)
 #undef XT_KILL
           default: break;
+          }
         }
         // this lane's part of row i's maximum.  The column before the query is
         // not part of the row: where it holds the maximum, the slots after it
@@ -278,13 +287,22 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
           const int32_t before = mid - 1 - i - u0;  // slot of column -1
           if (before >= 0 && before < K &&
               ((key & 31u) == (uint32_t)before || ((key >> 16) & 31u) == (uint32_t)before)) {
-#pragma unroll
-            for (int s = 0; s < K; ++s) s_row[s][threadIdx.x] = H[s];
             uint32_t a0 = 0, a1 = 0;
-            for (int s = before + 1; s < K; ++s) {
-              const uint32_t v = s_row[s][threadIdx.x];
-              a0 = max(a0, v << 16 | (uint32_t)(u0 + s));
-              a1 = max(a1, (v & 0xFFFF0000u) | (uint32_t)(u0 + s));
+            if constexpr (kFew) {
+#pragma unroll
+              for (int s = 1; s < K; ++s) {
+                if (s <= before) continue;
+                a0 = max(a0, H[s] << 16 | (uint32_t)(u0 + s));
+                a1 = max(a1, (H[s] & 0xFFFF0000u) | (uint32_t)(u0 + s));
+              }
+            } else {
+#pragma unroll
+              for (int s = 0; s < K; ++s) s_row[s][threadIdx.x] = H[s];
+              for (int s = before + 1; s < K; ++s) {
+                const uint32_t v = s_row[s][threadIdx.x];
+                a0 = max(a0, v << 16 | (uint32_t)(u0 + s));
+                a1 = max(a1, (v & 0xFFFF0000u) | (uint32_t)(u0 + s));
+              }
             }
             m2 = prmt(a0, a1, 0x7632u);
             mu2 = prmt(a0, a1, 0x5410u);
@@ -383,7 +401,7 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
       }
       // Past the query's end: once no cell computed since the last look can
       // raise the best or the end-to-end score, the rows left matter only to
-      // the last live row, which the bounds of xt_near.cuh give.  The look
+      // the last live row, which the bounds of xt_bounds.cuh give.  The look
       // bounds every cell computed after it, and is used one look later, when
       // the rows computed before it have reached the last lane.
       const int32_t i = t8 + 7 - p;

@@ -59,7 +59,7 @@ constexpr int kNumBuckets = kNumClasses * kClassBins;
 // 223 us; 5,000 of 64 bases 180 -> 164 us).
 constexpr int32_t kNearMinPairs = 4096;
 // k_near's narrow band: diagonals |i - j| <= kNearHalf; queries it takes, and
-// the calls' scoring it holds for (see xt_near.cuh)
+// the calls' scoring it holds for (see xt_bounds.cuh)
 constexpr int kNearHalf = 15;
 constexpr int kNearJMax = 9;
 constexpr int kNearMaxQ = (1 << kNearJMax) - 2;

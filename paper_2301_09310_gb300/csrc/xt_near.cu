@@ -1,4 +1,4 @@
-// xt_near.cu -- pairs whose query nearly matches its target (see xt_near.cuh
+// xt_near.cu -- pairs whose query nearly matches its target (see xt_bounds.cuh
 // for the bounds): k_diag settles those whose diagonal alone decides, k_near
 // those decided by a band of 31 diagonals, and the rest go on to the engines.
 #include <algorithm>
