@@ -369,6 +369,7 @@ constexpr int32_t kLaneSlots = 77824;    // one-lane thread slots of a full GPU 
 // time on one lane grows with its length, so a bucket of long queries needs
 // close to a full wave of pairs before the one-lane engine pays; short ones
 // finish fast even when a bucket leaves most lanes idle.
+constexpr int kBandLanesJ = 8;           // 127 bases and longer
 constexpr int kLongJ = 10;               // buckets of queries longer than 510 bases
 inline int32_t lane_min_pairs(int j) { return j >= kLongJ ? 32768 : (j >= 7 ? kBucketSmall : 0); }
 // The longest query of bucket j, and the in-band cells of a pair of query
@@ -466,6 +467,9 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
         const int jj = j < kJMin ? kJMin : j;
         est_cells += (double)cnt[cls][j] * band_cells_est(0.75 * pair_cells_q(jj), sc.w);
       }
+  // the band engine, where it holds the band
+  int bP = 0, bK = 0;
+  const bool band_ok = ctx->near_first && !ctx->forced_P && band_shape(sc, ctx->match, 0, &bP, &bK);
   // long queries: one lane per pair needs many pairs to fill the GPU, but
   // the long buckets of one call run side by side, so when together they
   // hold two full waves of lanes each of them takes the one-lane engine
@@ -474,10 +478,16 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
     for (int j = kLongJ; j < kNumJ; ++j)
       if (lane_ok[j]) long_pairs += cnt[cls][j];
   const bool long_lanes = long_pairs >= 2 * (int64_t)kLaneSlots;
-  auto min_pairs = [&](int jj) { return jj >= kLongJ && long_lanes ? 0 : lane_min_pairs(jj); };
-  // the band engine, where it holds the band
-  int bP = 0, bK = 0, bhw = 0;
-  const bool band_ok = ctx->near_first && !ctx->forced_P && band_shape(sc, ctx->match, 0, &bP, &bK);
+  // Where the band engine is the alternative, 126-base queries and longer need
+  // more pairs before one lane each is faster, the fewer the narrower the band:
+  // lanes cost less a pair, but a pair takes most of a millisecond on one (300k
+  // mixed reads 1,500 -> 807 us a call on bands, 1M 1,650 on lanes and 1,770 on
+  // bands; with w = 50 1,290 and 1,080 us, with w = 200 2,620 and 6,140).
+  auto min_pairs = [&](int jj) {
+    if (jj >= kLongJ) return long_lanes ? 0 : lane_min_pairs(jj);
+    if (jj < kBandLanesJ || !band_ok) return lane_min_pairs(jj);
+    return (int32_t)std::max<int64_t>(kBucketSmall, 2 * (int64_t)kBucketSmall * 201 / (2 * sc.w + 1));
+  };
   // pairs of each launch
   int32_t pairs_of[kMaxLaunches] = {};
   for (int cls : {CLS_PACKED, CLS_NARROW, CLS_WIDE, CLS_NEAR, CLS_BAND}) {
