@@ -25,6 +25,9 @@
 // (shuffles), above that a whole CTA (shuffles plus shared memory).  Pairs are
 // classified by G*K, and each class runs a persistent kernel whose groups take
 // pairs from a counter.
+//
+// Batches of many short queries run two pairs per lane instead (k_bwa_lane): a
+// row then needs no collectives at all.
 #include <algorithm>
 #include <climits>
 #include <cstdint>
@@ -34,6 +37,7 @@
 #include "xt.h"
 #include "xt_common.cuh"
 #include "xt_ctx.cuh"
+#include "xt_near.cuh"
 
 namespace xt {
 namespace {
@@ -46,7 +50,22 @@ namespace {
 #endif
 constexpr int kBwaK = XT_BWA_LANE_COLUMNS;
 static_assert(kBwaK == 16 || kBwaK == 32, "columns per lane: 16 or 32");
-constexpr int kBwaClasses = 8;               // G*K = 64 << class columns
+constexpr int kBwaGroupClasses = 8;          // G*K = 64 << class columns
+// Two pairs per lane: classes by the columns a lane's row buffer has room for; all
+// but the last keep a score in a byte.
+constexpr int kBwaLaneMinQ = 33;
+constexpr int kBwaLaneClasses = 3;
+__host__ __device__ constexpr int bwa_lane_cap(int c) { return 64 << c; }
+// With fewer pairs of a class its last pairs decide, which a group extends
+// sooner (500k / 128k / 64k mixed reads: 7.1 / 2.0 / 1.2 ms on groups alone, 5.2 /
+// 1.6 / 1.5 ms with every class on lanes, those up to 64 bases 0.77 and 0.95 ms of
+// it; 2M: 28.0 and 18.1 ms).
+__host__ __device__ constexpr int32_t bwa_lane_min(int c) { return c == 0 ? 1 << 18 : 1 << 15; }
+constexpr int kBwaClasses = 16;              // of them 11 in use (their order is the queue's)
+// The shortest lane class lies before the narrowest groups, which may take it.
+__host__ __device__ constexpr int bwa_lane_id(int c) { return c == 0 ? 0 : kBwaGroupClasses + c; }
+__host__ __device__ constexpr int bwa_group_id(int c) { return 1 + c; }
+__host__ __device__ constexpr bool bwa_is_lane(int id) { return id == 0 || id > kBwaGroupClasses; }
 constexpr int kBwaWarpThreads = 128;         // CTA size of the warp-segment classes
 constexpr int32_t kBwaNeg = -(1 << 29);      // below any reachable value
 constexpr uint8_t kBwaDone = 0xff;           // pair finished in classify
@@ -61,7 +80,10 @@ constexpr uint32_t kFMask = (1u << kCodeShift) - 1u;
 static_assert((int64_t)XT_MAX_H0 + (int64_t)XT_MAX_LEN * 127 < (1ll << kCodeShift), "F fits below the code");
 static_assert(kBwaLenBuckets * kBwaClasses % kBwaScanThreads == 0, "scan tiling");
 
-static_assert((64 << (kBwaClasses - 1)) == XT_BWA_MAX_WIDTH, "class range must end at the limit");
+static_assert((64 << (kBwaGroupClasses - 1)) == XT_BWA_MAX_WIDTH, "class range must end at the limit");
+
+// Two pairs per lane: the row's key is H * 32 + the chunk of 8 columns.
+constexpr int32_t kBwaLaneMaxH = 1023;
 
 struct BwaScore {
   int32_t match, mismatch, nsc;
@@ -82,6 +104,7 @@ struct BwaArgs {
   xt_result* out;
   int64_t* cells;
   BwaScore sc;
+  int mshift;        // 2^mshift > match
   uint8_t* pclass;   // [n]
   int32_t* order;    // [n] pairs by class, then by query length (longest first)
   int32_t* slots;    // [kBwaClasses * kBwaLenBuckets] pairs per (class, length), then positions
@@ -89,10 +112,12 @@ struct BwaArgs {
   int32_t* heads;    // [kBwaClasses] next pair of each class's persistent kernel
 };
 
-// Slot of a pair of class c and query length ql: classes in order, longer
-// queries first within a class.
-__device__ __forceinline__ int32_t bwa_slot(int c, int32_t ql) {
-  const int32_t b = ql < kBwaLenBuckets - 1 ? ql : kBwaLenBuckets - 1;
+// Slot of a pair of class c, query length ql and seed score h0: classes in order,
+// longer queries first within a class; with two pairs per lane, whose warps sweep
+// the columns alive in any of 64 pairs, pairs of like seed scores together.
+__device__ __forceinline__ int32_t bwa_slot(int c, int32_t ql, int32_t h0) {
+  const int32_t key = !bwa_is_lane(c) ? ql : 4 * (ql - 1) + min(h0 >> 4, 3);
+  const int32_t b = key < kBwaLenBuckets - 1 ? key : kBwaLenBuckets - 1;
   return c * kBwaLenBuckets + (kBwaLenBuckets - 1 - b);
 }
 
@@ -143,9 +168,18 @@ __global__ void k_bwa_classify(BwaArgs a) {
       put_result(a, (int32_t)k, h0, 0, 0, -1, 0, 0, XT_OK, 0);
     } else {
       int c = 0;
-      while ((64 << c) < width) ++c;
+      const int64_t bound = h0 + (int64_t)ql * a.sc.match;
+      if (ql >= kBwaLaneMinQ && ql <= bwa_lane_cap(kBwaLaneClasses - 1) && bound <= kBwaLaneMaxH &&
+          ((bound + 1) << a.mshift) <= 32767) {
+        while (bwa_lane_cap(c) < ql) ++c;
+        if (bound > 255) c = kBwaLaneClasses - 1;
+        c = bwa_lane_id(c);
+      } else {
+        while ((64 << c) < width) ++c;
+        c = bwa_group_id(c);
+      }
       cls = (uint8_t)c;
-      atomicAdd(&a.slots[bwa_slot(c, ql)], 1);
+      atomicAdd(&a.slots[bwa_slot(cls, ql, h0)], 1);
     }
     a.pclass[k] = cls;
   }
@@ -194,7 +228,7 @@ __global__ void k_bwa_scatter(BwaArgs a) {
        k += (int64_t)gridDim.x * blockDim.x) {
     const int c = a.pclass[k];
     if (c == kBwaDone) continue;
-    const int32_t pos = atomicAdd(&a.slots[bwa_slot(c, a.q_len[k])], 1);
+    const int32_t pos = atomicAdd(&a.slots[bwa_slot(c, a.q_len[k], a.h0[k])], 1);
     if (pos >= 0 && pos < a.n) a.order[pos] = (int32_t)k;
   }
 }
@@ -535,6 +569,255 @@ __device__ __forceinline__ void bwa_pair(const BwaArgs& a, const Group<G>& g, Bu
   g.sync();  // the buffer is free for the group's next pair
 }
 
+// -------------------------------------------------------- two pairs per lane
+// A lane sweeps the rows of its two pairs, one in each 16-bit half of every
+// register, in chunks of 8 columns from the first beg to the last end of the
+// two; columns outside a pair's own [beg, end) are masked to dead, and chunks
+// inside every pair's range of the warp skip the masks.  The row above is in
+// shared memory (lane-interleaved: the lanes' chunks differ without bank
+// conflicts): H and F of both pairs in one word, a byte each, or in two where a
+// score passes 255.  Besides a column's cell update the row keeps its maximum
+// with the chunk that holds it and the set of live chunks; the columns are then
+// looked up in those chunks.  A warp's pairs have like lengths (the class is
+// ordered by length), and a row lasts as long as the widest of them.
+//
+// Columns before beg need no mask while beg is the row above's first live column:
+// all before it are dead there, and a dead neighbourhood gives dead cells.
+// Column end of a row, if the query has it, is stored dead (the next row may
+// compute it), column -1
+// the boundary while the row computes column 0.
+//
+// Bounded by latency and issue: shared memory holds 10 warps of 128 columns
+// per SM (ALU pipe 72% busy) and 3 of 256 (31%), so the classes run side by side.
+// Of 500k mixed reads the 185k of 65-128 bases take 1.62 ms and the 78k longer ones
+// 2.59 ms, against 3.10 and 3.27 ms on groups.
+constexpr int kBwaChunk = 8;
+
+template <bool BYTES>
+struct BwaCells;
+template <>
+struct BwaCells<true> {
+  using T = uint32_t;  // H of both pairs, then F
+  static __device__ __forceinline__ void get(T v, uint32_t* h, uint32_t* f) {
+    *h = prmt(v, 0u, 0x4140u);
+    *f = prmt(v, 0u, 0x4342u);
+  }
+  static __device__ __forceinline__ T put(uint32_t h, uint32_t f) { return prmt(h, f, 0x6420u); }
+};
+template <>
+struct BwaCells<false> {
+  using T = uint2;
+  static __device__ __forceinline__ void get(T v, uint32_t* h, uint32_t* f) {
+    *h = v.x;
+    *f = v.y;
+  }
+  static __device__ __forceinline__ T put(uint32_t h, uint32_t f) { return make_uint2(h, f); }
+};
+
+template <int CAP, bool BYTES>
+__global__ void __launch_bounds__(32) k_bwa_lane(BwaArgs a, int32_t off, int32_t count, int cls) {
+  static_assert(CAP % kBwaChunk == 0 && CAP / kBwaChunk <= 32, "chunk index fits the key");
+  using Cells = BwaCells<BYTES>;
+  using T = typename Cells::T;
+  constexpr int C = kBwaChunk;
+  extern __shared__ __align__(16) unsigned char s_lane[];
+  T* const col0 = reinterpret_cast<T*>(s_lane) + 32 + threadIdx.x;  // columns -1 .. CAP + 7
+  uint32_t* const qn0 =
+      reinterpret_cast<uint32_t*>(reinterpret_cast<T*>(s_lane) + 32 * (CAP + C + 1)) + threadIdx.x;
+  const int lane = threadIdx.x;
+  const BwaScore& sc = a.sc;
+  const int32_t oe_ins = sc.o_ins + sc.e_ins, oe_del = sc.o_del + sc.e_del;
+  const uint32_t nai = pack16(-oe_ins, -oe_ins), nbi = pack16(-sc.e_ins, -sc.e_ins);
+  const uint32_t nad = pack16(-oe_del, -oe_del), nbd = pack16(-sc.e_del, -sc.e_del);
+  const uint32_t mcm = 1u << a.mshift;
+  const uint32_t nsc = (uint32_t)(uint8_t)sc.nsc, nn = nsc | (kPadScore << 8);
+  const uint32_t mism4 = (uint32_t)(uint8_t)sc.mismatch * 0x01010101u, mb = (uint32_t)(uint8_t)sc.match;
+  const uint8_t *q_hi = a.q_seq + a.q_bytes, *t_hi = a.t_seq + a.t_bytes;
+  const unsigned full = 0xffffffffu;
+  for (;;) {
+    int32_t base = 0;
+    if (lane == 0) base = atomicAdd(&a.heads[cls], 64);
+    base = __shfl_sync(full, base, 0);
+    if (base >= count) break;
+    int32_t kk[2], ql[2], tl[2], h0[2], w[2], beg[2], end[2];
+    bool live[2];
+    ByteStream ts[2];
+    {
+      ByteStream qs[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int32_t p = base + 2 * lane + h, idx = off + p;
+        int32_t k = p < count && idx >= 0 && idx < a.n ? a.order[idx] : -1;
+        if ((uint32_t)k >= (uint32_t)a.n || a.q_len[k] > CAP) k = -1;  // a corrupt workspace: no pair
+        kk[h] = k;
+        live[h] = k >= 0;
+        ql[h] = k >= 0 ? a.q_len[k] : 1;
+        tl[h] = k >= 0 ? a.t_len[k] : 0;
+        h0[h] = k >= 0 ? a.h0[k] : 1;
+        w[h] = bwa_band(sc, ql[h]);
+        beg[h] = 0;
+        end[h] = min(ql[h], w[h] + 1);
+        qs[h].init(a.q_seq, q_hi, a.q_seq + (k >= 0 ? a.q_off[k] : 0));
+        ts[h].init(a.t_seq, t_hi, a.t_seq + (k >= 0 ? a.t_off[k] : 0));
+      }
+      // row -1: the seed before the query, the insertion run from it in the band
+      col0[-32] = Cells::put(pack16(h0[0], h0[1]), 0u);
+      const int32_t chunks = __reduce_max_sync(full, max(ql[0], ql[1])) / C + 1;
+      for (int32_t c = 0; c < chunks; ++c) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          qn0[(2 * c + h) * 32] = nibbles(qs[h].next(a.q_seq, q_hi), ql[h] - C * c);
+        for (int32_t j = C * c; j < C * c + C; ++j) {
+          int32_t x[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            x[h] = j < ql[h] && j + 1 <= w[h] ? max(h0[h] - oe_ins - sc.e_ins * j, 0) : 0;
+          col0[j * 32] = Cells::put(pack16(x[0], x[1]), 0u);
+        }
+      }
+    }
+    int32_t best[2] = {h0[0], h0[1]}, bi[2] = {-1, -1}, bj[2] = {-1, -1}, max_off[2] = {0, 0};
+    int32_t gscore[2] = {-1, -1}, gtle[2] = {0, 0}, cells[2] = {0, 0};
+    bool edge[2] = {true, true};   // column -1 may hold the boundary
+    bool cut[2] = {false, false};  // the band has cut live columns off before beg
+    uint32_t tw[2] = {0, 0};
+    for (int32_t i = 0;; ++i) {
+      if ((i & 7) == 0)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) tw[h] = nibbles(ts[h].next(a.t_seq, t_hi), 8);
+      bool row[2];
+      int32_t b0 = CAP - 1, e0 = -1;
+      uint32_t tbl[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        row[h] = live[h] && i < tl[h] && beg[h] < end[h];
+        if (row[h]) {
+          b0 = min(b0, beg[h]);
+          e0 = max(e0, min(end[h], ql[h] - 1));
+        }
+        const uint32_t tc = tw[h] & 7u, sh = 8u * tc;
+        tbl[h] = tc >= 4u ? nsc * 0x01010101u : (mism4 & ~(0xFFu << sh)) | mb << sh;
+        tw[h] >>= 4;
+      }
+      const int32_t c0 = b0 / C;
+      const int32_t n_ch = e0 >= 0 ? e0 / C - c0 + 1 : 0;
+      const int32_t most = __reduce_max_sync(full, n_ch);
+      if (most == 0) break;
+      const uint32_t rows2 = (row[0] ? 0xFFFFu : 0u) | (row[1] ? 0xFFFF0000u : 0u);
+      uint32_t D, Y = 0, key = 0, live_c[2] = {0, 0}, unused;
+      Cells::get(col0[(c0 * C - 1) * 32], &D, &unused);
+      for (int32_t cc = 0; cc < most; ++cc) {
+        const bool mine = cc < n_ch;
+        const int32_t c = mine ? c0 + cc : 0, j0 = c * C;
+        T* const p = col0 + j0 * 32;
+        uint32_t in[2], Hu[C], Fu[C], s4[2] = {0, 0}, m8 = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          in[h] = row[h] ? bit_range(cut[h] ? beg[h] - j0 : 0, end[h] - 1 - j0, C) : 0u;
+        }
+        const uint32_t qa = qn0[2 * c * 32], qb = qn0[(2 * c + 1) * 32];
+#pragma unroll
+        for (int u = 0; u < C; ++u) Cells::get(p[u * 32], &Hu[u], &Fu[u]);
+        const bool inside = (!row[0] || in[0] == 0xFFu) && (!row[1] || in[1] == 0xFFu);
+        auto column = [&](int u, uint32_t bm) {
+          if (u % 4 == 0) {
+            s4[0] = prmt(tbl[0], nn, qa >> (u ? 16 : 0));
+            s4[1] = prmt(tbl[1], nn, qb >> (u ? 16 : 0));
+          }
+          constexpr uint32_t kSel[4] = {0xC480u, 0xD591u, 0xE6A2u, 0xF7B3u};
+          const uint32_t S = prmt(s4[0], s4[1], kSel[u % 4]);
+          const uint32_t M = __viaddmin_s16x2(D, S, D * mcm), F = Fu[u];
+          D = Hu[u];
+          const uint32_t H = __vimax3_s16x2(M, Y, F) & bm;
+          const uint32_t Fn = __viaddmax_s16x2_relu(F, nbd, add16x2(M, nad)) & bm;
+          Y = __viaddmax_s16x2_relu(Y, nbi, add16x2(M, nai)) & bm;
+          if (mine) p[u * 32] = Cells::put(H, Fn);
+          asm("max.s16x2 %0, %0, %1;" : "+r"(m8) : "r"(H));
+        };
+        if (__all_sync(full, inside || !mine)) {
+#pragma unroll
+          for (int u = 0; u < C; ++u) column(u, 0xFFFFFFFFu);
+        } else {
+          const uint32_t in2 = in[0] | in[1] << 16;
+#pragma unroll
+          for (int u = 0; u < C; ++u) column(u, prmt(in2 << (15 - u), 0u, 0xBB99u));
+        }
+        m8 = mine ? m8 & rows2 : 0u;
+        asm("max.s16x2 %0, %0, %1;" : "+r"(key) : "r"(m8 * 32u + (uint32_t)cc * 0x00010001u));
+        if (m8 & 0xFFFFu) live_c[0] |= 1u << cc;
+        if (m8 >> 16) live_c[1] |= 1u << cc;
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (!row[h]) continue;
+        auto h_at = [&](int32_t j) -> int32_t {
+          uint32_t hh, ff;
+          Cells::get(col0[j * 32], &hh, &ff);
+          return h ? hi16(hh) : lo16(hh);
+        };
+        if (end[h] == ql[h]) {
+          const int32_t gv = h_at(ql[h] - 1);
+          if (gv >= gscore[h]) {
+            gscore[h] = gv;
+            gtle[h] = i + 1;
+          }
+        }
+        const int32_t kv = h ? hi16(key) : lo16(key), m = kv >> 5;
+        if (m == 0) {
+          live[h] = false;
+          continue;
+        }
+        cells[h] += end[h] - beg[h];
+        const int32_t fc = (c0 + __ffs(live_c[h]) - 1) * C, lc = (c0 + 31 - __clz(live_c[h])) * C;
+        int32_t fl = 0, ll = 0;
+#pragma unroll
+        for (int u = 0; u < C; ++u) {
+          if (h_at(fc + C - 1 - u) > 0) fl = C - 1 - u;
+          if (h_at(lc + u) > 0) ll = u;
+        }
+        if (m > best[h] || (sc.zdrop > 0 && best[h] - m > sc.zdrop)) {
+          const int32_t mc = (c0 + (kv & 31)) * C;
+          int32_t mj = 0;
+#pragma unroll
+          for (int u = 0; u < C; ++u)
+            if (h_at(mc + u) == m) mj = mc + u;
+          if (m > best[h]) {
+            best[h] = m;
+            bi[h] = i;
+            bj[h] = mj;
+            max_off[h] = max(max_off[h], abs(mj - i));
+          } else {
+            const int32_t di = i - bi[h], dj = mj - bj[h];
+            const int32_t drop =
+                best[h] - m - (di > dj ? (di - dj) * sc.e_del : (dj - di) * sc.e_ins);
+            if (drop > sc.zdrop) live[h] = false;
+          }
+        }
+        beg[h] = fc + fl;
+        if (beg[h] < i + 1 - w[h]) {
+          beg[h] = i + 1 - w[h];
+          cut[h] = true;
+        }
+        if (edge[h]) {  // the boundary's H for the next row's column 0
+          edge[h] = beg[h] == 0;
+          const int32_t hb =
+              edge[h] && i + 1 <= w[h] ? max(0, h0[h] - oe_del - sc.e_del * i) : 0;
+          uint32_t hh, ff;
+          Cells::get(col0[-32], &hh, &ff);
+          hh = h ? (hh & 0xFFFFu) | (uint32_t)hb << 16 : (hh & 0xFFFF0000u) | (uint32_t)hb;
+          col0[-32] = Cells::put(hh, 0u);
+        }
+        end[h] = min(min(lc + ll + 2, i + w[h] + 2), ql[h]);
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (kk[h] >= 0)
+        put_result(a, kk[h], best[h], bj[h] + 1, bi[h] + 1, gscore[h], gtle[h], max_off[h], XT_OK,
+                   cells[h]);
+  }
+}
+
 // Columns per lane K and lanes per pair G of a class (capacity 64 << class).
 template <int C>
 struct BwaClass {
@@ -552,7 +835,7 @@ struct BwaClass {
 // dependency latency.
 template <int C>
 __global__ void __launch_bounds__(kBwaWarpThreads, 6) k_bwa_seg(BwaArgs a, int32_t off,
-                                                                int32_t count) {
+                                                                int32_t count, int cls) {
   using Cl = BwaClass<C>;
   constexpr int G = Cl::G;
   __shared__ int2 s_buf[Cl::kPairsPerBlock * Cl::kBufElems];
@@ -564,7 +847,7 @@ __global__ void __launch_bounds__(kBwaWarpThreads, 6) k_bwa_seg(BwaArgs a, int32
   const int gi = threadIdx.x / G;
   const RowBuf<S> buf{s_buf + (gi / S) * S * Cl::kBufElems + gi % S};
   for (;;) {
-    const int32_t p = g.claim(&a.heads[C]);
+    const int32_t p = g.claim(&a.heads[cls]);
     if (p >= count) break;
     const int32_t idx = off + p;
     if (idx < 0 || idx >= a.n) break;  // defensive: order index out of range
@@ -585,7 +868,7 @@ __global__ void __launch_bounds__(BwaClass<C>::G, 512 / BwaClass<C>::G)
   Group<G> g;
   g.init(&s);
   for (;;) {
-    const int32_t p = g.claim(&a.heads[C]);
+    const int32_t p = g.claim(&a.heads[bwa_group_id(C)]);
     if (p >= count) break;
     const int32_t idx = off + p;
     if (idx < 0 || idx >= a.n) break;
@@ -596,10 +879,10 @@ __global__ void __launch_bounds__(BwaClass<C>::G, 512 / BwaClass<C>::G)
 }
 
 template <int C>
-cudaError_t launch_class(xt_ctx* ctx, const BwaArgs& a, int32_t off, int32_t count,
+cudaError_t launch_class(xt_ctx* ctx, const BwaArgs& a, int32_t off, int32_t count, int cls,
                          cudaStream_t stream) {
   using Cl = BwaClass<C>;
-  int& resident = ctx->bwa_blocks[C];
+  int& resident = ctx->bwa_blocks[bwa_group_id(C)];
   const size_t dyn = Cl::kSeg ? 0 : Cl::kSmem;
   if (resident == 0) {
     cudaError_t e;
@@ -618,23 +901,54 @@ cudaError_t launch_class(xt_ctx* ctx, const BwaArgs& a, int32_t off, int32_t cou
   const int64_t want = ((int64_t)count + Cl::kPairsPerBlock - 1) / Cl::kPairsPerBlock;
   const int grid = (int)std::min<int64_t>(want, (int64_t)resident * ctx->num_sms);
   if constexpr (Cl::kSeg)
-    k_bwa_seg<C><<<grid, Cl::kThreads, 0, stream>>>(a, off, count);
+    k_bwa_seg<C><<<grid, Cl::kThreads, 0, stream>>>(a, off, count, cls);
   else
     k_bwa_cta<C><<<grid, Cl::kThreads, dyn, stream>>>(a, off, count);
+  return cudaGetLastError();
+}
+
+template <int C>
+cudaError_t launch_lane_class(xt_ctx* ctx, const BwaArgs& a, int32_t off, int32_t count,
+                              cudaStream_t stream) {
+  constexpr int kCap = bwa_lane_cap(C);
+  constexpr bool kBytes = C < kBwaLaneClasses - 1;
+  constexpr size_t kSmem = 32 * ((size_t)(kCap + kBwaChunk + 1) * sizeof(typename BwaCells<kBytes>::T) +
+                                 (size_t)(kCap / kBwaChunk + 1) * 2 * sizeof(uint32_t));
+  auto kern = k_bwa_lane<kCap, kBytes>;
+  int& resident = ctx->bwa_blocks[bwa_lane_id(C)];
+  if (resident == 0) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kern, 32, kSmem);
+    if (e != cudaSuccess) return e;
+    if (resident < 1) resident = 1;
+  }
+  const int64_t want = ((int64_t)count + 63) / 64;
+  const int grid = (int)std::min<int64_t>(want, (int64_t)resident * ctx->num_sms);
+  kern<<<grid, 32, kSmem, stream>>>(a, off, count, bwa_lane_id(C));
   return cudaGetLastError();
 }
 
 cudaError_t launch_bwa_class(xt_ctx* ctx, const BwaArgs& a, int cls, int32_t off, int32_t count,
                              cudaStream_t stream) {
   switch (cls) {
-    case 0: return launch_class<0>(ctx, a, off, count, stream);
-    case 1: return launch_class<1>(ctx, a, off, count, stream);
-    case 2: return launch_class<2>(ctx, a, off, count, stream);
-    case 3: return launch_class<3>(ctx, a, off, count, stream);
-    case 4: return launch_class<4>(ctx, a, off, count, stream);
-    case 5: return launch_class<5>(ctx, a, off, count, stream);
-    case 6: return launch_class<6>(ctx, a, off, count, stream);
-    case 7: return launch_class<7>(ctx, a, off, count, stream);
+    case bwa_lane_id(0): return launch_lane_class<0>(ctx, a, off, count, stream);
+    case bwa_group_id(0): return launch_class<0>(ctx, a, off, count, cls, stream);
+    case bwa_group_id(1): return launch_class<1>(ctx, a, off, count, cls, stream);
+    case bwa_group_id(2): return launch_class<2>(ctx, a, off, count, cls, stream);
+    case bwa_group_id(3): return launch_class<3>(ctx, a, off, count, cls, stream);
+    case bwa_group_id(4): return launch_class<4>(ctx, a, off, count, cls, stream);
+    case bwa_group_id(5): return launch_class<5>(ctx, a, off, count, cls, stream);
+    case bwa_group_id(6): return launch_class<6>(ctx, a, off, count, cls, stream);
+    case bwa_group_id(7): return launch_class<7>(ctx, a, off, count, cls, stream);
+    case bwa_lane_id(1):
+      return count >= bwa_lane_min(1) ? launch_lane_class<1>(ctx, a, off, count, stream)
+                                      : launch_class<1>(ctx, a, off, count, cls, stream);
+    case bwa_lane_id(2):
+      return count >= bwa_lane_min(2) ? launch_lane_class<2>(ctx, a, off, count, stream)
+                                      : launch_class<2>(ctx, a, off, count, cls, stream);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -705,6 +1019,8 @@ extern "C" xt_status xt_extend_batch_bwa(xt_ctx* ctx, const uint8_t* q_seq, int6
   // a band wider than any pair changes nothing; clamp so index arithmetic stays in int32
   a.sc.w = scr->w > 2 * XT_MAX_LEN ? 2 * XT_MAX_LEN : scr->w;
   a.sc.zdrop = scr->zdrop; a.sc.end_bonus = scr->end_bonus;
+  a.mshift = 0;
+  while ((1 << a.mshift) < scr->match + 1) ++a.mshift;
   a.pclass = reinterpret_cast<uint8_t*>(ws + o_cls);
   a.order = reinterpret_cast<int32_t*>(ws + o_order);
   a.slots = reinterpret_cast<int32_t*>(ws + o_slots);
@@ -740,9 +1056,34 @@ extern "C" xt_status xt_extend_batch_bwa(xt_ctx* ctx, const uint8_t* q_seq, int6
   if (total == 0) return XT_OK;
   k_bwa_scatter<<<grid, threads, 0, st>>>(a);
   e = cudaGetLastError();
-  // widest groups first: they hold the longest rows
-  for (int c = kBwaClasses - 1; c >= 0 && e == cudaSuccess; --c)
-    if (cnt[c] > 0) e = launch_bwa_class(ctx, a, c, off[c], cnt[c], st);
+  // The classes run side by side on the context's streams, the widest groups and
+  // the longest queries first: they hold the longest rows, and what limits one
+  // class (shared memory, issue, its last pairs) leaves room for another.
+  if (cnt[bwa_lane_id(0)] < bwa_lane_min(0)) {  // its pairs go first in the narrowest groups' launch
+    cnt[bwa_group_id(0)] += cnt[bwa_lane_id(0)];
+    off[bwa_group_id(0)] = off[bwa_lane_id(0)];
+    cnt[bwa_lane_id(0)] = 0;
+  }
+  int used = 0;
+  for (int c = 0; c < kBwaClasses; ++c) used += cnt[c] > 0;
+  const int nb = std::min(ctx->branches, used);
+  if (e == cudaSuccess && nb > 1) {
+    e = cudaEventRecord(ctx->fork_ev, st);
+    for (int b = 0; e == cudaSuccess && b < nb; ++b)
+      e = cudaStreamWaitEvent(ctx->aux[b], ctx->fork_ev, 0);
+  }
+  int rr = 0;
+  auto launch = [&](int c) {
+    if (cnt[c] > 0 && e == cudaSuccess)
+      e = launch_bwa_class(ctx, a, c, off[c], cnt[c], nb > 1 ? ctx->aux[rr++ % nb] : st);
+  };
+  for (int c = kBwaGroupClasses - 1; c >= 2; --c) launch(bwa_group_id(c));
+  for (int c = kBwaLaneClasses - 1; c >= 1; --c) launch(bwa_lane_id(c));
+  for (int id : {bwa_group_id(1), bwa_lane_id(0), bwa_group_id(0)}) launch(id);
+  for (int b = 0; nb > 1 && b < nb && e == cudaSuccess; ++b) {
+    e = cudaEventRecord(ctx->join_ev[b], ctx->aux[b]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ctx->join_ev[b], 0);
+  }
   if (e != cudaSuccess) return ctx_cuda_fail(ctx, e, "BWA extension");
   ctx->calls++;
   return XT_OK;

@@ -78,7 +78,7 @@ constexpr int kMaxChunks = 8;
 // the read-back regions do not overlap (bucket counts: two aligned tables)
 static_assert(2 * (4 * kNumClasses * kNumJ + 255) / 4 <= kSegHostSeedTotals, "bucket counts");
 static_assert(kSegHostSeedTotals + 4 <= kSegHostBwaCounts, "seed totals");
-static_assert(kSegHostBwaCounts + 16 <= kSegHostChunkEnds, "BWA class sizes");
+static_assert(kSegHostBwaCounts + 32 <= kSegHostChunkEnds, "BWA class sizes");
 static_assert(kSegHostChunkEnds + 4 * kMaxChunks <= kSegHostWords, "chunk ends");
 constexpr int32_t kChunkPairs = 1 << 20;   // calls of 2 x this many pairs or more are chunked
 constexpr int32_t kChunkFirstMin = 1 << 18; // pairs in the first (smallest) chunk at least
@@ -143,7 +143,7 @@ struct xt_ctx {
   // BWA-MEM-compatible calls: class bytes, order, counters
   void* bwa_ws = nullptr;
   size_t bwa_ws_bytes = 0;
-  int bwa_blocks[8] = {};        // resident CTAs per SM of each group-size kernel (0: unknown)
+  int bwa_blocks[16] = {};       // resident CTAs per SM of each class's kernel (0: unknown)
   // host-buffer calls: a copy stream and its events (chunked staging)
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t stage_ev[2 * xt::kMaxChunks + 2] = {};
