@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kQueueThreads)
 template <int R, bool PACKED, bool GRING, bool QSTAGE, int TB = 6>
 __global__ void __launch_bounds__(kLaneThreads, 4)
     k_lane(const Batch* __restrict__ bd, Score sc, Work w, int cls, int j_lo, int j_hi,
-           int head_id, int rs_log2, void* gring, int mparam, int qs_log2) {
+           int head_id, int rs_log2, void* gring, int mparam, int qs_log2, int cls2) {
   // batch arguments stay in shared memory and are read where used
   __shared__ Batch s_b;
   if (threadIdx.x == 0) s_b = *bd;
@@ -314,16 +314,22 @@ __global__ void __launch_bounds__(kLaneThreads, 4)
   pipe.slot0 = reinterpret_cast<int2*>(s_dyn) + threadIdx.x;
   const int32_t begin = w.seg_begin[cls * kNumJ + j_hi];
   const int32_t end = w.seg_end[cls * kNumJ + j_lo];
+  // (the second class starts at a multiple of 32: no warp mixes the two, whose
+  // lengths differ)
+  const int32_t begin2 = cls2 >= 0 ? w.seg_begin[cls2 * kNumJ + j_hi] : 0;
+  const int32_t end2 = cls2 >= 0 ? w.seg_end[cls2 * kNumJ + j_lo] : 0;
+  const int32_t first = (end - begin + 31) & ~31;
   int32_t* head = w.heads + head_id;
   // rounds of 32 consecutive pairs per warp, all lanes together
   for (;;) {
     int32_t base = 0;
     if (lane == 0) base = atomicAdd(head, 32);
-    base = begin + __shfl_sync(0xffffffffu, base, 0);
-    if (base >= end) break;
-    const int32_t idx = base + lane;
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (base >= first + (end2 - begin2)) break;
+    const bool second = base >= first;
+    const int32_t idx = (second ? begin2 + (base - first) : begin + base) + lane;
     Pair pr;
-    int32_t k = idx < end ? w.order[idx] : -1;
+    int32_t k = idx < (second ? end2 : end) ? w.order[idx] : -1;
     // an index outside the batch would mean a corrupt workspace: the lane
     // idles rather than read outside the caller's arrays
     const bool valid = (uint32_t)k < (uint32_t)b.n;
@@ -742,7 +748,7 @@ static cudaError_t launch_lane_t(const Batch* b, const Score& sc, const Work& w,
   cudaError_t e = raise_smem_limit(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<L.grid, kLaneThreads, smem, stream>>>(b, sc, w, L.cls, L.j_lo, L.j_hi, head_id,
-                                               L.rs_log2, gring, L.mparam, L.j_hi);
+                                               L.rs_log2, gring, L.mparam, L.j_hi, L.cls2);
   return cudaGetLastError();
 }
 

@@ -94,6 +94,7 @@ struct Launch {
   bool lane = false;         // one-lane engine (k_lane) instead of the group engine (k_queue)
   bool band = false;         // band engine (k_band): P lanes of R slots
   int near_hw = 0;           // > 0: on a narrower band of this half width
+  int cls2 = -1;             // one-lane engine: then this class's pairs of the same buckets
   bool after_prev = false;   // takes the pairs the launch before it left, on its stream
   int P = 1, R = 8;          // lanes per pair, rows per lane-strip (per half when packed)
   int rs_log2 = 0;           // ring entries per group = 1 << rs_log2
