@@ -362,6 +362,13 @@ void plan_batched(xt_ctx* ctx, const Score& sc, Plan* pl, bool allow_gring = tru
 // ---- count-aware planning (the batched path): classify runs first with
 // per-bucket flags that do not depend on the counts, then every non-empty
 // bucket is planned from its own pair count.
+// Fewer NEAR pairs go to the engines at once: k_near holds a pair's 31 diagonals in
+// one lane and takes 0.6 us a row, which the engines' first launches then wait
+// for (5,000 pairs of 64 / 250 bases 139 / 970 us a call with it, 112 / 484
+// without; 40k mixed reads 466 and 323, 80k 475 and 539).  Longer queries in the
+// call hide that time, and the pass saves work beside them (6,000 streamed pairs
+// 819 and 901 us).
+constexpr int32_t kNearPassMin = 8192;
 constexpr int kNearLeft = 3;             // one NEAR pair in so many is left for the engines
 constexpr int32_t kBucketSmall = XT_SMALL_BUCKET;  // fewer pairs: a bucket cannot fill the GPU
 constexpr int32_t kLaneSlots = 77824;    // one-lane thread slots of a full GPU (152 x 4 x 128)
@@ -450,11 +457,15 @@ Launch queue_launch(const xt_ctx* ctx, int cls, int j, int P, int R, int lg) {
 void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFlags& jf,
                  const bool* lane_ok, Plan* pl) {
   pl->jf = jf;
-  // the NEAR class is planned for the pairs k_near is expected to leave
-  for (int j = 0; j < kNumJ; ++j) {
-    int32_t& c = cnt[CLS_NEAR][j];
-    pl->near_pairs += c;
-    c = (c + kNearLeft - 1) / kNearLeft;
+  // the NEAR class is planned for the pairs k_near is expected to leave, or for
+  // all of them where it does not run
+  int32_t near = 0, longer = 0;
+  for (int j = 0; j < kNumJ; ++j) near += cnt[CLS_NEAR][j];
+  for (int cls = CLS_PACKED; cls < kNumClasses; ++cls)
+    for (int j = kNearJMax + 1; j < kNumJ; ++j) longer += cnt[cls][j];
+  if (near >= kNearPassMin || (near > 0 && longer > 0)) {
+    pl->near_pairs = near;
+    for (int j = 0; j < kNumJ; ++j) cnt[CLS_NEAR][j] = (cnt[CLS_NEAR][j] + kNearLeft - 1) / kNearLeft;
   }
   pl->near_grid = near_grid(pl->near_pairs, ctx->num_sms);
   const bool saved = ctx->plan_small;
@@ -501,7 +512,7 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
       bool lane = false, band = false;
       if (cls == CLS_BAND && !band_ok) {
         // a narrow band first, then the group engine for the pairs it leaves
-        if (pl->n_launch >= kMaxLaunches - 2 ||
+        if (pl->n_launch >= kMaxLaunches - 3 ||
             !band_near_shape(sc, ctx->match, jj, &L.P, &L.R, &L.near_hw)) {
           pl->bad = true;
           continue;
@@ -812,7 +823,7 @@ cudaError_t enqueue_dp(xt_ctx* ctx, bool plain, const Plan& pl, int plain_rs, co
     const bool leads = i + 1 < pl.n_launch && pl.launch[i + 1].after_prev;
     const bool ring = L.global_ring || (leads && pl.launch[i + 1].global_ring);
     if (!L.after_prev) st = nb > 1 ? ctx->aux[ring && pl.pool_serial ? 0 : (rr++ % nb)] : stream;
-    if (L.cls == CLS_NEAR && nb > 1) e = cudaStreamWaitEvent(st, ctx->near_ev, 0);
+    if (near && L.cls == CLS_NEAR && nb > 1) e = cudaStreamWaitEvent(st, ctx->near_ev, 0);
     if (e != cudaSuccess) break;
     void* gring = L.global_ring ? static_cast<void*>(reinterpret_cast<char*>(ctx->pool) + L.pool_off)
                                 : nullptr;
