@@ -58,6 +58,7 @@ BWA_ALU_OPS_PER_CELL, BWA_OPS_PER_CELL = 9, 10
 # multiply-add pipe instead)
 ALU_PROBES = ("max3.s16x2", "addmax.relu.s16x2", "prmt", "max3.s32")
 LANE_MAX_QLEN = 510  # one-lane (packed-capable) buckets: qlen + 2 <= 2^9
+BAND_MAX_DIAGONALS = 1024  # the band engine: 32 lanes of 32 diagonals
 WORKLOAD_TEXT = {
     "c1_tiny": "1,000 pairs, 100 bp queries, 116 bp targets, 2% sub / 0.2% indel",
     "c2_short": "1,000,000 pairs, qlen U[1,150], tlen = qlen + 200, 1% sub / 0.1% indel, 5% unrelated",
@@ -223,15 +224,17 @@ def aggregate(world, units_local: float, seconds_local: float):
 
 def cell_updates(b, cells, sc):
     """Cell updates the extension DP needs for this batch: cells of pairs that
-    the packed 16-bit class takes (score bound B = h0 + match*min(qlen,tlen)
-    with (B+1)*2^k and B*64+63 within int16, query within the one-lane
+    run in 16-bit halves (score bound B = h0 + match*min(qlen,tlen) with
+    (B+1)*2^k within int16, on the band engine where it holds the band, else on
+    one lane with B*64+63 within int16 and the query within the one-lane
     buckets) count half (two cells per update), the rest one each."""
     m = sc.match
     k = 0
     while (1 << k) < m + 1:
         k += 1
     bound = b.h0.astype(np.int64) + m * np.minimum(b.q_len, b.t_len).astype(np.int64)
-    packed = ((bound + 1) << k <= 32767) & (bound * 64 + 63 <= 32767) & (b.q_len <= LANE_MAX_QLEN)
+    lane = (bound * 64 + 63 <= 32767) & (b.q_len <= LANE_MAX_QLEN)
+    packed = ((bound + 1) << k <= 32767) & (lane | (2 * sc.w + 1 <= BAND_MAX_DIAGONALS))
     c = cells.astype(np.float64)
     updates = 0.5 * c[packed].sum() + c[~packed].sum()
     return float(updates), float(c[packed].sum() / max(c.sum(), 1.0))
@@ -656,7 +659,8 @@ def bwa_leg(b, wl, args, local, stream, rates, mhz):
                                            "all": BWA_OPS_PER_CELL},
                              kernel="whole call (classify, order, k_bwa)"),
             "scoring": list(sc.as_tuple()),
-            "kernel": "k_bwa: one pair per group of 2..256 lanes, a row's live columns at a time, int32"}
+            "kernel": "k_bwa: two pairs per lane (int16x2, queries of 33-256 bases in large classes), "
+                      "else one pair per group of 2..256 lanes (int32), a row's live columns at a time"}
 
 
 def packed4_leg(b, wl, args, local, stream, cells_step):
@@ -761,7 +765,8 @@ def c4_leg(args, local, stream, rates, mhz):
     return {"value": round(n_cells / (ms / 1e3) / 1e9, 3), "unit": "GCUPS",
             "ms_per_step": round(ms, 3), "ext_per_s": round(b.n / (ms / 1e3), 1),
             "useful_cells": n_cells, "pairs": b.n, "scoring": wl.scoring.as_tuple(),
-            "dtype": "int32" if packed_frac <= 0.0 else "int16x2+int32",
+            "dtype": ("int16x2" if packed_frac >= 1.0 else
+                      "int32" if packed_frac <= 0.0 else "int16x2+int32"),
             "workload": f"c4_long: {WORKLOAD_TEXT['c4_long']}",
             "plain": {"value": round(n_cells / (pms / 1e3) / 1e9, 3), "unit": "GCUPS",
                       "ms_per_step": round(pms, 3)},

@@ -141,9 +141,10 @@ static_assert(kSlots < (1 << kKeyBits) && kSlots <= 32, "slot index fits the row
 // sign-extended, side by side.
 //
 // Bounded by the integer ALU pipe: 31 slots of about 10 instructions per row
-// of two pairs.  Of the same 4M reads it takes the 1.2M left and settles half
-// of them in 1.53 ms; the call went from 18.3 to 5.0 ms (1M 150-base reads: 4.6
-// to 1.3 ms), as the full band's 201 diagonals are left to 15% of the pairs.
+// of two pairs.  Of the same 4M reads it took the 1.2M left and settled half of
+// them in 1.53 ms, 1.20 ms now that k_diag keeps from it the short ones it could
+// not settle; the call went from 18.3 to 4.5 ms (1M 150-base reads: 4.6 to 1.15
+// ms), as the full band's 201 diagonals are left to 15% of the pairs.
 // 31 diagonals are what two pairs' cells, with 16 bits each, leave of 168
 // registers; they admit a loss of 21 against a perfect match.
 __global__ void __launch_bounds__(kNearThreads, kNearBlocks)
