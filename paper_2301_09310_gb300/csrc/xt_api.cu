@@ -376,6 +376,7 @@ constexpr int32_t kLaneSlots = 77824;    // one-lane thread slots of a full GPU 
 // time on one lane grows with its length, so a bucket of long queries needs
 // close to a full wave of pairs before the one-lane engine pays; short ones
 // finish fast even when a bucket leaves most lanes idle.
+constexpr int kGroupMaxJ = 7;            // up to 126 bases
 constexpr int kBandLanesJ = 8;           // 127 bases and longer
 constexpr int kLongJ = 10;               // buckets of queries longer than 510 bases
 inline int32_t lane_min_pairs(int j) { return j >= kLongJ ? 32768 : (j >= 7 ? kBucketSmall : 0); }
@@ -552,8 +553,13 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
         }
       }
       // too few pairs for one lane each: groups of the band engine, whose rows
-      // stop at the query's end and which work in 16 bits
-      if (!lane && band_ok && packed_class(cls) && !tuned(ctx, sc.w, jj)) band = true;
+      // stop at the query's end and which work in 16 bits.  Queries of up to 126
+      // bases stay on the group engine, which has all their rows in flight at once
+      // where the band engine takes 0.6 us a row (1,000 pairs of 100 bases 121 and
+      // 95 us a call, 5,000 of 64 bases 111 and 94 us, of 128 bases 200 on bands and
+      // as much with 32 lanes)
+      if (!lane && band_ok && packed_class(cls) && !tuned(ctx, sc.w, jj) && jj > kGroupMaxJ)
+        band = true;
       if (band) {
         band_shape(sc, ctx->match, c, &L.P, &L.R);
         L.cls = cls; L.band = true;
@@ -573,6 +579,10 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
                               std::max(est_cells, 1.0);
           int want = 4;  // two-lane groups measured slower than four on every call size
           while (want < 32 && want < need) want *= 2;
+          // short queries: 8 rows a lane for as many rows as the bucket's longest
+          // query has, one chunk of them (32 lanes idle half: 5,000 pairs of 64 bases
+          // 109 us a call, 94 so)
+          if (jj <= kGroupMaxJ) want = std::max(4, 1 << (jj - 3));
           for (int q = want; q >= 2 && P == 0; q /= 2) {
             const int l = queue_ring_log2(jj, sc.w, q, 8);
             if (l <= kQueueRsCapLog2 && queue_smem_bytes(q, l) <= (size_t)ctx->smem_optin / 2 - 1024) {
