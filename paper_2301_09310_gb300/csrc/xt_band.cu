@@ -30,7 +30,7 @@
 // instruction with the tag as an immediate): a multiply-add needed the tag in
 // a register and took 378 ms.  With few slots and one warp per scheduler a row's
 // dependent instructions (330 with 8 slots) bound it, 0.57 us: 1,000 pairs of 100
-// bases 85 us.  A narrow band first: 5,000 pairs of 1,024 bases, w = 1,024, 4.90 ->
+// bases 85 us (so queries that short stay on the group engine).  A narrow band first: 5,000 pairs of 1,024 bases, w = 1,024, 4.90 ->
 // 1.46 ms a call on 512 diagonals.
 #include <algorithm>
 
