@@ -558,7 +558,10 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
       // where the band engine takes 0.6 us a row (1,000 pairs of 100 bases 121 and
       // 95 us a call, 5,000 of 64 bases 111 and 94 us, of 128 bases 200 on bands and
       // as much with 32 lanes)
-      if (!lane && band_ok && packed_class(cls) && !tuned(ctx, sc.w, jj) && jj > kGroupMaxJ)
+      // (so do a few pairs of up to 254 bases under a band of more diagonals than one
+      // warp holds at 8 a lane: 1,000 pairs of 250 bases, w = 250, 266 and 169 us)
+      const bool few_wide = jj == kGroupMaxJ + 1 && c < kBucketSmall / 4 && 2 * (int64_t)sc.w + 1 > 256;
+      if (!lane && band_ok && packed_class(cls) && !tuned(ctx, sc.w, jj) && jj > kGroupMaxJ && !few_wide)
         band = true;
       if (band) {
         band_shape(sc, ctx->match, c, &L.P, &L.R);
