@@ -60,16 +60,16 @@ struct NearEnd {
 // when it is not known.
 __device__ __forceinline__ int32_t near_last_row(const NearEnd& n, int32_t qlen, int32_t tlen,
                                                  int32_t h0, int32_t match, const Score& sc) {
-  const int64_t e = sc.beta, o = sc.alpha - sc.beta;
-  const int64_t d_end = n.row - (qlen - 1);
+  const int32_t e = sc.beta, o = sc.alpha - sc.beta;
+  const int32_t d_end = n.row - (qlen - 1);
   if (sc.zdrop > 0 && n.best - n.g + o + e * (n.d_best - d_end) > sc.zdrop) return -1;
-  const int64_t cap = min((int64_t)tlen - 1, (int64_t)qlen - 1 + sc.w);
-  if (cap <= n.row || e * (cap - n.row) <= (int64_t)n.g - o - 1) return (int32_t)cap;
-  const int64_t y = n.g + e * d_end;
-  const int64_t p = h0 + (int64_t)match * qlen;
+  const int32_t cap = (int32_t)min((int64_t)tlen - 1, (int64_t)qlen - 1 + sc.w);
+  if (cap <= n.row || e * (cap - n.row) <= n.g - o - 1) return cap;
+  const int32_t y = n.g + e * d_end;
+  const int32_t p = h0 + match * qlen;
   if (e == 0 || d_end < 0 || y < n.best || p - y > o) return -1;
-  const int64_t k = y - o - 1 >= 0 ? (y - o - 1) / e : 0;
-  return (int32_t)min(cap, max((int64_t)n.row, qlen - 1 + k));
+  const int32_t k = y - o - 1 >= 0 ? (y - o - 1) / e : 0;
+  return min(cap, max(n.row, qlen - 1 + k));
 }
 
 // (1') on row i with best the running best of the row or a lower one.

@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kQueueThreads)
 // Every lane extends whole pairs on its own; the warp takes consecutive queue
 // slots (one atomicAdd per warp per round), so neighbouring lanes get pairs
 // of nearly equal length.
-template <int R, bool PACKED, bool GRING, bool QSTAGE, int TB = 6>
+template <int R, bool PACKED, bool GRING, bool QSTAGE, int TB, int LIVE>
 __global__ void __launch_bounds__(kLaneThreads, 4)
     k_lane(const Batch* __restrict__ bd, Score sc, Work w, int cls, int j_lo, int j_hi,
            int head_id, int rs_log2, void* gring, int mparam, int qs_log2, int cls2) {
@@ -290,7 +290,16 @@ __global__ void __launch_bounds__(kLaneThreads, 4)
   using T = typename Ring<PACKED>::T;
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ uint32_t s_prof[8];
-  if (threadIdx.x == 0) copy_profile(sc, s_prof);
+  // the queue's runs of the two classes, read once a round: in registers they
+  // cost the pair's steps 4-5% (1M mixed reads 4.21 -> 4.02 ms a call)
+  __shared__ int32_t s_begin[2], s_end[2];
+  if (threadIdx.x == 0) {
+    copy_profile(sc, s_prof);
+    s_begin[0] = w.seg_begin[cls * kNumJ + j_hi];
+    s_end[0] = w.seg_end[cls * kNumJ + j_lo];
+    s_begin[1] = cls2 >= 0 ? w.seg_begin[cls2 * kNumJ + j_hi] : 0;
+    s_end[1] = cls2 >= 0 ? w.seg_end[cls2 * kNumJ + j_lo] : 0;
+  }
   __syncthreads();
   const int lane = threadIdx.x & 31;
   // ring: column c of lane t at [(c & mask) * kLaneThreads + t], so the lanes
@@ -312,24 +321,21 @@ __global__ void __launch_bounds__(kLaneThreads, 4)
   // 32-bit global rings feed their entries through shared-memory slots
   RingPipe<int2> pipe;
   pipe.slot0 = reinterpret_cast<int2*>(s_dyn) + threadIdx.x;
-  const int32_t begin = w.seg_begin[cls * kNumJ + j_hi];
-  const int32_t end = w.seg_end[cls * kNumJ + j_lo];
-  // (the second class starts at a multiple of 32: no warp mixes the two, whose
-  // lengths differ)
-  const int32_t begin2 = cls2 >= 0 ? w.seg_begin[cls2 * kNumJ + j_hi] : 0;
-  const int32_t end2 = cls2 >= 0 ? w.seg_end[cls2 * kNumJ + j_lo] : 0;
-  const int32_t first = (end - begin + 31) & ~31;
   int32_t* head = w.heads + head_id;
   // rounds of 32 consecutive pairs per warp, all lanes together
   for (;;) {
     int32_t base = 0;
     if (lane == 0) base = atomicAdd(head, 32);
     base = __shfl_sync(0xffffffffu, base, 0);
-    if (base >= first + (end2 - begin2)) break;
-    const bool second = base >= first;
-    const int32_t idx = (second ? begin2 + (base - first) : begin + base) + lane;
+    // (the second class starts at a multiple of 32: no warp mixes the two, whose
+    // lengths differ)
+    const volatile int32_t *begin = s_begin, *end = s_end;
+    const int32_t first = (end[0] - begin[0] + 31) & ~31;
+    if (base >= first + (end[1] - begin[1])) break;
+    const int second = base >= first;
+    const int32_t idx = begin[second] + base - (second ? first : 0) + lane;
     Pair pr;
-    int32_t k = idx < (second ? end2 : end) ? w.order[idx] : -1;
+    int32_t k = idx < end[second] ? w.order[idx] : -1;
     // an index outside the batch would mean a corrupt workspace: the lane
     // idles rather than read outside the caller's arrays
     const bool valid = (uint32_t)k < (uint32_t)b.n;
@@ -341,7 +347,7 @@ __global__ void __launch_bounds__(kLaneThreads, 4)
     Outcome o;
     qs.g = pr.q;
     if (PACKED)
-      o = lane_pair_p16<R, QSTAGE, TB>(pr, valid, sc, s_prof,
+      o = lane_pair_p16<R, QSTAGE, TB, LIVE>(pr, valid, sc, s_prof,
                                        *reinterpret_cast<Ring<true>*>(&ring), mparam & 0xFF, qs);
     else
       o = lane_pair_i32<R, GRING>(pr, valid, sc, s_prof, *reinterpret_cast<Ring<false>*>(&ring),
@@ -739,12 +745,32 @@ size_t lane_pipe_bytes(int cls, bool global_ring) {
   return (global_ring && !packed_class(cls)) ? (size_t)kLaneThreads * kPipeD * sizeof(int2) : 0;
 }
 
+// What packed one-lane launches look for (lane_pair_p16).  A gap from the seed dies
+// within a wide band, and the rows past the query's end are many there; in narrow
+// bands both looks find little, and their code costs the steps registers.  1M mixed
+// reads with 1% / with 14% errors, ms a call with none, the rows, rows and columns:
+//   w = 10    2.04 / 2.06    -              2.07 / 2.13
+//   w = 24    2.48 / 2.49    2.34 / 2.56    2.44 / 2.70
+//   w = 64    3.79 / 3.80    3.24 / 3.95    3.24 / 4.03
+//   w = 100   4.75 / 4.68    4.23 / 4.76    3.80 / 4.48
+// and with gaps that extend for 2, w = 50: 3.32 / 3.31, 3.20 / 3.37, 2.95 / 3.17; for
+// nothing, w = 100: 4.78 / 4.79 and 5.11 / 5.08.
+static int lane_live(const Score& sc) {
+  const int64_t reach = (int64_t)sc.beta * sc.w;
+  return reach < 24 ? 0 : (reach < 80 ? 1 : 2);
+}
+
 template <int R, bool PACKED, bool GRING, bool QSTAGE, int TB = 6>
 static cudaError_t launch_lane_t(const Batch* b, const Score& sc, const Work& w, const Launch& L,
                                  int head_id, void* gring, cudaStream_t stream) {
   const size_t smem = (GRING ? 0 : kLaneThreads * lane_ring_bytes(L.cls, L.rs_log2)) +
                       (QSTAGE ? lane_stage_bytes(L.j_hi) : 0) + lane_pipe_bytes(L.cls, GRING);
-  auto kern = k_lane<R, PACKED, GRING, QSTAGE, TB>;
+  auto kern = k_lane<R, PACKED, GRING, QSTAGE, TB, 0>;
+  if constexpr (PACKED) {
+    const int live = lane_live(sc);
+    if (live == 1) kern = k_lane<R, PACKED, GRING, QSTAGE, TB, 1>;
+    if (live == 2) kern = k_lane<R, PACKED, GRING, QSTAGE, TB, 2>;
+  }
   cudaError_t e = raise_smem_limit(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<L.grid, kLaneThreads, smem, stream>>>(b, sc, w, L.cls, L.j_lo, L.j_hi, head_id,

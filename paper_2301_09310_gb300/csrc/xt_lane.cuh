@@ -424,14 +424,16 @@ __device__ __forceinline__ void fold_keys(uint32_t (&K)[R], int32_t (&Blo)[R], i
 // match*min(qlen,tlen): (B + 1) << k <= 32767, (B + 1) * 2^TB - 1 <= 32767 (the row keys),
 // 1 <= qlen <= 65535 and tlen >= 1.
 //
-// A strip sweeps only the columns that can be alive in it: a cell (i, j) is
-// worth at most h0 + match (min(i, j) + 1) - gap_open - gap_extend |i - j|, so in
-// row i the columns from lo to hi below hold every live cell.
-// And once no path from a strip's bottom row can raise the end-to-end score, the
-// rows left matter only to the last live row, which the bounds of xt_bounds.cuh
-// give.  (Following the row's actual live cells costs more in every step than it
+// LIVE >= 1: once no path from a strip's bottom row can raise the end-to-end score,
+// the rows left matter only to the last live row, which the bounds of xt_bounds.cuh
+// give (that look reads a row's ring entries, so it is taken only where they do
+// give it: 1M reads with 14% errors 5.08 -> 4.84 ms a call).
+// LIVE == 2: a strip sweeps only the columns that can be alive in it: a cell (i, j)
+// is worth at most h0 + match (min(i, j) + 1) - gap_open - gap_extend |i - j|, so in
+// row i the columns from lo to hi below hold every live cell (gap_extend >= 1).
+// (Following the row's actual live cells costs more in every step than it
 // saves: 4M mixed reads 4.89 ms a call against 4.79, and 4.97 with neither.)
-template <int R, bool STAGED, int TB = 6>
+template <int R, bool STAGED, int TB, int LIVE>
 __device__ __forceinline__ Outcome lane_pair_p16(const Pair& pr, bool valid, const Score& sc,
                                                  const uint32_t* s_prof, const Ring<true>& ring,
                                                  int mshift, Query<STAGED> qs) {
@@ -455,29 +457,33 @@ __device__ __forceinline__ Outcome lane_pair_p16(const Pair& pr, bool valid, con
     int32_t lo = 1, hi = 0, rlast = 0;
     if (live) {
       rlast = min(tlen - 1, i0 + RR - 1);
-      // the row above the strip, which its first row reads, has no live column
-      // before lo (its diagonal, which needs no gap, aside); its last row none
-      // after hi
-      const int32_t dead = gopen + beta * (i0 - 1) - h0 - match;
-      lo = dead >= 0 ? min(dead / (match + beta) + 1, max(i0 - 1, 0)) : 0;
-      lo = max(lo, i0 - w);
+      lo = max(0, i0 - w);
       hi = min(qlen - 1, rlast + w);
-      if (beta > 0) hi = min(hi, rlast + max(h0 + match * (rlast + 1) - gopen - 1, 0) / beta);
+      if (LIVE == 2) {
+        // the row above the strip, which its first row reads, has no live column
+        // before lo (its diagonal, which needs no gap, aside); its last row none
+        // after hi
+        const int32_t dead = gopen + beta * (i0 - 1) - h0 - match;
+        if (dead >= 0) lo = max(lo, min(dead / (match + beta) + 1, max(i0 - 1, 0)));
+        hi = min(hi, rlast + max(h0 + match * (rlast + 1) - gopen - 1, 0) / beta);
+      }
       if (i0 >= tlen || lo > hi) live = false;
     }
     if (!__any_sync(0xffffffffu, live)) break;
-    // The lanes sweep the same columns, as far as each pair has them: a column's
-    // ring entries and codes are one line, and no lane ends in masked steps
-    // before the others.
-    const int32_t lo_warp = (int32_t)__reduce_min_sync(0xffffffffu, live ? (uint32_t)lo : 0x7FFFFFFFu);
-    const int32_t hi_warp = (int32_t)__reduce_max_sync(0xffffffffu, live ? (uint32_t)hi : 0u);
-    if (live) {
-      lo = lo_warp;
-      hi = min(hi_warp, min(qlen - 1, rlast + w));
+    if (LIVE == 2) {
+      // The lanes sweep the same columns, as far as each pair has them: a column's
+      // ring entries and codes are one line, and no lane ends in masked steps
+      // before the others.
+      const int32_t lo_warp = (int32_t)__reduce_min_sync(0xffffffffu, live ? (uint32_t)lo : 0x7FFFFFFFu);
+      const int32_t hi_warp = (int32_t)__reduce_max_sync(0xffffffffu, live ? (uint32_t)hi : 0u);
+      if (live) {
+        lo = lo_warp;
+        hi = min(hi_warp, min(qlen - 1, rlast + w));
+        // columns the row above did not reach are dead
+        if (i0 > 0)
+          for (; hi_prev < hi; ++hi_prev) ring.at(hi_prev + 1) = 0u;
+      }
     }
-    // columns the row above did not reach are dead
-    if (live && i0 > 0)
-      for (; hi_prev < hi; ++hi_prev) ring.at(hi_prev + 1) = 0u;
     uint32_t Hl[R], HAl[R], El[R], K[R], sel[R];
     int32_t Blo[R], Bhi[R];
 #pragma unroll
@@ -667,17 +673,17 @@ __device__ __forceinline__ Outcome lane_pair_p16(const Pair& pr, bool valid, con
       const int32_t edge = col_m1(rlast, h0, sc);
       if (st.stop || (last_m == 0 && edge == 0)) live = false;
       // past the query's end: the most a path from the bottom row can reach
-      if (live && rlast >= qlen - 1 && rlast + 1 < tlen && st.gscore > 0) {
-        int32_t z = edge > 0 ? edge + match : INT32_MIN / 2;
-#pragma unroll 4
-        for (int32_t c = lo; c <= hi; ++c) {
-          const int32_t h = lo16(ring.at(c));
-          z = max(z, h > 0 ? h - match * c : z);
-        }
-        if (z + match * (qlen - 1) <= st.gscore) {
-          const NearEnd n = {st.best, st.bi - st.bj, st.gscore, st.gtle - 1};
-          const int32_t last = near_last_row(n, qlen, tlen, h0, match, sc);
-          if (last >= 0) {
+      if (LIVE && live && rlast >= qlen - 1 && rlast + 1 < tlen && st.gscore > 0) {
+        const NearEnd n = {st.best, st.bi - st.bj, st.gscore, st.gtle - 1};
+        const int32_t last = near_last_row(n, qlen, tlen, h0, match, sc);
+        if (last >= 0) {
+          int32_t z = edge > 0 ? edge + match : INT32_MIN / 2;
+#pragma unroll 1
+          for (int32_t c = lo; c <= hi; ++c) {
+            const int32_t h = lo16(ring.at(c));
+            z = max(z, h > 0 ? h - match * c : z);
+          }
+          if (z + match * (qlen - 1) <= st.gscore) {
             st.last_live = last;
             live = false;
           }
