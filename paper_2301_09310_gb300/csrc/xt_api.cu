@@ -1,6 +1,7 @@
 // xt_api.cu -- the C ABI of include/xt.h: context, argument checks, device
 // workspace, launch plan and the host-buffer (end-to-end) variant.
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -147,7 +148,8 @@ xt_status get_work(xt_ctx* ctx, int32_t n, Work* w, Batch** desc) {
   const size_t o_counts = off; off = align_up(off + 4 * (size_t)kNumBuckets);
   const size_t o_cursor = off; off = align_up(off + 4 * (size_t)kNumBuckets);
   const size_t o_sb = off; off = align_up(off + 4 * (size_t)(kNumClasses * kNumJ));
-  const size_t o_se = off; off = align_up(off + 4 * (size_t)(kNumClasses * kNumJ));
+  const size_t o_se = off; off += 4 * (size_t)(kNumClasses * kNumJ);
+  const size_t o_hope = off; off = align_up(off + 4);  // read back with the bucket counts
   const size_t o_heads = off; off = align_up(off + 4 * (size_t)kMaxLaunches);
   const size_t o_left = off; off = align_up(off + 4 * (size_t)(kNearBins + kBandLeft));
   const size_t o_tmp = off; off = align_up(off + 4 * (size_t)n);
@@ -163,6 +165,7 @@ xt_status get_work(xt_ctx* ctx, int32_t n, Work* w, Batch** desc) {
   w->cursor = (int32_t*)(base + o_cursor);
   w->seg_begin = (int32_t*)(base + o_sb);
   w->seg_end = (int32_t*)(base + o_se);
+  w->near_hope = (int32_t*)(base + o_hope);
   w->heads = (int32_t*)(base + o_heads);
   w->near_left = (int32_t*)(base + o_left);
   w->band_left = w->near_left + kNearBins;
@@ -369,7 +372,18 @@ void plan_batched(xt_ctx* ctx, const Score& sc, Plan* pl, bool allow_gring = tru
 // call hide that time, and the pass saves work beside them (6,000 streamed pairs
 // 819 and 901 us).
 constexpr int32_t kNearPassMin = 8192;
-constexpr int kNearLeft = 3;             // one NEAR pair in so many is left for the engines
+constexpr int kNearLeft = 3;             // what it leaves is planned as one NEAR pair in so many
+// How much of the engines' work the pass has to save to be run.
+constexpr double kNearSaves = 0.1;
+// The share of the NEAR pairs k_near is expected to leave, from the share hope of
+// them whose diagonal lost so little until k_diag gave it up that at that rate the
+// whole query would stay within k_near's bound.  Over reads of 64-400 bases with
+// 0.3-14% errors (hope: left): 0.01: 1.0, 0.05: 0.98, 0.14: 0.90, 0.20: 0.79, 0.26:
+// 0.71, 0.37: 0.54, 0.45: 0.36-0.42, 0.50: 0.28-0.37, 0.57: 0.19-0.25, 0.67: 0.08.
+inline double near_left_est(int32_t hopeful, int32_t near) {
+  const double s = near > 0 ? (double)hopeful / near : 0.0;
+  return std::min(1.0, std::max(0.0, 1.0 - 0.9 * s * (1.0 + s)));
+}
 constexpr int32_t kBucketSmall = XT_SMALL_BUCKET;  // fewer pairs: a bucket cannot fill the GPU
 constexpr int32_t kLaneSlots = 77824;    // one-lane thread slots of a full GPU (152 x 4 x 128)
 // Built-in rule: the fewest pairs of a bucket for one lane per pair.  A pair's
@@ -455,30 +469,9 @@ Launch queue_launch(const xt_ctx* ctx, int cls, int j, int P, int R, int lg) {
 // empty buckets get no launch; a bucket too small to fill the GPU takes its
 // small-batch schedule, or by default a group schedule with enough lanes per
 // pair to fill it; larger buckets take the throughput schedule.
-void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFlags& jf,
-                 const bool* lane_ok, Plan* pl) {
+void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t hopeful,
+                 const JFlags& jf, const bool* lane_ok, Plan* pl) {
   pl->jf = jf;
-  // the NEAR class is planned for the pairs k_near is expected to leave, or for
-  // all of them where it does not run
-  int32_t near = 0, longer = 0;
-  for (int j = 0; j < kNumJ; ++j) near += cnt[CLS_NEAR][j];
-  for (int cls = CLS_PACKED; cls < kNumClasses; ++cls)
-    for (int j = kNearJMax + 1; j < kNumJ; ++j) longer += cnt[cls][j];
-  if (near >= kNearPassMin || (near > 0 && longer > 0)) {
-    pl->near_pairs = near;
-    for (int j = 0; j < kNumJ; ++j) cnt[CLS_NEAR][j] = (cnt[CLS_NEAR][j] + kNearLeft - 1) / kNearLeft;
-  }
-  pl->near_grid = near_grid(pl->near_pairs, ctx->num_sms);
-  const bool saved = ctx->plan_small;
-  // the call's estimated cells: each bucket's pairs at a query length three
-  // quarters of the way up the bucket
-  double est_cells = 0.0;
-  for (int cls = CLS_PACKED; cls < kNumClasses; ++cls)
-    for (int j = 0; j < kNumJ; ++j)
-      if (cnt[cls][j]) {
-        const int jj = j < kJMin ? kJMin : j;
-        est_cells += (double)cnt[cls][j] * band_cells_est(0.75 * pair_cells_q(jj), sc.w);
-      }
   // the band engine, where it holds the band
   int bP = 0, bK = 0;
   const bool band_ok = ctx->near_first && !ctx->forced_P && band_shape(sc, ctx->match, 0, &bP, &bK);
@@ -500,6 +493,50 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
     if (jj < kBandLanesJ || !band_ok) return lane_min_pairs(jj);
     return (int32_t)std::max<int64_t>(kBucketSmall, 2 * (int64_t)kBucketSmall * 201 / (2 * sc.w + 1));
   };
+  // Whether k_near runs.  It has to save a tenth of the short pairs' work (1M reads of
+  // mixed lengths, a call with and without it: 14% errors 4.81 / 4.46 ms, unrelated
+  // 2.07 / 1.81, 4% 3.48 / 3.70, 1% 1.55 / 2.00).  While the call's short pairs are
+  // within one wave of lanes an engine's time is a pair's: the pass has to leave next
+  // to nothing, or take a bucket from lanes to a sooner engine, and its longest bucket
+  // must not stay on lanes (55k reads, mixed with 2% errors 593 / 468 us, of 100 bases
+  // with 2% 591 / 504, of 250 bases with 1% 733 / 1,372).
+  int32_t near = 0, longer = 0, rest = 0;
+  for (int j = 0; j < kNumJ; ++j) {
+    near += cnt[CLS_NEAR][j];
+    if (j <= kNearJMax) rest += cnt[CLS_PACKED][j];
+  }
+  bool lanes_after = false, sooner = false;
+  for (int j = 0; j < kNumJ; ++j) {
+    const int32_t c = cnt[CLS_NEAR][j], m = min_pairs(j);
+    if (c > near / 8) lanes_after = c / kNearLeft >= m;  // the longest of a good size decides
+    if (c >= m && c / kNearLeft < m) sooner = true;
+  }
+  for (int cls = CLS_PACKED; cls < kNumClasses; ++cls)
+    for (int j = kNearJMax + 1; j < kNumJ; ++j) longer += cnt[cls][j];
+  const double left = near_left_est(hopeful, near);
+  bool pass = (near >= kNearPassMin || (near > 0 && longer > 0)) &&
+              near * (1.0 - left) >= kNearSaves * ((double)near + rest);
+  if (longer == 0 && (int64_t)near + rest <= kLaneSlots && (lanes_after || (!sooner && left > 0.34)))
+    pass = false;
+  // what it leaves: the engines are chosen for one pair in kNearLeft (the rules above
+  // were measured so), their CTAs for as many as expected
+  double near_ctas = 1.0;
+  if (pass) {
+    pl->near_pairs = near;
+    near_ctas = std::max(1.0, kNearLeft * left);
+    for (int j = 0; j < kNumJ; ++j) cnt[CLS_NEAR][j] = (cnt[CLS_NEAR][j] + kNearLeft - 1) / kNearLeft;
+  }
+  pl->near_grid = near_grid(pl->near_pairs, ctx->num_sms);
+  const bool saved = ctx->plan_small;
+  // the call's estimated cells: each bucket's pairs at a query length three
+  // quarters of the way up the bucket
+  double est_cells = 0.0;
+  for (int cls = CLS_PACKED; cls < kNumClasses; ++cls)
+    for (int j = 0; j < kNumJ; ++j)
+      if (cnt[cls][j]) {
+        const int jj = j < kJMin ? kJMin : j;
+        est_cells += (double)cnt[cls][j] * band_cells_est(0.75 * pair_cells_q(jj), sc.w);
+      }
   // pairs of each launch
   int32_t pairs_of[kMaxLaunches] = {};
   for (int cls : {CLS_PACKED, CLS_NARROW, CLS_WIDE, CLS_NEAR, CLS_BAND}) {
@@ -648,11 +685,12 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], const JFla
   // calls of like size share a graph)
   for (int i = 0; i < pl->n_launch; ++i) {
     Launch& L = pl->launch[i];
+    const int64_t pairs = L.cls == CLS_NEAR ? (int64_t)std::ceil(near_ctas * pairs_of[i]) : pairs_of[i];
     if (L.band) {
-      L.grid = band_grid(L.P, L.R, pairs_of[i], ctx->num_sms);
+      L.grid = band_grid(L.P, L.R, (int32_t)pairs, ctx->num_sms);
     } else if (!L.lane) {
       const int64_t per_cta = kQueueThreads / L.P;
-      L.grid = (int)std::min<int64_t>(L.grid, next_pow2((pairs_of[i] + per_cta - 1) / per_cta));
+      L.grid = (int)std::min<int64_t>(L.grid, next_pow2((pairs + per_cta - 1) / per_cta));
     }
   }
   // the NEAR class, which waits for k_near, after the others; within each,
@@ -942,13 +980,14 @@ xt_status run_begin(xt_ctx* ctx, bool plain, bool early, const uint8_t* q_seq, i
     batched_flags(ctx, pc.sc, n, &pc.jf, pc.lane_ok);
     // a forced schedule puts every pair on that schedule's engine.  The
     // diagonal bounds need a gap to cost something; the narrow band must lie
-    // inside the call's, and its padded columns need alpha < 128
+    // inside the call's, its padded columns need alpha < 128, and it admits no
+    // more loss than the diagonal where gaps extend for nothing
     const bool diag = pc.diag = ctx->near_first && !early && n >= kNearMinPairs && !ctx->forced_P &&
                       pc.sc.alpha >= 1;
-    const bool near = diag && pc.sc.alpha <= 127 && pc.sc.w >= kNearHalf;
+    const bool near = diag && pc.sc.alpha <= 127 && pc.sc.beta >= 1 && pc.sc.w >= kNearHalf;
     e = enqueue_front(pc.jf, pc.sc, scr->match, diag, near, pc.w, pc.desc, pc.n_cap, stream);
     const size_t seg_bytes =
-        (size_t)((const char*)(pc.w.seg_end + kNumClasses * kNumJ) - (const char*)pc.w.seg_begin);
+        (size_t)((const char*)(pc.w.near_hope + 1) - (const char*)pc.w.seg_begin);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(ctx->seg_host, pc.w.seg_begin, seg_bytes, cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaEventRecord(ctx->seg_ev, stream);
@@ -984,7 +1023,7 @@ xt_status run_finish(xt_ctx* ctx) {
     int32_t cnt[kNumClasses][kNumJ];
     for (int c = 0; c < kNumClasses; ++c)
       for (int j = 0; j < kNumJ; ++j) cnt[c][j] = se[c * kNumJ + j] - sb[c * kNumJ + j];
-    plan_counts(ctx, sc, cnt, pc.jf, pc.lane_ok, &pl);
+    plan_counts(ctx, sc, cnt, se[kNumClasses * kNumJ], pc.jf, pc.lane_ok, &pl);
     if (pl.bad) return fail(ctx, XT_ECUDA, "internal: inconsistent bucket plan");
   }
   const size_t want = layout_pool(ctx, &pl);
@@ -1755,7 +1794,8 @@ bool carve_static(void* base_ptr, int32_t n, Work* w, Batch** desc) {
   w->seg_begin = (int32_t*)(base + o_sb);
   w->seg_end = (int32_t*)(base + o_se);
   w->heads = (int32_t*)(base + o_heads);
-  w->near_left = nullptr;  // no near pass on this path
+  w->near_hope = nullptr;  // no near pass on this path
+  w->near_left = nullptr;
   w->band_left = nullptr;
   w->near_tmp = nullptr;
   *desc = (Batch*)(base + o_desc);

@@ -77,6 +77,7 @@ struct Work {
   int32_t* cursor;      // [kNumBuckets]
   int32_t* seg_begin;   // [kNumClasses * kNumJ]
   int32_t* seg_end;     // [kNumClasses * kNumJ]
+  int32_t* near_hope;   // [1] NEAR pairs whose diagonal promises that k_near settles them
   int32_t* heads;       // [kMaxLaunches]
   int32_t* near_left;   // [kNearBins] pairs k_near left, per exact length
   int32_t* band_left;   // [kBandLeft] pairs a narrow band launch left, per bucket

@@ -678,7 +678,7 @@ __device__ __forceinline__ Outcome lane_pair_p16(const Pair& pr, bool valid, con
         const int32_t last = near_last_row(n, qlen, tlen, h0, match, sc);
         if (last >= 0) {
           int32_t z = edge > 0 ? edge + match : INT32_MIN / 2;
-#pragma unroll 1
+#pragma unroll 4
           for (int32_t c = lo; c <= hi; ++c) {
             const int32_t h = lo16(ring.at(c));
             z = max(z, h > 0 ? h - match * c : z);

@@ -17,12 +17,13 @@ constexpr int kDiagThreads = 256;
 // where they come to a total loss D (matches not made) below o + e; n and
 // *bi receive the ends.  The diagonal of a row that holds no match is worth
 // at least 1 throughout, or the pair fails (a dead diagonal may be revived
-// from outside).
+// from outside).  *hope: it failed while losing no faster than would come to
+// k_near's bound at the query's end.
 __device__ __forceinline__ bool diag_scan(const Batch& b, const Pair& pr, const Score& sc,
-                                          int32_t match, NearEnd* n, int32_t* bi) {
+                                          int32_t match, NearEnd* n, int32_t* bi, bool* hope) {
   const int32_t loss_x = match - (int32_t)(int8_t)((sc.prof[0] >> 8) & 0xFF);
   const int32_t loss_n = match - (int32_t)(int8_t)(sc.nnnn & 0xFF);
-  const int32_t limit = sc.alpha - 1;
+  const int32_t limit = sc.alpha - 1, bound = sc.alpha + sc.beta * kNearHalf;
   ByteStream qs, ts;
   const uint8_t *qe = b.q_seq + b.q_bytes, *te = b.t_seq + b.t_bytes;
   qs.init(b.q_seq, qe, pr.q);
@@ -43,7 +44,10 @@ __device__ __forceinline__ bool diag_scan(const Batch& b, const Pair& pr, const 
       g += match - loss;
       lost += loss;
       pos = idx + 1;
-      if (lost > limit || g <= 0) return false;
+      if (lost > limit || g <= 0) {
+        *hope = g > 0 && (int64_t)lost * pr.qlen < (int64_t)bound * pos;
+        return false;
+      }
       bad &= bad - 1;
     }
   }
@@ -66,14 +70,14 @@ __device__ __forceinline__ bool diag_scan(const Batch& b, const Pair& pr, const 
 // 0.45 ms, about 2 TB/s of the sequences' diagonals and the metadata.
 __global__ void __launch_bounds__(kDiagThreads)
     k_diag(const Batch* __restrict__ bd, Score sc, int32_t match, bool near,
-           uint8_t* __restrict__ pclass) {
+           uint8_t* __restrict__ pclass, int32_t* __restrict__ hopeful) {
   __shared__ int32_t s_out[kDiagThreads * 7];
   __shared__ uint8_t s_done[kDiagThreads];
   const Batch b = *bd;
   const int64_t base = (int64_t)blockIdx.x * kDiagThreads;
   if (base >= b.n) return;
   const int64_t kk = base + threadIdx.x;
-  bool done = false;
+  bool done = false, hope = false;
   if (kk < b.n) {
     const int32_t k = (int32_t)kk;
     const int64_t qo = b.q_off[k], to = b.t_off[k];
@@ -89,7 +93,7 @@ __global__ void __launch_bounds__(kDiagThreads)
       pr.t = b.t_seq + to;
       NearEnd n;
       int32_t bi = -1, last = -1;
-      if (diag_scan(b, pr, sc, match, &n, &bi))
+      if (diag_scan(b, pr, sc, match, &n, &bi, &hope))
         last = near_last_row(n, pr.qlen, pr.tlen, pr.h0, match, sc);
       if (last >= 0) {
         done = true;
@@ -110,9 +114,11 @@ __global__ void __launch_bounds__(kDiagThreads)
       reach = sc.beta * rows <= pr.h0 + (int64_t)match * pr.qlen - 2 * o - 1;
     }
     pclass[k] = done ? (uint8_t)CLS_DONE : (reach && near ? (uint8_t)CLS_NEAR : kRest);
+    hope = hope && reach && pr.h0 + match * pr.qlen <= 511;  // (and of the packed class, about)
   }
   s_done[threadIdx.x] = done;
-  __syncthreads();
+  const int hopes = __syncthreads_count(hope);
+  if (threadIdx.x == 0 && near && hopes > 0) atomicAdd(hopeful, hopes);
   int32_t* out = reinterpret_cast<int32_t*>(b.out + base);
 #pragma unroll
   for (int u = 0; u < 7; ++u) {
@@ -397,7 +403,7 @@ cudaError_t launch_diag(const Batch* bd, int32_t n_cap, const Score& sc, int32_t
                         const Work& w, cudaStream_t stream) {
   if (n_cap == 0) return cudaSuccess;
   const int grid = (int)(((int64_t)n_cap + kDiagThreads - 1) / kDiagThreads);
-  k_diag<<<grid, kDiagThreads, 0, stream>>>(bd, sc, match, near, w.pclass);
+  k_diag<<<grid, kDiagThreads, 0, stream>>>(bd, sc, match, near, w.pclass, w.near_hope);
   return cudaGetLastError();
 }
 

@@ -66,7 +66,10 @@ static_assert(kNumBuckets % 4 == 0 && kNearBins % 4 == 0 && kMaxLaunches % 4 == 
 
 __global__ void __launch_bounds__(kDescThreads) k_store_desc(Batch* dst, Batch b, Work w) {
   const int4 z = make_int4(0, 0, 0, 0);
-  if (threadIdx.x == 0) *dst = b;
+  if (threadIdx.x == 0) {
+    *dst = b;
+    if (w.near_hope) *w.near_hope = 0;
+  }
   if (w.counts)
     for (int i = threadIdx.x; i < kNumBuckets / 4; i += kDescThreads)
       reinterpret_cast<int4*>(w.counts)[i] = z;

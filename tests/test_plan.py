@@ -1,0 +1,74 @@
+"""The launch plan of a batched call, from pair counts alone (the planner is host
+code: no GPU needed)."""
+import json
+import os
+import subprocess
+
+import pytest
+
+from paper_2301_09310_gb300 import build
+from paper_2301_09310_gb300.synth import ScoringParams
+
+PACKED, NARROW, WIDE, HUGE, NEAR, BAND = range(6)
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    lib = build.build()
+    exe = str(tmp_path_factory.mktemp("plan") / "plan_probe")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "plan_probe.cu")
+    subprocess.run([build.nvcc(), *build.ARCH_FLAGS, "-O1", "-std=c++17", f"-I{build.INCLUDE}",
+                    f"-I{build.CSRC}", src, "-o", exe, lib, "-Xlinker", "-rpath", "-Xlinker",
+                    os.path.dirname(lib)], check=True, capture_output=True)
+
+    def run(cases):
+        text = []
+        for c in cases:
+            sc, counts, tuned = c.get("sc", ScoringParams()), c["counts"], c.get("tuned", ())
+            n = c.get("n", sum(counts.values()))
+            text.append(f"{sc.w} {sc.match} {sc.mismatch} {sc.gap_open} {sc.gap_extend} {sc.zdrop} "
+                        f"{sc.n_score} {n} {c.get('hopeful', 0)} {c.get('budget', 0)} {len(tuned)} "
+                        f"{len(counts)}")
+            text += [" ".join(map(str, t)) for t in tuned]
+            text += [f"{cls} {j} {v}" for (cls, j), v in counts.items()]
+        r = subprocess.run([exe], input="\n".join(text) + "\n", capture_output=True, text=True, check=True)
+        out = [json.loads(line) for line in r.stdout.splitlines()]
+        assert len(out) == len(cases)
+        return out
+
+    return run
+
+
+def reads(n, share_near, hope, long_share=0.4):
+    """n pairs of up to 254 bases the diagonal pass left, so many of them near pairs."""
+    near, rest = int(n * share_near), int(n * (1 - share_near))
+    return {"counts": {(NEAR, 8): int(near * long_share), (NEAR, 7): near - int(near * long_share),
+                       (PACKED, 7): rest // 2, (PACKED, 6): rest - rest // 2},
+            "hopeful": int(near * hope), "n": n}
+
+
+@pytest.mark.parametrize("n", [30_000, 130_000, 900_000])
+def test_near_pass_only_where_reads_promise_it(plan, n):
+    none, noisy, good = plan([reads(n, 0.5, 0.0), reads(n, 0.5, 0.05), reads(n, 0.7, 0.57)])
+    assert none["near_pairs"] == 0 and noisy["near_pairs"] == 0
+    assert good["near_pairs"] == int(n * 0.7)
+
+
+def test_near_pass_not_before_lanes_within_one_wave(plan):
+    # one length bucket, a single wave of lanes: the pass would only delay them ...
+    lanes, sooner, waves = plan([
+        {"counts": {(NEAR, 7): 37_000}, "hopeful": 20_000, "n": 55_000},
+        # ... unless what it leaves goes to a sooner engine, or there are more waves
+        {"counts": {(NEAR, 8): 45_000}, "hopeful": 21_400, "n": 55_000},
+        {"counts": {(NEAR, 7): 200_000}, "hopeful": 110_000, "n": 300_000}])
+    assert lanes["near_pairs"] == 0
+    assert sooner["near_pairs"] == 45_000 and sooner["launches"][0]["engine"] == "band"
+    assert waves["near_pairs"] == 200_000
+
+
+def test_ctas_for_the_pairs_the_near_pass_leaves(plan):
+    few, many = plan([reads(200_000, 0.7, 0.6), reads(200_000, 0.7, 0.25)])
+    for a, b in zip(few["launches"], many["launches"]):
+        assert a["engine"] == b["engine"]
+        if a["engine"] == "band":
+            assert b["grid"] > 1.3 * a["grid"]
