@@ -751,13 +751,16 @@ size_t lane_pipe_bytes(int cls, bool global_ring) {
 // reads with 1% / with 14% errors, ms a call with none, the rows, rows and columns:
 //   w = 10    2.04 / 2.06    -              2.07 / 2.13
 //   w = 24    2.48 / 2.49    2.34 / 2.56    2.44 / 2.70
+//   w = 50    3.35 / 3.37    2.90 / 3.48    2.97 / 3.61
 //   w = 64    3.79 / 3.80    3.24 / 3.95    3.24 / 4.03
 //   w = 100   4.75 / 4.68    4.23 / 4.76    3.80 / 4.48
+// (what the near pass leaves of 300k such reads, w = 70: 726, 679 us a call with the
+// rows, with both; of 766k sides of seeds, w = 61: 1,504, 1,400)
 // and with gaps that extend for 2, w = 50: 3.32 / 3.31, 3.20 / 3.37, 2.95 / 3.17; for
 // nothing, w = 100: 4.78 / 4.79 and 5.11 / 5.08.
 static int lane_live(const Score& sc) {
   const int64_t reach = (int64_t)sc.beta * sc.w;
-  return reach < 24 ? 0 : (reach < 80 ? 1 : 2);
+  return reach < 24 ? 0 : (reach < 48 ? 1 : 2);
 }
 
 template <int R, bool PACKED, bool GRING, bool QSTAGE, int TB = 6>
