@@ -550,7 +550,7 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
       bool lane = false, band = false;
       if (cls == CLS_BAND && !band_ok) {
         // a narrow band first, then the group engine for the pairs it leaves
-        if (pl->n_launch >= kMaxLaunches - 3 ||
+        if (pl->n_launch >= kMaxLaunches - 3 ||  // (kept by kMaxLaunches' bound)
             !band_near_shape(sc, ctx->match, jj, &L.P, &L.R, &L.near_hw)) {
           pl->bad = true;
           continue;

@@ -67,7 +67,18 @@ static_assert(kNearJMax <= kExactJ, "one bin per length");
 constexpr int kNearBins = 1 << kNearJMax;
 constexpr int kBandLeft = (kNumJ + 3) / 4 * 4;
 constexpr int kQueueThreads = 128;       // threads per CTA of the queue kernels
-constexpr int kMaxLaunches = 64;         // queue-kernel launches per call (heads)
+// Queue-kernel launches per call (heads), at most one a bucket and class: WIDE pairs
+// in every bucket, PACKED and NARROW ones up to 65,535 bases, NEAR ones up to
+// kNearMaxQ, BAND ones up to 65,535 bases (where a narrow band comes first, at 511
+// and longer, up to three launches each), HUGE ones and the near pass one each.
+constexpr int kShortJMax = 17;           // bucket of 65,535-base queries
+constexpr int kBandLaunches = 3;
+constexpr int kMaxLaunches = 80;
+static_assert((kJMax - kJMin + 1) + 2 * (kShortJMax - kJMin + 1) + (kNearJMax - kJMin + 1) +
+                      (kShortJMax - kJMin + 1 > kBandLaunches * (kShortJMax - kBandNearJMin + 1)
+                           ? kShortJMax - kJMin + 1
+                           : kBandLaunches * (kShortJMax - kBandNearJMin + 1)) + 2 <= kMaxLaunches,
+              "a head for every launch");
 
 // Device workspace of one call (carved from the context's pool).
 struct Work {

@@ -72,3 +72,48 @@ def test_ctas_for_the_pairs_the_near_pass_leaves(plan):
         assert a["engine"] == b["engine"]
         if a["engine"] == "band":
             assert b["grid"] > 1.3 * a["grid"]
+
+
+def full_plan(rng, flags, j_top):
+    """Counts in every class and bucket that classify could fill, of sizes that keep
+    neighbouring buckets' launches apart."""
+    counts = {}
+    for j in range(5, j_top + 1):
+        f = flags[j]
+        classes = [WIDE] if not f & 4 and not f & 1 else [HUGE]
+        if j <= 17 and not f & 1:
+            classes.append(NARROW)
+            if f & 2:
+                classes += [PACKED] + ([NEAR] if j <= 9 else [])
+        if j <= 17 and f & 16:
+            classes.append(BAND)
+        for cls in classes:
+            if rng.random() < 0.97:
+                counts[cls, j] = rng.choice([1, 50, 3000, 8191, 8192, 9000, 40_000, 100_000])
+    return counts
+
+
+def test_every_class_and_bucket_gets_its_launch(plan):
+    import random
+    rng = random.Random(3)
+    scs = [ScoringParams(w=w) for w in (5, 20, 60, 100, 300, 511, 512, 700, 1000, 1900, 4000)]
+    schedules = [(1, 4), (1, 8), (1, 16), (2, 8), (4, 4), (8, 8), (16, 4), (32, 8), (32, 4)]
+    shapes = []
+    for k in range(800):
+        tuned = []
+        if k % 3 == 0:
+            tuned = [(j, s, *rng.choice(schedules)) for j in range(5, 22) for s in (0, 1)
+                     if rng.random() < 0.5 and j <= 9]
+        shapes.append({"sc": rng.choice(scs), "counts": {(WIDE, 5): 1}, "n": rng.choice([50_000, 1 << 20]),
+                       "tuned": tuned})
+    flags = [p["flags"] for p in plan(shapes)]
+    for c, f in zip(shapes, flags):
+        c["counts"] = full_plan(rng, f, 21)
+        c["hopeful"] = rng.choice([0, 60_000])
+    plans = plan(shapes)
+    assert not any(p["bad"] for p in plans)
+    for c, p in zip(shapes, plans):  # every non-empty (class, bucket) is drained once
+        for (cls, j), v in c["counts"].items():
+            runs = [L for L in p["launches"] if not L["near_hw"]
+                    and (L["cls"] == cls or L["cls2"] == cls) and L["j_lo"] <= j <= L["j_hi"]]
+            assert len(runs) == 1, (c["sc"], cls, j, runs)
