@@ -151,7 +151,7 @@ xt_status get_work(xt_ctx* ctx, int32_t n, Work* w, Batch** desc) {
   const size_t o_se = off; off += 4 * (size_t)(kNumClasses * kNumJ);
   const size_t o_hope = off; off = align_up(off + 4);  // read back with the bucket counts
   const size_t o_heads = off; off = align_up(off + 4 * (size_t)kMaxLaunches);
-  const size_t o_left = off; off = align_up(off + 4 * (size_t)(kNearBins + kBandLeft));
+  const size_t o_left = off; off = align_up(off + 4 * (size_t)kNearBins);
   const size_t o_tmp = off; off = align_up(off + 4 * (size_t)n);
   void* old = ctx->work;
   xt_status s = dev_alloc(ctx, &ctx->work, &ctx->work_bytes, off);
@@ -168,7 +168,6 @@ xt_status get_work(xt_ctx* ctx, int32_t n, Work* w, Batch** desc) {
   w->near_hope = (int32_t*)(base + o_hope);
   w->heads = (int32_t*)(base + o_heads);
   w->near_left = (int32_t*)(base + o_left);
-  w->band_left = w->near_left + kNearBins;
   w->near_tmp = (int32_t*)(base + o_tmp);
   return XT_OK;
 }
@@ -183,7 +182,7 @@ struct Plan {
   bool pool_serial = true;  // global-ring launches share one pool region, in order
   int32_t near_pairs = 0;   // pairs of the NEAR class (k_near runs when there are any)
   int near_grid = 0;
-  int band_near = 0;        // narrow band launches (each gathers the pairs it left)
+  int band_near = 0;        // narrow band launches (each packs the pairs it left)
 };
 
 int64_t next_pow2(int64_t x) { return (int64_t)1 << log2_ceil(x); }
@@ -406,7 +405,9 @@ inline double band_cells_est(double q, int w) {
 // (band geometry only), kJPacked where a one-lane schedule is possible for
 // the bucket in either size class, kJTag4 on such buckets of 511-base queries
 // and longer in calls of n >= kTag4MinPairs pairs.  lane_ok[j]: that one-lane
-// launch exists.
+// launch exists.  The whole band in registers is faster than packed lanes with 4-bit
+// tags, a narrow band first is not where the reads differ (1M pairs of the stream,
+// w = 600: 74.3 ms a call so, 61.8 on lanes).
 void batched_flags(xt_ctx* ctx, const Score& sc, int32_t n, JFlags* jf, bool* lane_ok) {
   *jf = JFlags{};
   for (int j = 0; j < kNumJ; ++j) lane_ok[j] = false;
@@ -436,7 +437,7 @@ void batched_flags(xt_ctx* ctx, const Score& sc, int32_t n, JFlags* jf, bool* la
     if (banded) jf->f[j] |= kJBand;
     if (lane_ok[j])
       jf->f[j] |= kJPacked |
-                  (packed_tag_bits(j) == 4 && n >= kTag4MinPairs && !banded ? kJTag4 : 0);
+                  (packed_tag_bits(j) == 4 && n >= kTag4MinPairs && !(banded && band) ? kJTag4 : 0);
     // the default rule's answer (tuned group schedules always fit, see
     // bucket_sched_ok, but a bucket's class must not depend on its count)
     const int fP = ctx->forced_P;
@@ -479,9 +480,9 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
   // the long buckets of one call run side by side, so when together they
   // hold two full waves of lanes each of them takes the one-lane engine
   int64_t long_pairs = 0;
-  for (int cls = CLS_PACKED; cls <= CLS_NARROW; ++cls)
+  for (int cls : {CLS_PACKED, CLS_NARROW, CLS_BAND})
     for (int j = kLongJ; j < kNumJ; ++j)
-      if (lane_ok[j]) long_pairs += cnt[cls][j];
+      if (lane_ok[j] && !(cls == CLS_BAND && band_ok)) long_pairs += cnt[cls][j];
   const bool long_lanes = long_pairs >= 2 * (int64_t)kLaneSlots;
   // Where the band engine is the alternative, 126-base queries and longer need
   // more pairs before one lane each is faster, the fewer the narrower the band:
@@ -537,6 +538,37 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
         const int jj = j < kJMin ? kJMin : j;
         est_cells += (double)cnt[cls][j] * band_cells_est(0.75 * pair_cells_q(jj), sc.w);
       }
+  // The group engine's schedule for c pairs of a bucket; true where only global slabs
+  // hold the band.
+  auto group_schedule = [&](int cls, int jj, int32_t c, int* P, int* R, int* lg) {
+    *P = 0; *R = 8; *lg = 0;
+    bool huge = false;
+    const BucketSched* t = ctx->forced_P ? nullptr : tuned(ctx, sc.w, jj);
+    if (!ctx->forced_P && !t && c < min_pairs(jj) && cls != CLS_WIDE) {
+      // enough lanes per pair that the bucket's longest pair takes no
+      // longer than the call's whole work spread over the GPU's one-lane
+      // slots (the call's buckets run side by side, so a small bucket
+      // need not fill the GPU on its own; fewer lanes per pair waste less
+      // of each chunk on the wavefront's fill), where the ring fits
+      const double need = band_cells_est(pair_cells_q(jj), sc.w) * (double)kLaneSlots /
+                          std::max(est_cells, 1.0);
+      int want = 4;  // two-lane groups measured slower than four on every call size
+      while (want < 32 && want < need) want *= 2;
+      // short queries: 8 rows a lane for as many rows as the bucket's longest
+      // query has, one chunk of them (32 lanes idle half: 5,000 pairs of 64 bases
+      // 109 us a call, 94 so)
+      if (jj <= kGroupMaxJ) want = std::max(4, 1 << (jj - 3));
+      for (int q = want; q >= 2 && *P == 0; q /= 2) {
+        const int l = queue_ring_log2(jj, sc.w, q, 8);
+        if (l <= kQueueRsCapLog2 && queue_smem_bytes(q, l) <= (size_t)ctx->smem_optin / 2 - 1024) {
+          *P = q;
+          *lg = l;
+        }
+      }
+    }
+    if (*P == 0) bucket_schedule(ctx, jj, sc.w, P, R, lg, &huge, true);
+    return huge;
+  };
   // pairs of each launch
   int32_t pairs_of[kMaxLaunches] = {};
   for (int cls : {CLS_PACKED, CLS_NARROW, CLS_WIDE, CLS_NEAR, CLS_BAND}) {
@@ -548,28 +580,10 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
       ctx->plan_small = c < kBucketSmall;
       Launch L;
       bool lane = false, band = false;
-      if (cls == CLS_BAND && !band_ok) {
-        // a narrow band first, then the group engine for the pairs it leaves
-        if (pl->n_launch >= kMaxLaunches - 3 ||  // (kept by kMaxLaunches' bound)
-            !band_near_shape(sc, ctx->match, jj, &L.P, &L.R, &L.near_hw)) {
-          pl->bad = true;
-          continue;
-        }
-        L.cls = cls; L.band = true; L.j_lo = L.j_hi = j;
-        pairs_of[pl->n_launch] = c;
-        pl->launch[pl->n_launch++] = L;
-        pl->band_near++;
-        int P, R, lg;
-        bool huge;
-        bucket_schedule(ctx, jj, sc.w, &P, &R, &lg, &huge, true);
-        L = huge ? huge_launch(ctx, sc, pl) : queue_launch(ctx, cls, jj, P, R, lg);
-        L.cls = cls; L.j_lo = L.j_hi = j; L.after_prev = true;
-        pairs_of[pl->n_launch] = (c + kNearLeft - 1) / kNearLeft;
-        pl->launch[pl->n_launch++] = L;
-        prev = -1;
-        continue;
-      }
-      if (cls == CLS_BAND) {
+      // BAND pairs the band engine does not hold: a narrow band first, then the engine
+      // NARROW pairs would take, for those it leaves
+      const bool narrow_first = cls == CLS_BAND && !band_ok;
+      if (cls == CLS_BAND && band_ok) {
         band = true;
       } else if (cls != CLS_WIDE && lane_ok[jj]) {
         lane = true;
@@ -589,6 +603,42 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
                                            (double)kLaneSlots <= est_cells;
         }
       }
+      // (not where the call's long buckets fill the GPU with lanes twice over: those run
+      // as one launch, and apart, in turn on one ring region, each waits for its longest
+      // pair: 250k reads of 1,000-10,000 bases with 8% errors, w = 512, 1,118 and 551 ms)
+      if (narrow_first && !(lane && long_lanes)) {
+        if (pl->n_launch >= kMaxLaunches - 2 - kBandLaunches ||  // (kept by kMaxLaunches' bound)
+            !band_near_shape(sc, ctx->match, jj, &L.P, &L.R, &L.near_hw)) {
+          pl->bad = true;
+          continue;
+        }
+        auto push = [&](const Launch& l, bool after) {
+          Launch& x = pl->launch[pl->n_launch];
+          x = l;
+          x.cls = cls; x.j_lo = x.j_hi = j; x.after_prev = after;
+          pairs_of[pl->n_launch++] = c;
+        };
+        L.band = true;
+        push(L, false);
+        pl->band_near++;
+        int P, R, lg;
+        const bool huge = group_schedule(cls, jj, c, &P, &R, &lg);
+        Launch g = huge ? huge_launch(ctx, sc, pl) : queue_launch(ctx, cls, jj, P, R, lg);
+        // many pairs: lanes if the narrow band leaves a good part of them (but where
+        // only global slabs hold the band, those: 40k long reads, w = 1,000, 267 ms, 307)
+        const bool or_lanes = lane && !huge;
+        const int32_t many = (int32_t)(next_pow2(c) / 4);
+        g.gate = or_lanes ? -many : 0;
+        push(g, true);
+        if (or_lanes) {
+          Launch l;
+          lane_launch(ctx, sc, cls, jj, true, &l);
+          l.gate = many;
+          push(l, true);
+        }
+        prev = -1;
+        continue;
+      }
       // too few pairs for one lane each: groups of the band engine, whose rows
       // stop at the query's end and which work in 16 bits.  Queries of up to 126
       // bases stay on the group engine, which has all their rows in flight at once
@@ -606,32 +656,8 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
       } else if (lane) {
         lane_launch(ctx, sc, cls, jj, true, &L);
       } else {
-        int P = 0, R = 8, lg = 0;
-        bool huge = false;
-        const BucketSched* t = ctx->forced_P ? nullptr : tuned(ctx, sc.w, jj);
-        if (!ctx->forced_P && !t && c < min_pairs(jj) && cls != CLS_WIDE) {
-          // enough lanes per pair that the bucket's longest pair takes no
-          // longer than the call's whole work spread over the GPU's one-lane
-          // slots (the call's buckets run side by side, so a small bucket
-          // need not fill the GPU on its own; fewer lanes per pair waste less
-          // of each chunk on the wavefront's fill), where the ring fits
-          const double need = band_cells_est(pair_cells_q(jj), sc.w) * (double)kLaneSlots /
-                              std::max(est_cells, 1.0);
-          int want = 4;  // two-lane groups measured slower than four on every call size
-          while (want < 32 && want < need) want *= 2;
-          // short queries: 8 rows a lane for as many rows as the bucket's longest
-          // query has, one chunk of them (32 lanes idle half: 5,000 pairs of 64 bases
-          // 109 us a call, 94 so)
-          if (jj <= kGroupMaxJ) want = std::max(4, 1 << (jj - 3));
-          for (int q = want; q >= 2 && P == 0; q /= 2) {
-            const int l = queue_ring_log2(jj, sc.w, q, 8);
-            if (l <= kQueueRsCapLog2 && queue_smem_bytes(q, l) <= (size_t)ctx->smem_optin / 2 - 1024) {
-              P = q;
-              lg = l;
-            }
-          }
-        }
-        if (P == 0) bucket_schedule(ctx, jj, sc.w, &P, &R, &lg, &huge, true);
+        int P, R, lg;
+        const bool huge = group_schedule(cls, jj, c, &P, &R, &lg);
         if (huge && cls != CLS_WIDE && lane_ok[jj]) {
           lane_launch(ctx, sc, cls, jj, true, &L);  // no group ring fits: one lane per pair
         } else if (huge) {
@@ -722,6 +748,22 @@ size_t ring_launch_bytes(const Launch& L) {
 // the call's branches, each filling the slots the others leave), else they
 // share one region and run one after another.
 size_t layout_pool(const xt_ctx* ctx, Plan* pl) {
+  auto allowed = [&](size_t bytes) {
+    return ctx->budget == 0 || bytes <= ctx->pool_bytes ||
+           ctx->held + (bytes - ctx->pool_bytes) <= ctx->budget;
+  };
+  // lanes for what a narrow band leaves only as far as the budget holds their rings:
+  // the group launch before them takes the pairs else
+  for (int i = 1; i < pl->n_launch;) {
+    const Launch& L = pl->launch[i];
+    if (L.gate <= 0 || !L.global_ring || allowed(ring_launch_bytes(L))) {
+      ++i;
+      continue;
+    }
+    pl->launch[i - 1].gate = 0;
+    for (int k = i; k + 1 < pl->n_launch; ++k) pl->launch[k] = pl->launch[k + 1];
+    --pl->n_launch;
+  }
   size_t sum = 0, most = 0;
   for (int i = 0; i < pl->n_launch; ++i) {
     Launch& L = pl->launch[i];
@@ -731,9 +773,7 @@ size_t layout_pool(const xt_ctx* ctx, Plan* pl) {
     sum += align_up(b);
     most = std::max(most, b);
   }
-  const bool fits = sum <= kPoolCap &&
-                    (ctx->budget == 0 || sum <= ctx->pool_bytes ||
-                     ctx->held + (sum - ctx->pool_bytes) <= ctx->budget);
+  const bool fits = sum <= kPoolCap && allowed(sum);
   pl->pool_serial = !fits;
   if (fits) return sum;
   for (int i = 0; i < pl->n_launch; ++i) pl->launch[i].pool_off = 0;
@@ -871,8 +911,8 @@ cudaError_t enqueue_dp(xt_ctx* ctx, bool plain, const Plan& pl, int plain_rs, co
   for (int i = 0; e == cudaSuccess && i < pl.n_launch; ++i) {
     const Launch& L = pl.launch[i];
     // a launch that takes what the one before it left follows on its stream
-    const bool leads = i + 1 < pl.n_launch && pl.launch[i + 1].after_prev;
-    const bool ring = L.global_ring || (leads && pl.launch[i + 1].global_ring);
+    bool ring = L.global_ring;
+    for (int k = i + 1; k < pl.n_launch && pl.launch[k].after_prev; ++k) ring |= pl.launch[k].global_ring;
     if (!L.after_prev) st = nb > 1 ? ctx->aux[ring && pl.pool_serial ? 0 : (rr++ % nb)] : stream;
     if (near && L.cls == CLS_NEAR && nb > 1) e = cudaStreamWaitEvent(st, ctx->near_ev, 0);
     if (e != cudaSuccess) break;
@@ -918,7 +958,7 @@ uint64_t plan_signature(const Plan& pl) {
   for (int i = 0; i < pl.n_launch; ++i) {
     const Launch& L = pl.launch[i];
     mix(L.cls); mix(L.j_lo); mix(L.j_hi); mix(L.lane); mix(L.band); mix(L.P); mix(L.R); mix(L.rs_log2);
-    mix(L.near_hw); mix(L.cls2); mix(L.after_prev); mix(L.global_ring); mix(L.slab); mix(L.grid); mix(L.mparam); mix((int64_t)L.pool_off);
+    mix(L.near_hw); mix(L.cls2); mix(L.after_prev); mix(L.gate); mix(L.global_ring); mix(L.slab); mix(L.grid); mix(L.mparam); mix((int64_t)L.pool_off);
   }
   mix(pl.pool_serial);
   mix(pl.near_grid);
@@ -1796,7 +1836,6 @@ bool carve_static(void* base_ptr, int32_t n, Work* w, Batch** desc) {
   w->heads = (int32_t*)(base + o_heads);
   w->near_hope = nullptr;  // no near pass on this path
   w->near_left = nullptr;
-  w->band_left = nullptr;
   w->near_tmp = nullptr;
   *desc = (Batch*)(base + o_desc);
   return true;

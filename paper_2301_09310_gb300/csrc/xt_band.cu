@@ -56,8 +56,7 @@ __host__ __device__ constexpr int base_age(int P) { return P + kBaseSteps; }
 
 // NEAR: the P * K slots hold diagonals |i - j| <= hw of a wider band (hw <
 // sc.w); a pair is settled only where the bounds of xt_bounds.cuh prove its
-// outputs, and the others go to near_tmp at their bucket's place in the queue
-// (counted in band_left).
+// outputs, and the others are marked in near_tmp, at their place in the queue.
 template <int P, int K, bool NEAR>
 __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
     k_band(const Batch* __restrict__ bd, Score sc, Work w, int cls, int j_lo, int j_hi,
@@ -164,10 +163,10 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
     // the last one seen (the rows since was_best was taken against that best,
     // those to come against the last); a failed pair is left
     int32_t was_best[2] = {h0[0], h0[1]};
+    const int32_t at = base_idx + 2 * (lane / P);
     auto leave = [&](int h) {
       act[h] = false;
-      const int j = bucket_of(ql[h]);
-      w.near_tmp[w.seg_begin[cls * kNumJ + j] + atomicAdd(&w.band_left[j], 1)] = kk[h];
+      w.near_tmp[at + h] = 1;
     };
     auto settled = [&](int h, int32_t i) -> bool {
       const int32_t top = half(best2, h), cap = min(tl[h] - 1, ql[h] - 1 + sc.w);
@@ -177,6 +176,7 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
     };
     auto finish = [&](int h, int32_t last) {
       act[h] = false;
+      if (NEAR) w.near_tmp[at + h] = 0;
       const int32_t d = mid - half(bu2, h);  // diagonal of the best
       write_result(b, kk[h], half(best2, h), brow[h] - d + 1, brow[h] + 1, g[h],
                    g[h] > 0 ? grow[h] + 1 : 0, half(off2, h), XT_OK,
@@ -440,7 +440,15 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
       if (NEAR && p == P - 1 && i >= 0) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          if (act[h] && !near_row_ok(i, ql[h], h0[h], match, hw, was_best[h], sc)) leave(h);
+          // (1') bounds the loss on the rows up to the last hw + 1.  A pair that loses
+          // so fast that it would come to twice that (from row 255 on half as much
+          // again) is left at once: long reads with 8% errors fail some way down their
+          // thousands of rows anyway (1,000 of them, w = 512, 28.5 -> 17.4 ms with the CTAs for what is left)
+          const int32_t rows = ql[h] - hw - 1, seen = i - 7;  // (was_best is of eight rows ago)
+          const float lost = h0[h] + match * seen - was_best[h];
+          const bool fast = i >= 127 && i < rows &&
+                            lost * rows > (i < 255 ? 2.0f : 1.5f) * (alpha - beta + beta * (hw + 1)) * seen;
+          if (act[h] && (fast || !near_row_ok(i, ql[h], h0[h], match, hw, was_best[h], sc))) leave(h);
           was_best[h] = half(best2, h);
         }
       }
@@ -456,13 +464,48 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
   }
 }
 
-// The pairs the NEAR launch of bucket j left, from near_tmp to the front of the
-// bucket's run in the queue.
-__global__ void k_band_gather(Work w, int cls, int j) {
-  const int32_t at = w.seg_begin[cls * kNumJ + j], n = w.band_left[j];
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    w.order[at + i] = w.near_tmp[at + i];
-  if (blockIdx.x == 0 && threadIdx.x == 0) w.seg_end[cls * kNumJ + j] = at + n;
+// The pairs the NEAR launch of bucket j left move to the front of the bucket's run in
+// the queue, in their order (longest first: lanes of a warp then hold pairs of like
+// length; in the order they were left 55k streamed pairs, w = 600, took 9.0 ms a call, 7.1
+// so).  One block, each thread kPackPer neighbouring places a round; a round's places
+// are read before they are written, and none is written before its own round.
+constexpr int kPackThreads = 1024;
+constexpr int kPackPer = 8;
+
+__global__ void __launch_bounds__(kPackThreads) k_band_pack(Work w, int cls, int j) {
+  __shared__ int32_t s_warp[kPackThreads / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int32_t begin = w.seg_begin[cls * kNumJ + j], end = w.seg_end[cls * kNumJ + j];
+  int32_t out = begin;
+  for (int32_t round = begin; round < end; round += kPackThreads * kPackPer) {
+    const int32_t first = round + threadIdx.x * kPackPer;
+    int32_t pair[kPackPer], mine = 0;
+#pragma unroll
+    for (int u = 0; u < kPackPer; ++u) {
+      const bool left = first + u < end && w.near_tmp[first + u] != 0;
+      pair[u] = left ? w.order[first + u] : -1;
+      mine += left;
+    }
+    int32_t inc = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int32_t v = __shfl_up_sync(0xffffffffu, inc, d);
+      if (lane >= d) inc += v;
+    }
+    if (lane == 31) s_warp[wid] = inc;
+    __syncthreads();
+    int32_t at = out + inc - mine, total = 0;
+    for (int u = 0; u < kPackThreads / 32; ++u) {
+      if (u < wid) at += s_warp[u];
+      total += s_warp[u];
+    }
+#pragma unroll
+    for (int u = 0; u < kPackPer; ++u)
+      if (pair[u] >= 0) w.order[at++] = pair[u];
+    out += total;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) w.seg_end[cls * kNumJ + j] = out;
 }
 
 // The lane counts and slots compiled: per lane count, fewest slots first.
@@ -537,7 +580,7 @@ cudaError_t launch_band(const Batch* bd, const Score& sc, int32_t match, const W
     k_band<PP, KK, NN><<<L.grid, kBandThreads, 0, stream>>>(                                   \
         bd, sc, w, L.cls, L.j_lo, L.j_hi, head_id, match, 1u << mshift, 1u << kKeyBits, fall,  \
         num_sms, NN ? L.near_hw : sc.w);                                                       \
-    if (NN) k_band_gather<<<16, 256, 0, stream>>>(w, L.cls, L.j_lo);                           \
+    if (NN) k_band_pack<<<1, kPackThreads, 0, stream>>>(w, L.cls, L.j_lo);                           \
     return cudaGetLastError();                                                                 \
   }
   XT_BL(2, 32, false) XT_BL(4, 32, false) XT_BL(8, 26, false) XT_BL(8, 32, false)

@@ -65,7 +65,6 @@ constexpr int kNearJMax = 9;
 constexpr int kNearMaxQ = (1 << kNearJMax) - 2;
 static_assert(kNearJMax <= kExactJ, "one bin per length");
 constexpr int kNearBins = 1 << kNearJMax;
-constexpr int kBandLeft = (kNumJ + 3) / 4 * 4;
 constexpr int kQueueThreads = 128;       // threads per CTA of the queue kernels
 // Queue-kernel launches per call (heads), at most one a bucket and class: WIDE pairs
 // in every bucket, PACKED and NARROW ones up to 65,535 bases, NEAR ones up to
@@ -91,8 +90,8 @@ struct Work {
   int32_t* near_hope;   // [1] NEAR pairs whose diagonal promises that k_near settles them
   int32_t* heads;       // [kMaxLaunches]
   int32_t* near_left;   // [kNearBins] pairs k_near left, per exact length
-  int32_t* band_left;   // [kBandLeft] pairs a narrow band launch left, per bucket
-  int32_t* near_tmp;    // [n] those pairs, each length's (bucket's) run where its queue run was
+  int32_t* near_tmp;    // [n] those pairs, each length's run where its queue run was; or 1 at
+                        // the places in the queue of the pairs a narrow band left
 };
 
 constexpr int kLaneThreads = 128;        // threads per CTA of the one-lane kernels
@@ -108,6 +107,9 @@ struct Launch {
   int near_hw = 0;           // > 0: on a narrower band of this half width
   int cls2 = -1;             // one-lane engine: then this class's pairs of the same buckets
   bool after_prev = false;   // takes the pairs the launch before it left, on its stream
+  // runs only where its segment holds at least gate pairs, or (negative) fewer than
+  // -gate: two engines for what a narrow band leaves, which only the device knows
+  int32_t gate = 0;
   int P = 1, R = 8;          // lanes per pair, rows per lane-strip (per half when packed)
   int rs_log2 = 0;           // ring entries per group = 1 << rs_log2
   bool global_ring = false;  // ring in a global slab per group instead of shared memory

@@ -74,8 +74,8 @@ __global__ void __launch_bounds__(kDescThreads) k_store_desc(Batch* dst, Batch b
     for (int i = threadIdx.x; i < kNumBuckets / 4; i += kDescThreads)
       reinterpret_cast<int4*>(w.counts)[i] = z;
   if (w.heads && threadIdx.x < kMaxLaunches / 4) reinterpret_cast<int4*>(w.heads)[threadIdx.x] = z;
-  if (w.near_left)  // and band_left after it
-    for (int i = threadIdx.x; i < (kNearBins + kBandLeft) / 4; i += kDescThreads)
+  if (w.near_left)
+    for (int i = threadIdx.x; i < kNearBins / 4; i += kDescThreads)
       reinterpret_cast<int4*>(w.near_left)[i] = z;
 }
 

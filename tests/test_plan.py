@@ -116,4 +116,24 @@ def test_every_class_and_bucket_gets_its_launch(plan):
         for (cls, j), v in c["counts"].items():
             runs = [L for L in p["launches"] if not L["near_hw"]
                     and (L["cls"] == cls or L["cls2"] == cls) and L["j_lo"] <= j <= L["j_hi"]]
-            assert len(runs) == 1, (c["sc"], cls, j, runs)
+            gates = sorted(L["gate"] for L in runs)
+            assert gates in ([0], [-gates[-1], gates[-1]]), (c["sc"], cls, j, runs)
+
+
+def test_what_a_narrow_band_leaves_gets_the_engines_narrow_pairs_take(plan):
+    sc = ScoringParams(w=512, zdrop=400)
+    few, many, tight = plan([
+        {"sc": sc, "counts": {(BAND, 12): 3000}},
+        {"sc": sc, "counts": {(BAND, 12): 60_000}},
+        {"sc": sc, "counts": {(BAND, 12): 60_000}, "budget": 64 << 20}])
+    # a CTA of the group launch for every four pairs, up to the GPU's own number
+    narrow, group = few["launches"]
+    assert narrow["near_hw"] > 0 and group["engine"] == "group" and group["after_prev"]
+    assert group["P"] == 32 and group["grid"] >= 456 and group["gate"] == 0
+    # where lanes would take all of them, lanes or groups by the number left
+    narrow, group, lane = many["launches"]
+    assert (group["engine"], lane["engine"]) == ("group", "lane")
+    assert group["gate"] == -lane["gate"] and 60_000 / 4 <= lane["gate"] <= 60_000 / 2
+    # no rings beyond the budget
+    assert [L["engine"] for L in tight["launches"]] == ["band", "group"]
+    assert tight["launches"][1]["gate"] == 0 and tight["pool"] <= 64 << 20
