@@ -61,6 +61,10 @@ __host__ __device__ constexpr int bwa_lane_cap(int c) { return 64 << c; }
 // 1.6 / 1.5 ms with every class on lanes, those up to 64 bases 0.77 and 0.95 ms of
 // it; 2M: 28.0 and 18.1 ms).
 __host__ __device__ constexpr int32_t bwa_lane_min(int c) { return c == 0 ? 1 << 18 : 1 << 15; }
+// The widest lane class holds so little of the SM that rows of few columns run sooner
+// on groups of two to four lanes (400k reads of 200 bases, w = 10 / 20 / 40 / 70: 5.06 /
+// 6.54 / 9.1 / 11.8 ms on lanes, 3.55 / 5.14 / 9.9 / 16.0 on groups).
+constexpr int kBwaLaneMinWidth = 89;
 constexpr int kBwaClasses = 16;              // of them 11 in use (their order is the queue's)
 // The shortest lane class lies before the narrowest groups, which may take it.
 __host__ __device__ constexpr int bwa_lane_id(int c) { return c == 0 ? 0 : kBwaGroupClasses + c; }
@@ -169,13 +173,17 @@ __global__ void k_bwa_classify(BwaArgs a) {
     } else {
       int c = 0;
       const int64_t bound = h0 + (int64_t)ql * a.sc.match;
-      if (ql >= kBwaLaneMinQ && ql <= bwa_lane_cap(kBwaLaneClasses - 1) && bound <= kBwaLaneMaxH &&
-          ((bound + 1) << a.mshift) <= 32767) {
+      bool lane = ql >= kBwaLaneMinQ && ql <= bwa_lane_cap(kBwaLaneClasses - 1) &&
+                  bound <= kBwaLaneMaxH && ((bound + 1) << a.mshift) <= 32767;
+      if (lane) {
         while (bwa_lane_cap(c) < ql) ++c;
         if (bound > 255) c = kBwaLaneClasses - 1;
+        lane = c < kBwaLaneClasses - 1 || width >= kBwaLaneMinWidth;
+      }
+      if (lane) {
         c = bwa_lane_id(c);
       } else {
-        while ((64 << c) < width) ++c;
+        for (c = 0; (64 << c) < width;) ++c;
         c = bwa_group_id(c);
       }
       cls = (uint8_t)c;
