@@ -10,6 +10,7 @@
 
 #include "xt.h"
 #include "xt_ctx.cuh"
+#include "xt_fork.cuh"
 #include "xt_kernels.cuh"
 
 using namespace xt;
@@ -896,15 +897,13 @@ cudaError_t enqueue_dp(xt_ctx* ctx, bool plain, const Plan& pl, int plain_rs, co
   // leaves wait for it on theirs.
   const bool near = pl.near_pairs > 0;
   const int nb = std::min(ctx->branches, pl.n_launch + (near ? 1 : 0));
-  if (e == cudaSuccess && nb > 1) {
-    e = cudaEventRecord(ctx->fork_ev, stream);
-    for (int b = 0; e == cudaSuccess && b < nb; ++b) e = cudaStreamWaitEvent(ctx->aux[b], ctx->fork_ev, 0);
-  }
+  Fork fork(stream, ctx->aux, ctx->fork_ev, ctx->join_ev, e == cudaSuccess ? nb : 0);
+  if (e == cudaSuccess) e = fork.error();
   int rr = 0;
   if (e == cudaSuccess && near) {
-    cudaStream_t st = nb > 1 ? ctx->aux[rr++] : stream;
+    cudaStream_t st = fork.branch(rr++);
     e = launch_near(desc, sc, ctx->match, pl.near_grid, w, kMaxLaunches - 1, st);
-    if (e == cudaSuccess && nb > 1) e = cudaEventRecord(ctx->near_ev, st);
+    if (e == cudaSuccess && fork.apart()) e = cudaEventRecord(ctx->near_ev, st);
     dp += 2;
   }
   cudaStream_t st = stream;
@@ -913,8 +912,8 @@ cudaError_t enqueue_dp(xt_ctx* ctx, bool plain, const Plan& pl, int plain_rs, co
     // a launch that takes what the one before it left follows on its stream
     bool ring = L.global_ring;
     for (int k = i + 1; k < pl.n_launch && pl.launch[k].after_prev; ++k) ring |= pl.launch[k].global_ring;
-    if (!L.after_prev) st = nb > 1 ? ctx->aux[ring && pl.pool_serial ? 0 : (rr++ % nb)] : stream;
-    if (near && L.cls == CLS_NEAR && nb > 1) e = cudaStreamWaitEvent(st, ctx->near_ev, 0);
+    if (!L.after_prev) st = fork.branch(ring && pl.pool_serial ? 0 : rr++);
+    if (near && L.cls == CLS_NEAR && fork.apart()) e = cudaStreamWaitEvent(st, ctx->near_ev, 0);
     if (e != cudaSuccess) break;
     void* gring = L.global_ring ? static_cast<void*>(reinterpret_cast<char*>(ctx->pool) + L.pool_off)
                                 : nullptr;
@@ -931,12 +930,8 @@ cudaError_t enqueue_dp(xt_ctx* ctx, bool plain, const Plan& pl, int plain_rs, co
     }
     dp += L.near_hw > 0 ? 2 : 1;
   }
-  if (e == cudaSuccess && nb > 1) {
-    for (int b = 0; e == cudaSuccess && b < nb; ++b) {
-      e = cudaEventRecord(ctx->join_ev[b], ctx->aux[b]);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ctx->join_ev[b], 0);
-    }
-  }
+  const cudaError_t joined = fork.join();
+  if (e == cudaSuccess) e = joined;
   if (e == cudaSuccess && timed) {
     cudaEventRecord(ctx->ev[slot][1], stream);
     ctx->ev_pending = slot + 1;

@@ -37,6 +37,7 @@
 #include "xt.h"
 #include "xt_common.cuh"
 #include "xt_ctx.cuh"
+#include "xt_fork.cuh"
 #include "xt_near.cuh"
 
 namespace xt {
@@ -1075,23 +1076,18 @@ extern "C" xt_status xt_extend_batch_bwa(xt_ctx* ctx, const uint8_t* q_seq, int6
   int used = 0;
   for (int c = 0; c < kBwaClasses; ++c) used += cnt[c] > 0;
   const int nb = std::min(ctx->branches, used);
-  if (e == cudaSuccess && nb > 1) {
-    e = cudaEventRecord(ctx->fork_ev, st);
-    for (int b = 0; e == cudaSuccess && b < nb; ++b)
-      e = cudaStreamWaitEvent(ctx->aux[b], ctx->fork_ev, 0);
-  }
+  Fork fork(st, ctx->aux, ctx->fork_ev, ctx->join_ev, e == cudaSuccess ? nb : 0);
+  if (e == cudaSuccess) e = fork.error();
   int rr = 0;
   auto launch = [&](int c) {
     if (cnt[c] > 0 && e == cudaSuccess)
-      e = launch_bwa_class(ctx, a, c, off[c], cnt[c], nb > 1 ? ctx->aux[rr++ % nb] : st);
+      e = launch_bwa_class(ctx, a, c, off[c], cnt[c], fork.branch(rr++));
   };
   for (int c = kBwaGroupClasses - 1; c >= 2; --c) launch(bwa_group_id(c));
   for (int c = kBwaLaneClasses - 1; c >= 1; --c) launch(bwa_lane_id(c));
   for (int id : {bwa_group_id(1), bwa_lane_id(0), bwa_group_id(0)}) launch(id);
-  for (int b = 0; nb > 1 && b < nb && e == cudaSuccess; ++b) {
-    e = cudaEventRecord(ctx->join_ev[b], ctx->aux[b]);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ctx->join_ev[b], 0);
-  }
+  const cudaError_t joined = fork.join();
+  if (e == cudaSuccess) e = joined;
   if (e != cudaSuccess) return ctx_cuda_fail(ctx, e, "BWA extension");
   ctx->calls++;
   return XT_OK;
