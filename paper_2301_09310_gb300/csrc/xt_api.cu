@@ -992,6 +992,9 @@ xt_status run_begin(xt_ctx* ctx, bool plain, bool early, const uint8_t* q_seq, i
   pc.n_cap = pc.n_cap_log2 >= 31 ? INT32_MAX : (1 << pc.n_cap_log2);
   pc.has_cells = cells != nullptr;
   pc.stream = stream;
+  pc.forced_P = ctx->forced_P;
+  pc.forced_R = ctx->forced_R;
+  pc.near_first = ctx->near_first;
   s = get_work(ctx, pc.n_cap, &pc.w, &pc.desc);
   if (s != XT_OK) return s;
   ctx->match = scr->match;
@@ -1032,6 +1035,26 @@ xt_status run_begin(xt_ctx* ctx, bool plain, bool early, const uint8_t* q_seq, i
   return XT_OK;
 }
 
+// The context with a begun call's override and near passes, for as long as it lives.
+struct BegunRules {
+  xt_ctx* ctx;
+  int P, R;
+  bool near_first;
+  BegunRules(xt_ctx* c, const PendingCall& pc)
+      : ctx(c), P(c->forced_P), R(c->forced_R), near_first(c->near_first) {
+    c->forced_P = pc.forced_P;
+    c->forced_R = pc.forced_R;
+    c->near_first = pc.near_first;
+  }
+  BegunRules(const BegunRules&) = delete;
+  BegunRules& operator=(const BegunRules&) = delete;
+  ~BegunRules() {
+    ctx->forced_P = P;
+    ctx->forced_R = R;
+    ctx->near_first = near_first;
+  }
+};
+
 // The second half: plan from the counts (waiting for them if needed) and
 // enqueue the extension kernels, through a captured graph when one exists.
 xt_status run_finish(xt_ctx* ctx) {
@@ -1039,6 +1062,7 @@ xt_status run_finish(xt_ctx* ctx) {
   if (!pc.active) return fail(ctx, XT_EINVAL, "no begun call to finish");
   pc.active = false;
   if (pc.n == 0) return XT_OK;
+  const BegunRules rules(ctx, pc);
   cudaError_t e = cudaSetDevice(ctx->device);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaSetDevice");
   const bool plain = pc.plain;

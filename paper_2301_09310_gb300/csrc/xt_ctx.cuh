@@ -111,6 +111,10 @@ struct PendingCall {
   bool has_cells = false;
   cudaStream_t stream = nullptr;
   JFlags jf{};
+  // the context's schedule override and near passes at _begin: the pairs' classes
+  // follow from them, so the plan does too, whatever is set before _finish
+  int forced_P = 0, forced_R = 0;
+  bool near_first = true;
   bool diag = false;            // the diagonal pass ran
   bool lane_ok[kNumJ] = {};
 };
