@@ -69,9 +69,21 @@ Score make_score(const xt_scoring* s) {
   return sc;
 }
 
+// Give back the near passes' buffer (cudaFree waits for the kernels that use it).
+bool drop_near_buf(xt_ctx* ctx) {
+  if (!ctx->near_buf) return false;
+  cudaFree(ctx->near_buf);
+  ctx->held -= ctx->near_bytes;
+  ctx->near_buf = nullptr;
+  ctx->near_bytes = 0;
+  drop_graphs(ctx);
+  return true;
+}
+
 xt_status dev_alloc(xt_ctx* ctx, void** p, size_t* have, size_t want) {
   if (*have >= want) return XT_OK;
   const size_t grow = want - *have;
+  if (ctx->budget && ctx->held + grow > ctx->budget && p != &ctx->near_buf) drop_near_buf(ctx);
   if (ctx->budget && ctx->held + grow > ctx->budget)
     return fail(ctx, XT_ENOMEM, "device memory budget exceeded");
   if (*p) {
@@ -81,6 +93,10 @@ xt_status dev_alloc(xt_ctx* ctx, void** p, size_t* have, size_t want) {
     *have = 0;
   }
   cudaError_t e = cudaMalloc(p, want);
+  if (e != cudaSuccess && p != &ctx->near_buf && drop_near_buf(ctx)) {
+    cudaGetLastError();
+    e = cudaMalloc(p, want);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
@@ -153,7 +169,6 @@ xt_status get_work(xt_ctx* ctx, int32_t n, Work* w, Batch** desc) {
   const size_t o_hope = off; off = align_up(off + 4);  // read back with the bucket counts
   const size_t o_heads = off; off = align_up(off + 4 * (size_t)kMaxLaunches);
   const size_t o_left = off; off = align_up(off + 4 * (size_t)kNearBins);
-  const size_t o_tmp = off; off = align_up(off + 4 * (size_t)n);
   void* old = ctx->work;
   xt_status s = dev_alloc(ctx, &ctx->work, &ctx->work_bytes, off);
   if (s != XT_OK) return s;
@@ -169,8 +184,20 @@ xt_status get_work(xt_ctx* ctx, int32_t n, Work* w, Batch** desc) {
   w->near_hope = (int32_t*)(base + o_hope);
   w->heads = (int32_t*)(base + o_heads);
   w->near_left = (int32_t*)(base + o_left);
-  w->near_tmp = (int32_t*)(base + o_tmp);
+  w->near_tmp = nullptr;  // of a plan that runs the near passes (get_near)
   return XT_OK;
+}
+
+// The buffer of the pairs the near passes leave, for calls of n pairs; false where the
+// budget or the device does not hold it.
+bool get_near(xt_ctx* ctx, int32_t n, Work* w) {
+  void* old = ctx->near_buf;
+  const std::string last_error = ctx->last_error;
+  const bool ok = dev_alloc(ctx, &ctx->near_buf, &ctx->near_bytes, 4 * (size_t)n) == XT_OK;
+  if (ctx->near_buf != old) drop_graphs(ctx);
+  if (!ok) ctx->last_error = last_error;
+  w->near_tmp = ok ? (int32_t*)ctx->near_buf : nullptr;
+  return ok;
 }
 
 struct Plan {
@@ -471,7 +498,8 @@ Launch queue_launch(const xt_ctx* ctx, int cls, int j, int P, int R, int lg) {
 // empty buckets get no launch; a bucket too small to fill the GPU takes its
 // small-batch schedule, or by default a group schedule with enough lanes per
 // pair to fill it; larger buckets take the throughput schedule.
-void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t hopeful,
+// near_ok: there is a buffer for what near passes leave.
+void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t hopeful, bool near_ok,
                  const JFlags& jf, const bool* lane_ok, Plan* pl) {
   pl->jf = jf;
   // the band engine, where it holds the band
@@ -516,7 +544,7 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
   for (int cls = CLS_PACKED; cls < kNumClasses; ++cls)
     for (int j = kNearJMax + 1; j < kNumJ; ++j) longer += cnt[cls][j];
   const double left = near_left_est(hopeful, near);
-  bool pass = (near >= kNearPassMin || (near > 0 && longer > 0)) &&
+  bool pass = near_ok && (near >= kNearPassMin || (near > 0 && longer > 0)) &&
               near * (1.0 - left) >= kNearSaves * ((double)near + rest);
   if (longer == 0 && (int64_t)near + rest <= kLaneSlots && (lanes_after || (!sooner && left > 0.34)))
     pass = false;
@@ -607,7 +635,7 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
       // (not where the call's long buckets fill the GPU with lanes twice over: those run
       // as one launch, and apart, in turn on one ring region, each waits for its longest
       // pair: 250k reads of 1,000-10,000 bases with 8% errors, w = 512, 1,118 and 551 ms)
-      if (narrow_first && !(lane && long_lanes)) {
+      if (narrow_first && near_ok && !(lane && long_lanes)) {
         if (pl->n_launch >= kMaxLaunches - 2 - kBandLaunches ||  // (kept by kMaxLaunches' bound)
             !band_near_shape(sc, ctx->match, jj, &L.P, &L.R, &L.near_hw)) {
           pl->bad = true;
@@ -659,7 +687,10 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
       } else {
         int P, R, lg;
         const bool huge = group_schedule(cls, jj, c, &P, &R, &lg);
-        if (huge && cls != CLS_WIDE && lane_ok[jj]) {
+        if (huge && narrow_first) {
+          L = huge_launch(ctx, sc, pl);
+          L.cls = cls;
+        } else if (huge && cls != CLS_WIDE && lane_ok[jj]) {
           lane_launch(ctx, sc, cls, jj, true, &L);  // no group ring fits: one lane per pair
         } else if (huge) {
           // the flags gave these pairs no HUGE class, so they would be lost
@@ -800,6 +831,7 @@ xt_status xt::ctx_reserve(xt_ctx* ctx, int32_t n_pairs, size_t conv_bytes, size_
   xt_status s = get_work(ctx, lg >= 31 ? INT32_MAX : (1 << lg), &w, &desc);
   if (s == XT_OK && conv_bytes) s = dev_alloc(ctx, &ctx->conv, &ctx->conv_bytes, conv_bytes);
   if (s != XT_OK) return s;
+  get_near(ctx, lg >= 31 ? INT32_MAX : (1 << lg), &w);  // (given back where anything else needs it)
   size_t pool = std::min(pool_bytes, kPoolCap);
   if (ctx->budget) {
     const size_t left = ctx->budget > ctx->held ? ctx->budget - ctx->held : 0;
@@ -1035,6 +1067,15 @@ xt_status run_begin(xt_ctx* ctx, bool plain, bool early, const uint8_t* q_seq, i
   return XT_OK;
 }
 
+// The ring pool for a plan that needs `want` bytes of it.
+xt_status get_pool(xt_ctx* ctx, size_t want) {
+  if (!want) return XT_OK;
+  void* old = ctx->pool;
+  const xt_status s = dev_alloc(ctx, (void**)&ctx->pool, &ctx->pool_bytes, want);
+  if (s == XT_OK && (void*)ctx->pool != old) drop_graphs(ctx);
+  return s;
+}
+
 // The context with a begun call's override and near passes, for as long as it lives.
 struct BegunRules {
   xt_ctx* ctx;
@@ -1079,18 +1120,28 @@ xt_status run_finish(xt_ctx* ctx) {
     if (e != cudaSuccess) return cuda_fail(ctx, e, "classify");
     const int32_t* sb = ctx->seg_host;
     const int32_t* se = ctx->seg_host + (w.seg_end - w.seg_begin);
-    int32_t cnt[kNumClasses][kNumJ];
-    for (int c = 0; c < kNumClasses; ++c)
-      for (int j = 0; j < kNumJ; ++j) cnt[c][j] = se[c * kNumJ + j] - sb[c * kNumJ + j];
-    plan_counts(ctx, sc, cnt, se[kNumClasses * kNumJ], pc.jf, pc.lane_ok, &pl);
+    const int32_t hopeful = se[kNumClasses * kNumJ];
+    auto plan = [&](bool near_ok) {
+      int32_t cnt[kNumClasses][kNumJ];
+      for (int c = 0; c < kNumClasses; ++c)
+        for (int j = 0; j < kNumJ; ++j) cnt[c][j] = se[c * kNumJ + j] - sb[c * kNumJ + j];
+      pl = Plan();
+      plan_counts(ctx, sc, cnt, hopeful, near_ok, pc.jf, pc.lane_ok, &pl);
+    };
+    plan(true);
+    const size_t want = layout_pool(ctx, &pl);
+    xt_status s = get_pool(ctx, want);
+    // the near passes are a shortcut: without memory for them the engines take all
+    if ((pl.near_pairs > 0 || pl.band_near > 0) && (s != XT_OK || !get_near(ctx, pc.n_cap, &pc.w))) {
+      plan(false);
+      s = get_pool(ctx, layout_pool(ctx, &pl));
+    }
+    if (s != XT_OK) return s;
     if (pl.bad) return fail(ctx, XT_ECUDA, "internal: inconsistent bucket plan");
   }
-  const size_t want = layout_pool(ctx, &pl);
-  if (want) {
-    void* old = ctx->pool;
-    xt_status s = dev_alloc(ctx, (void**)&ctx->pool, &ctx->pool_bytes, want);
+  if (plain) {
+    const xt_status s = get_pool(ctx, layout_pool(ctx, &pl));
     if (s != XT_OK) return s;
-    if ((void*)ctx->pool != old) drop_graphs(ctx);
   }
   // the plain path's whole call, or the batched path's extension kernels,
   // replay as one graph once a call with the same key has been seen
@@ -1107,6 +1158,7 @@ xt_status run_finish(xt_ctx* ctx) {
     std::memset(&key, 0, sizeof(key));
     key.plain = plain; key.sc = pc.scr; key.forced_P = ctx->forced_P; key.forced_R = ctx->forced_R;
     key.n_cap_log2 = pc.n_cap_log2; key.work = ctx->work; key.pool = ctx->pool;
+    key.near_buf = ctx->near_buf;
     key.has_cells = pc.has_cells;
     key.plan_sig = plan_signature(pl);
     key.branches = ctx->branches;
@@ -1230,6 +1282,7 @@ xt_status xt_ctx_destroy(xt_ctx* ctx) {
   cudaDeviceSynchronize();
   if (ctx->work) cudaFree(ctx->work);
   if (ctx->pool) cudaFree(ctx->pool);
+  if (ctx->near_buf) cudaFree(ctx->near_buf);
   if (ctx->dev_in) cudaFree(ctx->dev_in);
   if (ctx->conv) cudaFree(ctx->conv);
   if (ctx->seed_ws) cudaFree(ctx->seed_ws);

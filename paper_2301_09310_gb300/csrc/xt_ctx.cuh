@@ -19,6 +19,7 @@ struct GraphKey {
   int n_cap_log2;
   void* work;
   void* pool;
+  void* near_buf;
   bool has_cells;
   uint64_t plan_sig;   // the plan of the extension kernels (count-aware)
   int branches;
@@ -130,6 +131,10 @@ struct xt_ctx {
   // per-call workspace (grown on demand)
   void* work = nullptr;
   size_t work_bytes = 0;
+  // what the near passes leave (Work::near_tmp): held only by calls that run them, and
+  // given back where the budget needs it for anything else
+  void* near_buf = nullptr;
+  size_t near_bytes = 0;
   // global ring pool for pairs whose band does not fit in shared memory
   int2* pool = nullptr;
   size_t pool_bytes = 0;

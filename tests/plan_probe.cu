@@ -1,6 +1,6 @@
 // Runs the library's planner on pair counts without a GPU (tests/test_plan.py).
 // Each case on standard input: a line "w match mismatch gap_open gap_extend zdrop
-// n_score n hopeful budget tunings counts", then `tunings` lines "j batch_class P R"
+// n_score n hopeful budget near_ok tunings counts", then `tunings` lines "j batch_class P R"
 // and `counts` lines "class j pairs"; one JSON line out per case.
 #include "xt_api.cu"
 
@@ -8,9 +8,9 @@
 
 int main() {
   xt_scoring s;
-  int64_t n, hopeful, budget, tunings, counts;
+  int64_t n, hopeful, budget, near_ok, tunings, counts;
   while (std::cin >> s.w >> s.match >> s.mismatch >> s.gap_open >> s.gap_extend >> s.zdrop >>
-         s.n_score >> n >> hopeful >> budget >> tunings >> counts) {
+         s.n_score >> n >> hopeful >> budget >> near_ok >> tunings >> counts) {
     xt_ctx* ctx = new xt_ctx();
     ctx->num_sms = 152;
     ctx->smem_optin = 227 * 1024;
@@ -38,7 +38,7 @@ int main() {
     bool lane_ok[kNumJ];
     batched_flags(ctx, sc, (int32_t)n, &jf, lane_ok);
     Plan pl;
-    plan_counts(ctx, sc, cnt, (int32_t)hopeful, jf, lane_ok, &pl);
+    plan_counts(ctx, sc, cnt, (int32_t)hopeful, near_ok != 0, jf, lane_ok, &pl);
     const size_t pool = layout_pool(ctx, &pl);
     std::printf("{\"bad\": %d, \"near_pairs\": %d, \"near_grid\": %d, \"signature\": \"%016llx\", "
                 "\"pool\": %zu, \"max_launches\": %d, \"launches\": [",

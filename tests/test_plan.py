@@ -27,7 +27,7 @@ def plan(tmp_path_factory):
             sc, counts, tuned = c.get("sc", ScoringParams()), c["counts"], c.get("tuned", ())
             n = c.get("n", sum(counts.values()))
             text.append(f"{sc.w} {sc.match} {sc.mismatch} {sc.gap_open} {sc.gap_extend} {sc.zdrop} "
-                        f"{sc.n_score} {n} {c.get('hopeful', 0)} {c.get('budget', 0)} {len(tuned)} "
+                        f"{sc.n_score} {n} {c.get('hopeful', 0)} {c.get('budget', 0)} {int(c.get('near_ok', True))} {len(tuned)} "
                         f"{len(counts)}")
             text += [" ".join(map(str, t)) for t in tuned]
             text += [f"{cls} {j} {v}" for (cls, j), v in counts.items()]
@@ -137,3 +137,15 @@ def test_what_a_narrow_band_leaves_gets_the_engines_narrow_pairs_take(plan):
     # no rings beyond the budget
     assert [L["engine"] for L in tight["launches"]] == ["band", "group"]
     assert tight["launches"][1]["gate"] == 0 and tight["pool"] <= 64 << 20
+
+
+def test_without_a_buffer_for_what_near_passes_leave(plan):
+    plans = plan([
+        {"counts": {(NEAR, 8): 50_000, (NEAR, 7): 60_000}, "hopeful": 62_000, "n": 400_000, "near_ok": False},
+        {"sc": ScoringParams(w=600), "counts": {(BAND, 11): 3000, (BAND, 14): 200}, "near_ok": False},
+        {"sc": ScoringParams(w=9000), "counts": {(BAND, 14): 300}, "near_ok": False}])
+    for p in plans:
+        assert not p["bad"] and p["near_pairs"] == 0
+        assert not any(L["near_hw"] or L["after_prev"] or L["gate"] for L in p["launches"])
+    assert plans[1]["launches"][0]["j_hi"] == 14 and plans[1]["launches"][-1]["j_lo"] == 11
+    assert plans[2]["launches"][0]["global_ring"]
