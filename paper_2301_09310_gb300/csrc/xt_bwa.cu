@@ -110,9 +110,11 @@ struct BwaArgs {
   int64_t* cells;
   BwaScore sc;
   int mshift;        // 2^mshift > match
+  int coarse;        // 2^coarse neighbouring length buckets of a class in one slot
   uint8_t* pclass;   // [n]
   int32_t* order;    // [n] pairs by class, then by query length (longest first)
-  int32_t* slots;    // [kBwaClasses * kBwaLenBuckets] pairs per (class, length), then positions
+  int32_t* slots;    // [kBwaClasses * (kBwaLenBuckets >> coarse)] pairs per (class, length), then
+                     // positions
   int32_t* counts;   // [kBwaClasses] pairs per class
   int32_t* heads;    // [kBwaClasses] next pair of each class's persistent kernel
 };
@@ -120,10 +122,10 @@ struct BwaArgs {
 // Slot of a pair of class c, query length ql and seed score h0: classes in order,
 // longer queries first within a class; with two pairs per lane, whose warps sweep
 // the columns alive in any of 64 pairs, pairs of like seed scores together.
-__device__ __forceinline__ int32_t bwa_slot(int c, int32_t ql, int32_t h0) {
+__device__ __forceinline__ int32_t bwa_slot(int c, int32_t ql, int32_t h0, int coarse) {
   const int32_t key = !bwa_is_lane(c) ? ql : 4 * (ql - 1) + min(h0 >> 4, 3);
   const int32_t b = key < kBwaLenBuckets - 1 ? key : kBwaLenBuckets - 1;
-  return c * kBwaLenBuckets + (kBwaLenBuckets - 1 - b);
+  return (c * kBwaLenBuckets + (kBwaLenBuckets - 1 - b)) >> coarse;
 }
 
 // The narrowed band half-width of a pair with query length qlen.
@@ -188,7 +190,7 @@ __global__ void k_bwa_classify(BwaArgs a) {
         c = bwa_group_id(c);
       }
       cls = (uint8_t)c;
-      atomicAdd(&a.slots[bwa_slot(cls, ql, h0)], 1);
+      atomicAdd(&a.slots[bwa_slot(cls, ql, h0, a.coarse)], 1);
     }
     a.pclass[k] = cls;
   }
@@ -198,7 +200,8 @@ __global__ void k_bwa_classify(BwaArgs a) {
 // and the pairs per class.
 __global__ void __launch_bounds__(kBwaScanThreads) k_bwa_scan(BwaArgs a) {
   constexpr int kPer = kBwaClasses * kBwaLenBuckets / kBwaScanThreads;
-  constexpr int kPerClass = kBwaLenBuckets / kPer;  // threads per class
+  constexpr int kPerClass = kBwaLenBuckets / kPer;  // threads per class (of coarse slots too)
+  const int per = kPer >> a.coarse;
   __shared__ int32_t s_warp[kBwaScanThreads / 32];
   __shared__ int32_t s_class[kBwaClasses];
   const int tid = threadIdx.x;
@@ -206,7 +209,7 @@ __global__ void __launch_bounds__(kBwaScanThreads) k_bwa_scan(BwaArgs a) {
   int32_t sum = 0;
 #pragma unroll
   for (int u = 0; u < kPer; ++u) {
-    v[u] = a.slots[tid * kPer + u];
+    v[u] = u < per ? a.slots[tid * per + u] : 0;
     sum += v[u];
   }
   if (tid < kBwaClasses) s_class[tid] = 0;
@@ -224,7 +227,7 @@ __global__ void __launch_bounds__(kBwaScanThreads) k_bwa_scan(BwaArgs a) {
   atomicAdd(&s_class[tid / kPerClass], sum);
 #pragma unroll
   for (int u = 0; u < kPer; ++u) {
-    a.slots[tid * kPer + u] = before;
+    if (u < per) a.slots[tid * per + u] = before;
     before += v[u];
   }
   __syncthreads();
@@ -237,7 +240,7 @@ __global__ void k_bwa_scatter(BwaArgs a) {
        k += (int64_t)gridDim.x * blockDim.x) {
     const int c = a.pclass[k];
     if (c == kBwaDone) continue;
-    const int32_t pos = atomicAdd(&a.slots[bwa_slot(c, a.q_len[k], a.h0[k])], 1);
+    const int32_t pos = atomicAdd(&a.slots[bwa_slot(c, a.q_len[k], a.h0[k], a.coarse)], 1);
     if (pos >= 0 && pos < a.n) a.order[pos] = (int32_t)k;
   }
 }
@@ -1013,12 +1016,22 @@ extern "C" xt_status xt_extend_batch_bwa(xt_ctx* ctx, const uint8_t* q_seq, int6
   const size_t o_cls = 0;
   const size_t o_order = align256(o_cls + n);
   const size_t o_slots = align256(o_order + 4 * n);
-  const size_t n_ctr = (size_t)kBwaClasses * kBwaLenBuckets + 2 * kBwaClasses;
-  const size_t bytes = align256(o_slots + 4 * n_ctr);
-  s = ctx_alloc(ctx, &ctx->bwa_ws, &ctx->bwa_ws_bytes, bytes);
+  // (half as many slots where a budget does not hold them all: lengths in pairs)
+  BwaArgs a;
+  a.coarse = 0;
+  size_t n_ctr = 0;
+  for (int coarse = 0; coarse < 2; ++coarse) {
+    const std::string last_error = ctx->last_error;
+    a.coarse = coarse;
+    n_ctr = (size_t)kBwaClasses * (kBwaLenBuckets >> coarse) + 2 * kBwaClasses;
+    s = ctx_alloc(ctx, &ctx->bwa_ws, &ctx->bwa_ws_bytes, align256(o_slots + 4 * n_ctr));
+    if (s == XT_OK) {
+      ctx->last_error = last_error;
+      break;
+    }
+  }
   if (s != XT_OK) return s;
   char* ws = static_cast<char*>(ctx->bwa_ws);
-  BwaArgs a;
   a.q_seq = q_seq; a.t_seq = t_seq; a.q_off = q_off; a.t_off = t_off; a.q_len = q_len;
   a.t_len = t_len; a.h0 = h0; a.q_bytes = q_bytes; a.t_bytes = t_bytes; a.n = n_pairs;
   a.out = out; a.cells = cells_out;
@@ -1033,7 +1046,7 @@ extern "C" xt_status xt_extend_batch_bwa(xt_ctx* ctx, const uint8_t* q_seq, int6
   a.pclass = reinterpret_cast<uint8_t*>(ws + o_cls);
   a.order = reinterpret_cast<int32_t*>(ws + o_order);
   a.slots = reinterpret_cast<int32_t*>(ws + o_slots);
-  a.counts = a.slots + kBwaClasses * kBwaLenBuckets;
+  a.counts = a.slots + kBwaClasses * (kBwaLenBuckets >> a.coarse);
   a.heads = a.counts + kBwaClasses;
   const int threads = 256;
   const int grid = (int)std::min<int64_t>(((int64_t)n_pairs + threads - 1) / threads,
