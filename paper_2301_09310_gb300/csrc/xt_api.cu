@@ -191,11 +191,14 @@ xt_status get_work(xt_ctx* ctx, int32_t n, Work* w, Batch** desc) {
 // The buffer of the pairs the near passes leave, for calls of n pairs; false where the
 // budget or the device does not hold it.
 bool get_near(xt_ctx* ctx, int32_t n, Work* w) {
-  void* old = ctx->near_buf;
-  const std::string last_error = ctx->last_error;
-  const bool ok = dev_alloc(ctx, &ctx->near_buf, &ctx->near_bytes, 4 * (size_t)n) == XT_OK;
-  if (ctx->near_buf != old) drop_graphs(ctx);
-  if (!ok) ctx->last_error = last_error;
+  bool ok = ctx->near_bytes >= 4 * (size_t)n;
+  if (!ok) {
+    void* old = ctx->near_buf;
+    const std::string last_error = ctx->last_error;
+    ok = dev_alloc(ctx, &ctx->near_buf, &ctx->near_bytes, 4 * (size_t)n) == XT_OK;
+    if (ctx->near_buf != old) drop_graphs(ctx);
+    if (!ok) ctx->last_error = last_error;
+  }
   w->near_tmp = ok ? (int32_t*)ctx->near_buf : nullptr;
   return ok;
 }
@@ -1125,7 +1128,7 @@ xt_status run_finish(xt_ctx* ctx) {
       int32_t cnt[kNumClasses][kNumJ];
       for (int c = 0; c < kNumClasses; ++c)
         for (int j = 0; j < kNumJ; ++j) cnt[c][j] = se[c * kNumJ + j] - sb[c * kNumJ + j];
-      pl = Plan();
+      if (pl.n_launch > 0) pl = Plan();
       plan_counts(ctx, sc, cnt, hopeful, near_ok, pc.jf, pc.lane_ok, &pl);
     };
     plan(true);

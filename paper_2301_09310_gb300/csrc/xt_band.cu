@@ -567,7 +567,9 @@ bool band_near_shape(const Score& sc, int32_t match, int j, int* P, int* K, int*
 int band_grid(int P, int K, int32_t pairs, int num_sms) {
   const int64_t per_cta = 2 * (int64_t)kBandThreads / P;
   const int64_t want = ((int64_t)pairs + per_cta - 1) / per_cta;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms * band_blocks(K)));
+  int64_t grid = 1;  // calls of like size share a graph
+  while (grid < want) grid *= 2;
+  return (int)std::min<int64_t>(grid, (int64_t)num_sms * band_blocks(K));
 }
 
 cudaError_t launch_band(const Batch* bd, const Score& sc, int32_t match, const Work& w,

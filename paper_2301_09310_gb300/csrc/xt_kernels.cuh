@@ -135,6 +135,10 @@ cudaError_t launch_diag(const Batch* bd, int32_t n_cap, const Score& sc, int32_t
                         const Work& w, cudaStream_t stream);
 // The NEAR class on its narrow band; its segment table and queue region then
 // hold the pairs left, longest first.
+// (Grids are rounded up, so that calls of like size share a graph; a CTA without a
+// pair ends at once.  Four sizes an octave here: the pairs spread over the CTAs there
+// are, and wider apart they leave the launches beside them less room, 55k streamed
+// pairs 1,068 -> 1,084 us with 128 CTAs for 82.)
 int near_grid(int32_t pairs, int num_sms);
 cudaError_t launch_near(const Batch* bd, const Score& sc, int32_t match, int grid, const Work& w,
                         int head_id, cudaStream_t stream);

@@ -149,3 +149,28 @@ def test_without_a_buffer_for_what_near_passes_leave(plan):
         assert not any(L["near_hw"] or L["after_prev"] or L["gate"] for L in p["launches"])
     assert plans[1]["launches"][0]["j_hi"] == 14 and plans[1]["launches"][-1]["j_lo"] == 11
     assert plans[2]["launches"][0]["global_ring"]
+
+
+@pytest.mark.parametrize("name,mean,sc", [
+    ("mixed reads", {(NEAR, 8): 3200, (NEAR, 7): 8200, (PACKED, 7): 1300, (PACKED, 6): 2900, (PACKED, 5): 1200},
+     ScoringParams()),
+    ("mixed reads", {(NEAR, 8): 64_000, (NEAR, 7): 148_000, (PACKED, 7): 21_000, (PACKED, 6): 50_000,
+                     (PACKED, 5): 22_000}, ScoringParams()),
+    ("small calls", {(NEAR, 8): 70, (NEAR, 7): 190, (PACKED, 6): 70, (PACKED, 5): 31}, ScoringParams()),
+    ("stream", {(BAND, 11): 1100, (BAND, 10): 3600, (PACKED, 9): 1500, (NEAR, 9): 6900, (NEAR, 8): 10_100,
+                (NEAR, 7): 5300, (PACKED, 7): 600, (PACKED, 6): 1300, (PACKED, 5): 1150}, ScoringParams()),
+    ("wide bands", {(BAND, 11): 1100, (BAND, 10): 3600, (NEAR, 8): 10_100, (PACKED, 6): 1300},
+     ScoringParams(w=600)),
+])
+def test_calls_of_like_size_share_a_plan(plan, name, mean, sc):
+    # batches of up to 7% fewer pairs than one, as a stream of reads forms them
+    import random
+    rng = random.Random(11)
+    cases = []
+    for _ in range(200):
+        size = rng.uniform(0.93, 1.0)
+        counts = {k: max(1, round(rng.gauss(v * size, (v * size) ** 0.5))) for k, v in mean.items()}
+        near = sum(v for (cls, _), v in counts.items() if cls == NEAR)
+        cases.append({"sc": sc, "counts": counts, "n": 1 << 16, "hopeful": round(near * 0.56)})
+    signatures = {p["signature"] for p in plan(cases)}
+    assert len(signatures) <= 8, len(signatures)
