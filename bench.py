@@ -539,7 +539,7 @@ def run_xt(args):
         "gpu_launches": launches,
         "roofline": dict(roof, **{
             "traffic": traffic,
-            "kernel": "extension DP launches of one step (k_near, k_lane, k_band, k_queue)",
+            "kernel": "extension DP launches of one step (k_diag, k_near, k_lane, k_band, k_queue)",
             "kernel_ms_per_step": round(dp_ms, 4),
             "cell_updates_per_step": updates_step,
             "ops_per_update": {"alu_pipe": ALU_OPS_PER_UPDATE, "mad_pipe": MAD_OPS_PER_UPDATE,

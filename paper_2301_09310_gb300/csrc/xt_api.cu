@@ -895,12 +895,25 @@ xt_status check_args(xt_ctx* ctx, const void* q_seq, int64_t q_bytes, const void
   return XT_OK;
 }
 
+// One of a pair of timing events, created on first use.
+void record_timed(cudaEvent_t (&ev)[2], int which, cudaStream_t stream) {
+  if (!ev[which]) cudaEventCreate(&ev[which]);
+  cudaEventRecord(ev[which], stream);
+}
+
 // The front of a call: classify, order the queue (launch_store_desc ran before
 // and reset the counters).
-cudaError_t enqueue_front(const JFlags& jf, const Score& sc, int32_t match, bool diag, bool near,
-                          const Work& w, const Batch* desc, int32_t n_cap, cudaStream_t stream) {
+cudaError_t enqueue_front(xt_ctx* ctx, const JFlags& jf, const Score& sc, int32_t match, bool diag,
+                          bool near, const Work& w, const Batch* desc, int32_t n_cap,
+                          cudaStream_t stream) {
   cudaError_t e = cudaSuccess;
+  // the diagonal pass extends pairs: a timed call's time takes it in
+  const int slot = ctx->ev_pending;
+  const bool timed = ctx->timing && slot < xt_ctx::kEvRing;
+  if (slot < xt_ctx::kEvRing) ctx->diag_timed[slot] = timed && diag;
+  if (timed && diag) record_timed(ctx->diag_ev[slot], 0, stream);
   if (diag) e = launch_diag(desc, n_cap, sc, match, near, w, stream);
+  if (timed && diag) record_timed(ctx->diag_ev[slot], 1, stream);
   if (e == cudaSuccess) e = launch_classify(desc, n_cap, sc, match, jf, diag, w, stream);
   if (e == cudaSuccess) e = launch_order(desc, n_cap, w, stream);
   return e;
@@ -913,11 +926,7 @@ cudaError_t enqueue_dp(xt_ctx* ctx, bool plain, const Plan& pl, int plain_rs, co
   cudaError_t e = cudaSuccess;
   const int slot = ctx->ev_pending;
   const bool timed = ctx->timing && slot < xt_ctx::kEvRing;
-  if (timed) {
-    for (int k = 0; k < 2; ++k)
-      if (!ctx->ev[slot][k]) cudaEventCreate(&ctx->ev[slot][k]);
-    cudaEventRecord(ctx->ev[slot][0], stream);
-  }
+  if (timed) record_timed(ctx->ev[slot], 0, stream);
   int dp = 0;
   if (e == cudaSuccess && plain) {
     e = launch_plain(desc, n_cap, sc, w, plain_rs, stream);
@@ -968,7 +977,7 @@ cudaError_t enqueue_dp(xt_ctx* ctx, bool plain, const Plan& pl, int plain_rs, co
   const cudaError_t joined = fork.join();
   if (e == cudaSuccess) e = joined;
   if (e == cudaSuccess && timed) {
-    cudaEventRecord(ctx->ev[slot][1], stream);
+    record_timed(ctx->ev[slot], 1, stream);
     ctx->ev_pending = slot + 1;
   }
   *dp_out = dp;
@@ -1058,7 +1067,7 @@ xt_status run_begin(xt_ctx* ctx, bool plain, bool early, const uint8_t* q_seq, i
     const bool diag = pc.diag = ctx->near_first && !early && n >= kNearMinPairs && !ctx->forced_P &&
                       pc.sc.alpha >= 1;
     const bool near = diag && pc.sc.alpha <= 127 && pc.sc.beta >= 1 && pc.sc.w >= kNearHalf;
-    e = enqueue_front(pc.jf, pc.sc, scr->match, diag, near, pc.w, pc.desc, pc.n_cap, stream);
+    e = enqueue_front(ctx, pc.jf, pc.sc, scr->match, diag, near, pc.w, pc.desc, pc.n_cap, stream);
     const size_t seg_bytes =
         (size_t)((const char*)(pc.w.near_hope + 1) - (const char*)pc.w.seg_begin);
     if (e == cudaSuccess)
@@ -1150,7 +1159,7 @@ xt_status run_finish(xt_ctx* ctx) {
   // replay as one graph once a call with the same key has been seen
   auto body = [&](cudaStream_t st, int* dp) -> cudaError_t {
     cudaError_t r = cudaSuccess;
-    if (plain) r = enqueue_front(pl.jf, sc, pc.scr.match, false, false, w, pc.desc, pc.n_cap, st);
+    if (plain) r = enqueue_front(ctx, pl.jf, sc, pc.scr.match, false, false, w, pc.desc, pc.n_cap, st);
     if (r == cudaSuccess) r = enqueue_dp(ctx, plain, pl, plain_rs, sc, w, pc.desc, pc.n_cap, st, dp);
     return r;
   };
@@ -1207,8 +1216,9 @@ xt_status run_finish(xt_ctx* ctx) {
     if (e != cudaSuccess) return cuda_fail(ctx, e, ("launch " + ctx->launch_error).c_str());
   }
   ctx->calls += 1;
-  // descriptor, (diagonals,) classify, scan, scatter + DP kernels
-  ctx->launches += 4 + (pc.diag ? 1 : 0) + dp;
+  // descriptor, classify, scan, scatter + DP kernels (the diagonal pass among them)
+  if (pc.diag) ++dp;
+  ctx->launches += 4 + dp;
   ctx->dp_launches += dp;
   return XT_OK;
 }
@@ -1291,9 +1301,10 @@ xt_status xt_ctx_destroy(xt_ctx* ctx) {
   if (ctx->seed_ws) cudaFree(ctx->seed_ws);
   if (ctx->seed_rev) cudaFree(ctx->seed_rev);
   if (ctx->bwa_ws) cudaFree(ctx->bwa_ws);
-  for (auto& pr : ctx->ev)
-    for (auto& e : pr)
-      if (e) cudaEventDestroy(e);
+  for (auto* ring : {ctx->ev, ctx->diag_ev})
+    for (int k = 0; k < xt_ctx::kEvRing; ++k)
+      for (auto& e : ring[k])
+        if (e) cudaEventDestroy(e);
   drop_graphs(ctx);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
   if (ctx->seg_host) cudaFreeHost(ctx->seg_host);
@@ -1803,6 +1814,11 @@ xt_status xt_ctx_stats(xt_ctx* ctx, xt_stats* out) {
     if (e == cudaSuccess) e = cudaEventElapsedTime(&t, ctx->ev[i][0], ctx->ev[i][1]);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "event timing");
     ms += t;
+    if (ctx->diag_timed[i]) {
+      e = cudaEventElapsedTime(&t, ctx->diag_ev[i][0], ctx->diag_ev[i][1]);
+      if (e != cudaSuccess) return cuda_fail(ctx, e, "event timing");
+      ms += t;
+    }
   }
   for (auto* c : ctx->chunk_ctx)
     if (c) {

@@ -160,6 +160,8 @@ struct xt_ctx {
   bool timing = false;
   static constexpr int kEvRing = 256;
   cudaEvent_t ev[kEvRing][2] = {};
+  cudaEvent_t diag_ev[kEvRing][2] = {};  // around a timed call's diagonal pass,
+  bool diag_timed[kEvRing] = {};         // where it has one
   int ev_pending = 0;
   int calls = 0, launches = 0, dp_launches = 0;
   // per-call batch descriptor: pinned host slots copied to a device slot
