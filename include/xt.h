@@ -293,7 +293,10 @@ xt_status xt_ctx_get_bucket_schedule_for(xt_ctx* ctx, int w, int j, int batch_cl
  * Autotuner.  For every bucket j = 5..j_max, times each available (P, R) on
  * synthetic pairs of that bucket's lengths (each query a mutated copy of its
  * target, so pairs extend over the full band) with the scoring `sc`, and
- * keeps the fastest as the bucket's schedule for sc->w on this context.  A
+ * keeps the fastest as the bucket's schedule for sc->w on this context.  The
+ * band engine, which the built-in rule uses too, is timed beside them (it has
+ * no (P, R)): where it is faster, the bucket's pairs it takes run on it, and the
+ * schedule kept is for the others.  A
  * trial batch holds enough pairs to fill the GPU four times over with the
  * one-lane engine (throughput at saturation), but at most about
  * cells_per_trial useful cells (0 = 3e10); for long queries, where that

@@ -233,11 +233,16 @@ const BucketSched* tuned(const xt_ctx* ctx, int w, int j) {
   return nullptr;
 }
 
-// Whether bucket j has a tuned schedule for band w in either size class.
-bool tuned_any(const xt_ctx* ctx, int w, int j) {
-  for (const auto& t : ctx->tuning)
-    if (t.w == w && (t.small[j].P > 0 || t.b[j].P > 0)) return true;
-  return false;
+// Whether bucket j's schedules for band w leave pairs to the band engine in either
+// size class (the class of a pair must not depend on its bucket's count).
+bool band_left_to(const xt_ctx* ctx, int w, int j) {
+  bool any = false;
+  for (const auto& t : ctx->tuning) {
+    if (t.w != w) continue;
+    if (t.small[j].band || t.b[j].band) return true;
+    any |= t.small[j].P > 0 || t.b[j].P > 0;
+  }
+  return !any;
 }
 
 // Ring entries (log2) of a group-engine pair of bucket j under band w.
@@ -443,8 +448,8 @@ void batched_flags(xt_ctx* ctx, const Score& sc, int32_t n, JFlags* jf, bool* la
   *jf = JFlags{};
   for (int j = 0; j < kNumJ; ++j) lane_ok[j] = false;
   int bP, bK, bhw;
-  const bool may_band = ctx->near_first && !ctx->forced_P;
-  const bool band = may_band && band_shape(sc, ctx->match, 0, &bP, &bK);
+  const bool band = !ctx->forced_P && band_shape(sc, ctx->match, 0, &bP, &bK);
+  const bool narrow = !ctx->forced_P && ctx->near_first && !band;
   const bool saved = ctx->plan_small;
   for (int j = kJMin; j <= kJMax; ++j) {
     Launch L;
@@ -457,14 +462,14 @@ void batched_flags(xt_ctx* ctx, const Score& sc, int32_t n, JFlags* jf, bool* la
         const BucketSched* t = tuned(ctx, sc.w, j);
         // untuned buckets of any length may take the one-lane engine where
         // its ring fits (the count decides later)
-        want |= t ? t->P == 1 : bucket_sched_ok(ctx, sc.w, j, 1, lane_default_R(j));
+        want |= t && !t->band ? t->P == 1 : bucket_sched_ok(ctx, sc.w, j, 1, lane_default_R(j));
       }
       ctx->plan_small = false;
     }
     lane_ok[j] = want && lane_launch(ctx, sc, CLS_PACKED, j, true, &L) &&
                  lane_launch(ctx, sc, CLS_NARROW, j, true, &L);
-    const bool banded = may_band && !tuned_any(ctx, sc.w, j) &&
-                        (band || band_near_shape(sc, ctx->match, j, &bP, &bK, &bhw));
+    const bool banded = (band || (narrow && band_near_shape(sc, ctx->match, j, &bP, &bK, &bhw))) &&
+                        band_left_to(ctx, sc.w, j);
     if (banded) jf->f[j] |= kJBand;
     if (lane_ok[j])
       jf->f[j] |= kJPacked |
@@ -507,7 +512,7 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
   pl->jf = jf;
   // the band engine, where it holds the band
   int bP = 0, bK = 0;
-  const bool band_ok = ctx->near_first && !ctx->forced_P && band_shape(sc, ctx->match, 0, &bP, &bK);
+  const bool band_ok = !ctx->forced_P && band_shape(sc, ctx->match, 0, &bP, &bK);
   // long queries: one lane per pair needs many pairs to fill the GPU, but
   // the long buckets of one call run side by side, so when together they
   // hold two full waves of lanes each of them takes the one-lane engine
@@ -615,7 +620,8 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
       // BAND pairs the band engine does not hold: a narrow band first, then the engine
       // NARROW pairs would take, for those it leaves
       const bool narrow_first = cls == CLS_BAND && !band_ok;
-      if (cls == CLS_BAND && band_ok) {
+      const BucketSched* const ts = tuned(ctx, sc.w, jj);
+      if (band_ok && (cls == CLS_BAND ? !ts || ts->band : ts && ts->band && cls != CLS_WIDE && cls != CLS_NARROW)) {
         band = true;
       } else if (cls != CLS_WIDE && lane_ok[jj]) {
         lane = true;
@@ -680,7 +686,7 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
       // (so do a few pairs of up to 254 bases under a band of more diagonals than one
       // warp holds at 8 a lane: 1,000 pairs of 250 bases, w = 250, 266 and 169 us)
       const bool few_wide = jj == kGroupMaxJ + 1 && c < kBucketSmall / 4 && 2 * (int64_t)sc.w + 1 > 256;
-      if (!lane && band_ok && packed_class(cls) && !tuned(ctx, sc.w, jj) && jj > kGroupMaxJ && !few_wide)
+      if (!lane && band_ok && packed_class(cls) && !ts && jj > kGroupMaxJ && !few_wide)
         band = true;
       if (band) {
         band_shape(sc, ctx->match, c, &L.P, &L.R);
@@ -846,6 +852,13 @@ xt_status xt::ctx_reserve(xt_ctx* ctx, int32_t n_pairs, size_t conv_bytes, size_
     if (ctx->pool != old) drop_graphs(ctx);
   }
   return s;
+}
+
+bool xt::band_engine_ok(const xt_scoring* sc, int w) {
+  Score s = make_score(sc);
+  s.w = w;
+  int P, K;
+  return band_shape(s, sc->match, 0, &P, &K);
 }
 
 bool xt::bucket_sched_ok(const xt_ctx* ctx, int w, int j, int P, int R) {
@@ -1755,6 +1768,7 @@ xt_status xt_ctx_set_bucket_schedule_for(xt_ctx* ctx, int w, int j, int batch_cl
   BucketSched& b = batch_class == XT_BATCH_SMALL ? e->small[j] : e->b[j];
   b.P = P;
   b.R = P ? R : 0;
+  b.band = false;
   drop_graphs(ctx);
   return XT_OK;
 }

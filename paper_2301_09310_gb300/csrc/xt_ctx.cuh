@@ -34,9 +34,11 @@ struct GraphEntry {
 constexpr int kMaxBranches = 8;  // streams the DP launches of one call fork onto
 
 // Schedule of one length bucket: P lanes per pair (1: the one-lane engine),
-// R rows per lane.  P = 0: the built-in rule.
+// R rows per lane.  P = 0: the built-in rule.  band (autotuner's tables): the band
+// engine was faster, and runs the pairs it takes; the others run by P and R.
 struct BucketSched {
   int P = 0, R = 0;
+  bool band = false;
 };
 // The schedules of every bucket for calls whose band is w: one set for
 // buckets that fill the GPU (tuned at saturation) and one for buckets of
@@ -51,6 +53,8 @@ struct TuneEntry {
 // Whether (P, R) is an instantiated schedule whose ring fits for bucket j
 // under band w on this context's device.
 bool bucket_sched_ok(const struct ::xt_ctx* ctx, int w, int j, int P, int R);
+// Whether the band engine holds band w under a scoring record.
+bool band_engine_ok(const xt_scoring* sc, int w);
 // The context's pinned read-back area (int32 words): the bucket counts of a
 // batched call first, then the small values other calls bring back.
 constexpr int kSegHostWords = 1024;

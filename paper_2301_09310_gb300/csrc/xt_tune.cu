@@ -180,6 +180,7 @@ struct Entry {
     double gcups;
     int Ps, Rs;  // small-batch schedule (0: none)
     double gcups_s;
+    bool band, band_s;  // the band engine was faster (then the rates are its)
   };
   std::vector<B> buckets;
 };
@@ -204,9 +205,11 @@ bool entry_from_json(const Json& e, Entry* out) {
       return false;
     const Json *Ps = b.get("Ps"), *Rs = b.get("Rs"), *gs = b.get("gcups_s");
     const bool small = Ps && Rs && Ps->kind == Json::NUM && Rs->kind == Json::NUM;
+    const Json *bd = b.get("band"), *bds = b.get("band_s");
     out->buckets.push_back({(int)j->num, (int)P->num, (int)R->num, g ? g->num : 0.0,
-                            small ? (int)Ps->num : 0, small ? (int)Rs->num : 0,
-                            gs ? gs->num : 0.0});
+                            small ? (int)Ps->num : 0, small ? (int)Rs->num : 0, gs ? gs->num : 0.0,
+                            bd && bd->kind == Json::NUM && bd->num != 0,
+                            small && bds && bds->kind == Json::NUM && bds->num != 0});
   }
   return true;
 }
@@ -222,8 +225,9 @@ std::string entry_to_json(const Entry& e) {
     const auto& b = e.buckets[k];
     std::snprintf(buf, sizeof(buf),
                   "%s\n       {\"j\": %d, \"P\": %d, \"R\": %d, \"gcups\": %.3f, "
-                  "\"Ps\": %d, \"Rs\": %d, \"gcups_s\": %.3f}",
-                  k ? "," : "", b.j, b.P, b.R, b.gcups, b.Ps, b.Rs, b.gcups_s);
+                  "\"Ps\": %d, \"Rs\": %d, \"gcups_s\": %.3f, \"band\": %d, \"band_s\": %d}",
+                  k ? "," : "", b.j, b.P, b.R, b.gcups, b.Ps, b.Rs, b.gcups_s, (int)b.band,
+                  (int)b.band_s);
     s += buf;
   }
   return s + "]}";
@@ -342,14 +346,16 @@ cudaError_t upload(const HostPairs& hp, DevPairs* d) {
   return e;
 }
 
-// Candidate schedules in the order they are tried.
-std::vector<BucketSched> candidates(const xt_ctx* ctx, int w, int j) {
+// Candidate schedules in the order they are tried: lanes and groups, then the band
+// engine where it holds the band (for the pairs it takes; the others by the first).
+std::vector<BucketSched> candidates(const xt_ctx* ctx, const xt_scoring* sc, int w, int j) {
   static const int kCand[][2] = {{1, 8}, {1, 4}, {1, 16}, {2, 8}, {2, 4}, {2, 16}, {4, 8},
                                  {4, 4}, {4, 16}, {8, 8}, {8, 4}, {16, 8}, {16, 4}, {32, 8},
                                  {32, 4}};
   std::vector<BucketSched> v;
   for (auto& c : kCand)
     if (bucket_sched_ok(ctx, w, j, c[0], c[1])) v.push_back({c[0], c[1]});
+  if (!v.empty() && band_engine_ok(sc, w)) v.push_back({v[0].P, v[0].R, true});
   return v;
 }
 
@@ -375,7 +381,7 @@ void set_sched(xt_ctx* ctx, int w, int j, BucketSched s, bool small) {
 constexpr int kSmallTrialPairs = 2048;
 
 struct Trial {
-  BucketSched best{};
+  BucketSched best{};  // of lanes and groups; with band where the band engine is faster
   double gcups = -1;
 };
 
@@ -446,7 +452,8 @@ xt_status tune_bucket(xt_ctx* ctx, const xt_scoring* sc, int w, int j, int n,
     const double gcups = (double)total / (ms / reps * 1e-3) / 1e9;
     if (gcups > tr->gcups) {
       tr->gcups = gcups;
-      tr->best = cand[c];
+      if (cand[c].band) tr->best.band = true;
+      else tr->best = cand[c];
     }
   }
   cudaEventDestroy(e0);
@@ -505,7 +512,7 @@ xt_status xt_autotune(xt_ctx* ctx, const xt_scoring* sc, int j_max, double cells
     std::vector<BucketSched> cand;
     {
       std::lock_guard<std::mutex> lk(ctx->mu);
-      cand = candidates(ctx, w, j);
+      cand = candidates(ctx, sc, w, j);
     }
     if (cand.empty()) continue;
     // large calls: a trial fills the GPU, four pairs per one-lane thread slot
@@ -527,7 +534,7 @@ xt_status xt_autotune(xt_ctx* ctx, const xt_scoring* sc, int j_max, double cells
       n = (int)wave;
       big_cand.clear();
       for (auto& c : cand)
-        if ((c.P == 1 && c.R >= 8) || (c.P >= 16 && c.R == 8)) big_cand.push_back(c);
+        if (c.band || (c.P == 1 && c.R >= 8) || (c.P >= 16 && c.R == 8)) big_cand.push_back(c);
       big_reps = 1;
     }
     Trial big;
@@ -548,7 +555,7 @@ xt_status xt_autotune(xt_ctx* ctx, const xt_scoring* sc, int j_max, double cells
       set_sched(ctx, w, j, little.best, true);
     }
     entry.buckets.push_back({j, big.best.P, big.best.R, big.gcups, little.best.P, little.best.R,
-                             little.gcups});
+                             little.gcups, big.best.band, little.best.band});
   }
   {
     std::lock_guard<std::mutex> lk(ctx->mu);
@@ -585,9 +592,10 @@ xt_status xt_ctx_load_tuning(xt_ctx* ctx, const char* table_path) {
     if (e.device != dev || e.sms != ctx->num_sms || e.w < 0) continue;
     for (const auto& b : e.buckets) {
       if (b.j < kJMin || b.j > kJMax) continue;
-      if (bucket_sched_ok(ctx, e.w, b.j, b.P, b.R)) set_sched(ctx, e.w, b.j, {b.P, b.R}, false);
+      if (bucket_sched_ok(ctx, e.w, b.j, b.P, b.R))
+        set_sched(ctx, e.w, b.j, {b.P, b.R, b.band}, false);
       if (b.Ps > 0 && bucket_sched_ok(ctx, e.w, b.j, b.Ps, b.Rs))
-        set_sched(ctx, e.w, b.j, {b.Ps, b.Rs}, true);
+        set_sched(ctx, e.w, b.j, {b.Ps, b.Rs, b.band_s}, true);
     }
   }
   return XT_OK;
