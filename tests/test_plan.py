@@ -174,3 +174,16 @@ def test_calls_of_like_size_share_a_plan(plan, name, mean, sc):
         cases.append({"sc": sc, "counts": counts, "n": 1 << 16, "hopeful": round(near * 0.56)})
     signatures = {p["signature"] for p in plan(cases)}
     assert len(signatures) <= 8, len(signatures)
+
+
+def test_band_shapes_by_band_and_count(plan):
+    from tests.band_shapes import KEY_EDGES, SHAPES
+    plans = plan([{"sc": ScoringParams(w=w), "counts": {(BAND, 10): n}} for w, n, _, _ in SHAPES])
+    for (w, n, P, K), p in zip(SHAPES, plans):
+        (L,) = p["launches"]
+        assert (L["engine"], L["P"], L["R"]) == ("band", P, K), (w, n)
+    # where they do not fit: no band pairs, or a narrower band first
+    for (sc, n, fits), p in zip(KEY_EDGES, plan([{"sc": sc, "counts": {(BAND, 10): n}}
+                                                 for sc, n, _ in KEY_EDGES])):
+        whole = p["flags"][10] & 16 and p["launches"][0]["near_hw"] == 0
+        assert bool(whole) == fits, sc
