@@ -85,6 +85,10 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
   const int p = lane % P;
   const int32_t begin = w.seg_begin[cls * kNumJ + j_hi];
   const int32_t end = w.seg_end[cls * kNumJ + j_lo];
+  // the grid is rounded up: the CTAs that hold no pair are the last ones
+  constexpr int kPerCta = 2 * kBandThreads / P;
+  const int ctas = min((int)gridDim.x, (end - begin + kPerCta - 1) / kPerCta);
+  if ((int)blockIdx.x >= ctas) return;
   int32_t* head = w.heads + head_id;
   const int32_t alpha = sc.alpha, beta = sc.beta;
   const int32_t pad = P * K - (2 * hw + 1);    // dead slots before the band's first
@@ -106,13 +110,13 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
   // wave of warps: 9.8 -> 8.2 ms against first come, first served).  Later
   // pairs come from the queue.
   const int row = blockIdx.x / sms, col = blockIdx.x - row * sms;
-  const int cols = min(sms, (int)gridDim.x - row * sms);
+  const int cols = min(sms, ctas - row * sms);
   const int place = row * sms + (row & 1 ? cols - 1 - col : col);
   int32_t next = (place * (kBandThreads / 32) + (int)(threadIdx.x >> 5)) * (2 * kGroups);
   for (bool first = true;; first = false) {
     if (!first) {
       if (lane == 0)
-        next = (int32_t)gridDim.x * (kBandThreads / 32) * (2 * kGroups) +
+        next = ctas * (kBandThreads / 32) * (2 * kGroups) +
                atomicAdd(head, 2 * kGroups);
       next = __shfl_sync(full, next, 0);
     }
@@ -567,9 +571,7 @@ bool band_near_shape(const Score& sc, int32_t match, int j, int* P, int* K, int*
 int band_grid(int P, int K, int32_t pairs, int num_sms) {
   const int64_t per_cta = 2 * (int64_t)kBandThreads / P;
   const int64_t want = ((int64_t)pairs + per_cta - 1) / per_cta;
-  int64_t grid = 1;  // calls of like size share a graph
-  while (grid < want) grid *= 2;
-  return (int)std::min<int64_t>(grid, (int64_t)num_sms * band_blocks(K));
+  return rounded_grid(want, num_sms, band_blocks(K));
 }
 
 cudaError_t launch_band(const Batch* bd, const Score& sc, int32_t match, const Work& w,

@@ -135,11 +135,23 @@ cudaError_t launch_diag(const Batch* bd, int32_t n_cap, const Score& sc, int32_t
                         const Work& w, cudaStream_t stream);
 // The NEAR class on its narrow band; its segment table and queue region then
 // hold the pairs left, longest first.
-// (Grids are rounded up, so that calls of like size share a graph; a CTA without a
-// pair ends at once.  Four sizes an octave here: the pairs spread over the CTAs there
-// are, and wider apart they leave the launches beside them less room, 55k streamed
-// pairs 1,068 -> 1,084 us with 128 CTAs for 82.)
 int near_grid(int32_t pairs, int num_sms);
+// Grids of these passes and of the band engine are rounded up, so that calls of like
+// size share a graph, to four sizes an octave: CTAs without a pair end at once, but
+// many of them cost the launches beside them room (55k streamed pairs 1,068 -> 1,084 us
+// with 128 CTAs of k_near for 82).
+// Nor does the rounding pass a whole number of CTAs per SM: the spare ones would take
+// the place of others (5,000 tables of 180 bases, 286 CTAs of k_band in 304 / 320: 267,
+// 320 us).
+inline int rounded_grid(int64_t want, int num_sms, int per_sm) {
+  if (want < 1) return 0;
+  int64_t step = 1;
+  while (8 * step < want) step *= 2;
+  const int64_t grid = (want + step - 1) / step * step;
+  const int64_t whole = (want + num_sms - 1) / num_sms * num_sms;
+  const int64_t most = (int64_t)num_sms * per_sm;
+  return (int)(grid < whole ? (grid < most ? grid : most) : (whole < most ? whole : most));
+}
 cudaError_t launch_near(const Batch* bd, const Score& sc, int32_t match, int grid, const Work& w,
                         int head_id, cudaStream_t stream);
 cudaError_t launch_order(const Batch* bd, int32_t n_cap, const Work& w, cudaStream_t stream);

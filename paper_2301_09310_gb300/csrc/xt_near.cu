@@ -409,9 +409,7 @@ cudaError_t launch_diag(const Batch* bd, int32_t n_cap, const Score& sc, int32_t
 
 int near_grid(int32_t pairs, int num_sms) {
   const int64_t want = ((int64_t)pairs + 2 * kNearThreads - 1) / (2 * kNearThreads);
-  int64_t step = 1;
-  while (8 * step < want) step *= 2;
-  return (int)std::min<int64_t>((want + step - 1) / step * step, (int64_t)num_sms * kNearBlocks);
+  return rounded_grid(want, num_sms, kNearBlocks);
 }
 
 cudaError_t launch_near(const Batch* bd, const Score& sc, int32_t match, int grid, const Work& w,
