@@ -187,3 +187,13 @@ def test_band_shapes_by_band_and_count(plan):
                                                  for sc, n, _ in KEY_EDGES])):
         whole = p["flags"][10] & 16 and p["launches"][0]["near_hw"] == 0
         assert bool(whole) == fits, sc
+
+
+@pytest.mark.parametrize("w,j,n,lanes", [(255, 8, 60_000, False), (256, 8, 60_000, True), (256, 9, 60_000, True),
+                                         (256, 10, 60_000, False), (400, 8, 30_000, False),
+                                         (191, 7, 60_000, False), (192, 7, 60_000, True)])
+def test_short_queries_under_wide_bands_go_to_lanes(plan, w, j, n, lanes):
+    # scores beyond the packed lanes': one bucket of the band engine's pairs
+    (p,) = plan([{"sc": ScoringParams(5, -4, 8, 2, w, 100, -1), "counts": {(BAND, j): n}, "n": 100_000}])
+    (L,) = p["launches"]
+    assert L["engine"] == ("lane" if lanes else "band")
