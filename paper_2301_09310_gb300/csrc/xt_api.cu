@@ -667,22 +667,20 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
           x.cls = cls; x.j_lo = x.j_hi = j; x.after_prev = after;
           pairs_of[pl->n_launch++] = c;
         };
-        L.band = true;
-        push(L, false);
-        pl->band_near++;
         int P, R, lg;
         const bool huge = group_schedule(cls, jj, c, &P, &R, &lg);
-        Launch g = huge ? huge_launch(ctx, sc, pl) : queue_launch(ctx, cls, jj, P, R, lg);
         // many pairs: lanes if the narrow band leaves a good part of them (but where
         // only global slabs hold the band, those: 40k long reads, w = 1,000, 267 ms, 307)
         const bool or_lanes = lane && !huge;
-        const int32_t many = (int32_t)(next_pow2(c) / 4);
-        g.gate = or_lanes ? -many : 0;
-        push(g, true);
+        L.band = true;
+        L.lanes_from = or_lanes ? (int32_t)(next_pow2(c) / 4) : 0;
+        push(L, false);
+        pl->band_near++;
+        push(huge ? huge_launch(ctx, sc, pl) : queue_launch(ctx, cls, jj, P, R, lg), true);
         if (or_lanes) {
           Launch l;
           lane_launch(ctx, sc, cls, jj, true, &l);
-          l.gate = many;
+          l.lanes_left = true;
           push(l, true);
         }
         prev = -1;
@@ -806,13 +804,13 @@ size_t layout_pool(const xt_ctx* ctx, Plan* pl) {
   };
   // lanes for what a narrow band leaves only as far as the budget holds their rings:
   // the group launch before them takes the pairs else
-  for (int i = 1; i < pl->n_launch;) {
+  for (int i = 2; i < pl->n_launch;) {
     const Launch& L = pl->launch[i];
-    if (L.gate <= 0 || !L.global_ring || allowed(ring_launch_bytes(L))) {
+    if (!L.lanes_left || !L.global_ring || allowed(ring_launch_bytes(L))) {
       ++i;
       continue;
     }
-    pl->launch[i - 1].gate = 0;
+    pl->launch[i - 2].lanes_from = 0;  // narrow band, group, lanes
     for (int k = i; k + 1 < pl->n_launch; ++k) pl->launch[k] = pl->launch[k + 1];
     --pl->n_launch;
   }
@@ -1021,7 +1019,7 @@ uint64_t plan_signature(const Plan& pl) {
   for (int i = 0; i < pl.n_launch; ++i) {
     const Launch& L = pl.launch[i];
     mix(L.cls); mix(L.j_lo); mix(L.j_hi); mix(L.lane); mix(L.band); mix(L.P); mix(L.R); mix(L.rs_log2);
-    mix(L.near_hw); mix(L.cls2); mix(L.after_prev); mix(L.gate); mix(L.global_ring); mix(L.slab); mix(L.grid); mix(L.mparam); mix((int64_t)L.pool_off);
+    mix(L.near_hw); mix(L.cls2); mix(L.after_prev); mix(L.lanes_from); mix(L.lanes_left); mix(L.global_ring); mix(L.slab); mix(L.grid); mix(L.mparam); mix((int64_t)L.pool_off);
   }
   mix(pl.pool_serial);
   mix(pl.near_grid);

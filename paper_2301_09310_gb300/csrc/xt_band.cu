@@ -473,10 +473,12 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
 // length; in the order they were left 55k streamed pairs, w = 600, took 9.0 ms a call, 7.1
 // so).  One block, each thread kPackPer neighbouring places a round; a round's places
 // are read before they are written, and none is written before its own round.
+// lanes_from > 0: so many pairs or more become the segment of those left to lanes.
 constexpr int kPackThreads = 1024;
 constexpr int kPackPer = 8;
 
-__global__ void __launch_bounds__(kPackThreads) k_band_pack(Work w, int cls, int j) {
+__global__ void __launch_bounds__(kPackThreads) k_band_pack(Work w, int cls, int j,
+                                                            int32_t lanes_from) {
   __shared__ int32_t s_warp[kPackThreads / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int32_t begin = w.seg_begin[cls * kNumJ + j], end = w.seg_end[cls * kNumJ + j];
@@ -509,7 +511,14 @@ __global__ void __launch_bounds__(kPackThreads) k_band_pack(Work w, int cls, int
     out += total;
     __syncthreads();
   }
-  if (threadIdx.x == 0) w.seg_end[cls * kNumJ + j] = out;
+  if (threadIdx.x == 0) {
+    const bool lanes = lanes_from > 0 && out - begin >= lanes_from;
+    w.seg_end[cls * kNumJ + j] = lanes ? begin : out;
+    if (lanes_from > 0) {
+      w.seg_begin[kLanesLeftSeg * kNumJ + j] = begin;
+      w.seg_end[kLanesLeftSeg * kNumJ + j] = lanes ? out : begin;
+    }
+  }
 }
 
 // The lane counts and slots compiled: per lane count, fewest slots first.
@@ -584,7 +593,7 @@ cudaError_t launch_band(const Batch* bd, const Score& sc, int32_t match, const W
     k_band<PP, KK, NN><<<L.grid, kBandThreads, 0, stream>>>(                                   \
         bd, sc, w, L.cls, L.j_lo, L.j_hi, head_id, match, 1u << mshift, 1u << kKeyBits, fall,  \
         num_sms, NN ? L.near_hw : sc.w);                                                       \
-    if (NN) k_band_pack<<<1, kPackThreads, 0, stream>>>(w, L.cls, L.j_lo);                           \
+    if (NN) k_band_pack<<<1, kPackThreads, 0, stream>>>(w, L.cls, L.j_lo, L.lanes_from);                           \
     return cudaGetLastError();                                                                 \
   }
   XT_BL(2, 32, false) XT_BL(4, 32, false) XT_BL(8, 26, false) XT_BL(8, 32, false)

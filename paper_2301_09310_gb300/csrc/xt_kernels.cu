@@ -227,15 +227,10 @@ __device__ __forceinline__ void copy_profile(const Score& sc, uint32_t* s_prof) 
   for (int c = 0; c < 5; ++c) s_prof[c] = sc.prof[c];
 }
 
-// Launch::gate.
-__device__ __forceinline__ bool gated_off(int32_t gate, int32_t pairs) {
-  return gate > 0 ? pairs < gate : (gate < 0 && pairs >= -gate);
-}
-
 template <int P, int R, bool WIDE>
 __global__ void __launch_bounds__(kQueueThreads)
     k_queue(const Batch* __restrict__ bd, Score sc, Work w, int cls, int j_lo, int j_hi,
-            int head_id, int rs_log2, int2* gring, int64_t slab, int32_t gate) {
+            int head_id, int rs_log2, int2* gring, int64_t slab) {
   // batch arguments stay in shared memory and are read where used
   __shared__ Batch s_b;
   if (threadIdx.x == 0) s_b = *bd;
@@ -252,7 +247,6 @@ __global__ void __launch_bounds__(kQueueThreads)
   const unsigned gmask = (P == 32) ? 0xffffffffu : (((1u << P) - 1u) << (lane - p));
   const int32_t begin = w.seg_begin[cls * kNumJ + j_hi];
   const int32_t end = w.seg_end[cls * kNumJ + j_lo];
-  if (gated_off(gate, end - begin)) return;
   int2* ring;
   int stride, rmask;
   if (gring) {
@@ -288,8 +282,7 @@ __global__ void __launch_bounds__(kQueueThreads)
 template <int R, bool PACKED, bool GRING, bool QSTAGE, int TB, int LIVE>
 __global__ void __launch_bounds__(kLaneThreads, 4)
     k_lane(const Batch* __restrict__ bd, Score sc, Work w, int cls, int j_lo, int j_hi,
-           int head_id, int rs_log2, void* gring, int mparam, int qs_log2, int cls2,
-           int32_t gate) {
+           int head_id, int rs_log2, void* gring, int mparam, int qs_log2, int cls2) {
   // batch arguments stay in shared memory and are read where used
   __shared__ Batch s_b;
   if (threadIdx.x == 0) s_b = *bd;
@@ -304,7 +297,6 @@ __global__ void __launch_bounds__(kLaneThreads, 4)
     copy_profile(sc, s_prof);
     s_begin[0] = w.seg_begin[cls * kNumJ + j_hi];
     s_end[0] = w.seg_end[cls * kNumJ + j_lo];
-    if (gated_off(gate, s_end[0] - s_begin[0])) s_end[0] = s_begin[0];
     s_begin[1] = cls2 >= 0 ? w.seg_begin[cls2 * kNumJ + j_hi] : 0;
     s_end[1] = cls2 >= 0 ? w.seg_end[cls2 * kNumJ + j_lo] : 0;
   }
@@ -716,7 +708,7 @@ static cudaError_t launch_queue_t(const Batch* b, const Score& sc, const Work& w
   if (e != cudaSuccess) return e;
   kern<<<L.grid, kQueueThreads, smem, stream>>>(b, sc, w, L.cls, L.j_lo, L.j_hi, head_id,
                                                 L.rs_log2, L.global_ring ? gring : nullptr,
-                                                L.slab, L.gate);
+                                                L.slab);
   return cudaGetLastError();
 }
 
@@ -784,9 +776,9 @@ static cudaError_t launch_lane_t(const Batch* b, const Score& sc, const Work& w,
   }
   cudaError_t e = raise_smem_limit(kern, smem);
   if (e != cudaSuccess) return e;
-  kern<<<L.grid, kLaneThreads, smem, stream>>>(b, sc, w, L.cls, L.j_lo, L.j_hi, head_id,
-                                               L.rs_log2, gring, L.mparam, L.j_hi, L.cls2,
-                                               L.gate);
+  const int seg = L.lanes_left ? kLanesLeftSeg : L.cls;
+  kern<<<L.grid, kLaneThreads, smem, stream>>>(b, sc, w, seg, L.j_lo, L.j_hi, head_id,
+                                               L.rs_log2, gring, L.mparam, L.j_hi, L.cls2);
   return cudaGetLastError();
 }
 

@@ -21,6 +21,8 @@ enum PairClass : uint8_t {
   CLS_DONE = 6
 };
 constexpr int kNumClasses = 6;           // classes that need a DP kernel
+// The segments of BAND pairs left to lanes: the buckets of CLS_NEAR it has no pairs in.
+constexpr int kLanesLeftSeg = CLS_NEAR;
 constexpr uint8_t kRest = 0xFF;          // seen by k_diag, class still to be found
 constexpr bool packed_class(int cls) { return cls == CLS_PACKED || cls == CLS_NEAR; }
 // per-bucket flags (Work::jflags)
@@ -64,6 +66,7 @@ constexpr int kNearHalf = 15;
 constexpr int kNearJMax = 9;
 constexpr int kNearMaxQ = (1 << kNearJMax) - 2;
 static_assert(kNearJMax <= kExactJ, "one bin per length");
+static_assert(kNearJMax < kBandNearJMin, "kLanesLeftSeg's buckets are free");
 constexpr int kNearBins = 1 << kNearJMax;
 constexpr int kQueueThreads = 128;       // threads per CTA of the queue kernels
 // Queue-kernel launches per call (heads), at most one a bucket and class: WIDE pairs
@@ -107,9 +110,10 @@ struct Launch {
   int near_hw = 0;           // > 0: on a narrower band of this half width
   int cls2 = -1;             // one-lane engine: then this class's pairs of the same buckets
   bool after_prev = false;   // takes the pairs the launch before it left, on its stream
-  // runs only where its segment holds at least gate pairs, or (negative) fewer than
-  // -gate: two engines for what a narrow band leaves, which only the device knows
-  int32_t gate = 0;
+  // a narrow band launch: from so many pairs left on they go to lanes (0: never), which
+  // only the device knows; and the one-lane launch that takes them then
+  int32_t lanes_from = 0;
+  bool lanes_left = false;
   int P = 1, R = 8;          // lanes per pair, rows per lane-strip (per half when packed)
   int rs_log2 = 0;           // ring entries per group = 1 << rs_log2
   bool global_ring = false;  // ring in a global slab per group instead of shared memory

@@ -48,9 +48,9 @@ int main() {
       const Launch& L = pl.launch[i];
       std::printf("%s{\"engine\": \"%s\", \"cls\": %d, \"cls2\": %d, \"j_lo\": %d, \"j_hi\": %d, \"P\": %d, "
                   "\"R\": %d, \"grid\": %d, \"near_hw\": %d, \"after_prev\": %d, \"global_ring\": %d, "
-                  "\"gate\": %d}",
+                  "\"lanes_from\": %d, \"lanes_left\": %d}",
                   i ? ", " : "", L.band ? "band" : (L.lane ? "lane" : "group"), L.cls, L.cls2, L.j_lo,
-                  L.j_hi, L.P, L.R, L.grid, L.near_hw, (int)L.after_prev, (int)L.global_ring, L.gate);
+                  L.j_hi, L.P, L.R, L.grid, L.near_hw, (int)L.after_prev, (int)L.global_ring, L.lanes_from, (int)L.lanes_left);
     }
     std::printf("], \"flags\": [");
     for (int j = 0; j < kNumJ; ++j) std::printf("%s%d", j ? ", " : "", jf.f[j]);

@@ -116,8 +116,7 @@ def test_every_class_and_bucket_gets_its_launch(plan):
         for (cls, j), v in c["counts"].items():
             runs = [L for L in p["launches"] if not L["near_hw"]
                     and (L["cls"] == cls or L["cls2"] == cls) and L["j_lo"] <= j <= L["j_hi"]]
-            gates = sorted(L["gate"] for L in runs)
-            assert gates in ([0], [-gates[-1], gates[-1]]), (c["sc"], cls, j, runs)
+            assert sorted(L["lanes_left"] for L in runs) in ([0], [0, 1]), (c["sc"], cls, j, runs)
 
 
 def test_what_a_narrow_band_leaves_gets_the_engines_narrow_pairs_take(plan):
@@ -129,14 +128,14 @@ def test_what_a_narrow_band_leaves_gets_the_engines_narrow_pairs_take(plan):
     # a CTA of the group launch for every four pairs, up to the GPU's own number
     narrow, group = few["launches"]
     assert narrow["near_hw"] > 0 and group["engine"] == "group" and group["after_prev"]
-    assert group["P"] == 32 and group["grid"] >= 456 and group["gate"] == 0
+    assert group["P"] == 32 and group["grid"] >= 456 and narrow["lanes_from"] == 0
     # where lanes would take all of them, lanes or groups by the number left
     narrow, group, lane = many["launches"]
     assert (group["engine"], lane["engine"]) == ("group", "lane")
-    assert group["gate"] == -lane["gate"] and 60_000 / 4 <= lane["gate"] <= 60_000 / 2
+    assert lane["lanes_left"] and 60_000 / 4 <= narrow["lanes_from"] <= 60_000 / 2
     # no rings beyond the budget
     assert [L["engine"] for L in tight["launches"]] == ["band", "group"]
-    assert tight["launches"][1]["gate"] == 0 and tight["pool"] <= 64 << 20
+    assert tight["launches"][0]["lanes_from"] == 0 and tight["pool"] <= 64 << 20
 
 
 def test_without_a_buffer_for_what_near_passes_leave(plan):
@@ -146,7 +145,7 @@ def test_without_a_buffer_for_what_near_passes_leave(plan):
         {"sc": ScoringParams(w=9000), "counts": {(BAND, 14): 300}, "near_ok": False}])
     for p in plans:
         assert not p["bad"] and p["near_pairs"] == 0
-        assert not any(L["near_hw"] or L["after_prev"] or L["gate"] for L in p["launches"])
+        assert not any(L["near_hw"] or L["after_prev"] or L["lanes_left"] for L in p["launches"])
     assert plans[1]["launches"][0]["j_hi"] == 14 and plans[1]["launches"][-1]["j_lo"] == 11
     assert plans[2]["launches"][0]["global_ring"]
 
