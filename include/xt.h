@@ -93,7 +93,12 @@ typedef struct xt_ctx xt_ctx;
 /*
  * Create a context on CUDA device `device` (made current for the call).
  * mem_budget_bytes caps the device workspace the context may hold (0 = no
- * cap beyond the device).  *ctx receives the handle; XT_EINVAL on a NULL ctx
+ * cap beyond the device).  A batched call needs 5 bytes a pair (n_pairs rounded
+ * up to a power of two, at least 1024) and about 0.1 MB, plus rings in device
+ * memory where a band's do not fit in shared memory (up to 2 GB; some tens of MB
+ * for short queries) and, with an alphabet other than base codes, the converted
+ * sequences.  4 bytes a pair more let it settle near-matching pairs ahead of the
+ * engines; where a budget does not hold them the engines take all pairs.  *ctx receives the handle; XT_EINVAL on a NULL ctx
  * or a bad device, XT_ECUDA when the device cannot be used.
  */
 xt_status xt_ctx_create(xt_ctx** ctx, int device, size_t mem_budget_bytes);
@@ -105,11 +110,14 @@ xt_status xt_ctx_destroy(xt_ctx* ctx);
 xt_status xt_ctx_sync(xt_ctx* ctx, void* stream);
 
 /*
- * Batched extension (the fast path).  A classify pass validates each pair
- * and sorts the batch into length buckets; persistent kernels then pull pairs
- * from device-side queues, each bucket with its own schedule (pairs per warp,
- * rows per lane, packed 16-bit or 32-bit arithmetic where a per-pair score
- * bound makes it exact).  The call waits on the host for the classify pass
+ * Batched extension (the fast path).  In calls of 4,096 pairs and more a first
+ * pass settles the pairs whose diagonal alone decides.  A classify pass validates
+ * each pair and sorts the batch into length buckets; persistent kernels then pull
+ * pairs from device-side queues, each bucket with its own schedule (lanes or
+ * groups of lanes per pair with rows per lane, or the whole band in registers;
+ * packed 16-bit or 32-bit arithmetic where a per-pair score bound makes it exact),
+ * after a pass over a narrow band where the batch's reads promise that it settles
+ * enough of them.  Results never depend on the engine.  The call waits on the host for the classify pass
  * (a few hundred bytes of bucket counts come back) before it enqueues the
  * extension kernels; those are asynchronous.
  *
@@ -140,7 +148,11 @@ xt_status xt_extend_batch(xt_ctx* ctx, const uint8_t* q_seq, int64_t q_bytes,
  * those counts are on the host; _finish plans and enqueues the extension
  * kernels (waiting for the counts if they are not there yet).  Between
  * _begin and _finish the context holds the call: other calls on it return
- * XT_EBUSY.  xt_extend_batch is _begin followed by _finish.
+ * XT_EBUSY; schedules set meanwhile hold from the next call on.  Results are those
+ * of xt_extend_batch.  _begin reads the lengths, offsets and seed scores only; the
+ * sequences have to be in place on `stream` by _finish.  So the call runs without the
+ * passes that settle near-matching pairs by their sequences before the pairs are
+ * classified, and xt_extend_batch is faster on such batches.
  */
 xt_status xt_extend_batch_begin(xt_ctx* ctx, const uint8_t* q_seq, int64_t q_bytes,
                                 const int64_t* q_off, const int32_t* q_len, const uint8_t* t_seq,
@@ -233,11 +245,12 @@ typedef struct {
 xt_status xt_ctx_set_timing(xt_ctx* ctx, int enable);
 
 /*
- * CUDA graphs (on by default).  The second call with the same scoring,
- * schedule, capacity class (n rounded up to a power of two, at least 1024)
- * and workspace is captured as one graph; later such calls replay it, so a
- * call costs the classify pass, one descriptor-store kernel and one graph
- * launch on the host.
+ * CUDA graphs (on by default).  The extension kernels of the second call with
+ * the same scoring, capacity class (n rounded up to a power of two, at least
+ * 1024), workspace and plan (the engines and grids its bucket counts lead to;
+ * calls of like size share one of a few) are captured as one graph; later such
+ * calls replay it, so a call costs the classify pass, one descriptor-store kernel
+ * and one graph launch on the host.
  * Calls with timing enabled launch directly.  enable = 0 turns capture off.
  * A context's calls must be ordered on the GPU (one stream, or synchronised):
  * they share its workspace.
@@ -270,9 +283,12 @@ xt_status xt_ctx_set_streams(xt_ctx* ctx, int branches);
  * pair's latency on its engine decides), XT_BATCH_LARGE ones to larger
  * buckets, and to small buckets without a small schedule.  A call uses the
  * schedules set for its own scoring's w and the built-in rule for buckets
- * without one (one lane per pair where the bucket is large enough: 8192
- * pairs for queries of 63..510 bases, 32768 above; otherwise enough lanes
- * per pair to fill the GPU).  P = 0 removes a bucket's
+ * without one: one lane per pair where the bucket is large enough (8192 pairs
+ * for queries of 63..126 bases, about 16384 x 201 / (2w+1) up to 510, 32768
+ * above); smaller buckets, and pairs whose scores need more than a packed lane
+ * has, keep the whole band in registers (the band engine: queries of 127 bases
+ * and longer, bands of up to 1,024 diagonals); what it does not take runs on
+ * enough lanes per pair to fill the GPU.  P = 0 removes a bucket's
  * schedule.  XT_EINVAL if (P, R) does not exist or its band ring does not
  * fit on this device.  Results never depend on the schedule.
  * xt_ctx_set_bucket_schedule sets both classes.

@@ -592,10 +592,10 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
                           std::max(est_cells, 1.0);
       int want = 4;  // two-lane groups measured slower than four on every call size
       while (want < 32 && want < need) want *= 2;
-      // short queries: 8 rows a lane for as many rows as the bucket's longest
-      // query has, one chunk of them (32 lanes idle half: 5,000 pairs of 64 bases
-      // 109 us a call, 94 so)
-      if (jj <= kGroupMaxJ) want = std::max(4, 1 << (jj - 3));
+      // queries of 63 to 126 bases (shorter ones have lanes): 8 rows a lane for as many
+      // rows as the longest has, one chunk of them (32 lanes idle half: 5,000 pairs of
+      // 64 bases 109 us a call, 94 so)
+      if (jj == kGroupMaxJ) want = 16;
       for (int q = want; q >= 2 && *P == 0; q /= 2) {
         const int l = queue_ring_log2(jj, sc.w, q, 8);
         if (l <= kQueueRsCapLog2 && queue_smem_bytes(q, l) <= (size_t)ctx->smem_optin / 2 - 1024) {
@@ -1029,9 +1029,8 @@ uint64_t plan_signature(const Plan& pl) {
 
 // The first half of a call: checks, workspace, descriptor, and for the
 // batched path the classify pass and the copy of its bucket counts.  The
-// call's state waits in ctx->pending for run_finish.  early: the caller may
-// still be filling the sequence buffers until _finish, so only the lengths are
-// read here (no diagonal pass).
+// call's state waits in ctx->pending for run_finish.  early: a two-step call, whose
+// sequences need not be there before _finish (no diagonal pass).
 xt_status run_begin(xt_ctx* ctx, bool plain, bool early, const uint8_t* q_seq, int64_t q_bytes,
                     const int64_t* q_off, const int32_t* q_len, const uint8_t* t_seq,
                     int64_t t_bytes, const int64_t* t_off, const int32_t* t_len,

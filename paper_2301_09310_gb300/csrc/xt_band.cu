@@ -30,8 +30,9 @@
 // instruction with the tag as an immediate): a multiply-add needed the tag in
 // a register and took 378 ms.  With few slots and one warp per scheduler a row's
 // dependent instructions (330 with 8 slots) bound it, 0.57 us: 1,000 pairs of 100
-// bases 85 us (so queries that short stay on the group engine).  A narrow band first: 5,000 pairs of 1,024 bases, w = 1,024, 4.90 ->
-// 1.46 ms a call on 512 diagonals.
+// bases 85 us (so queries that short stay on the group engine).  A narrow band
+// first: 5,000 pairs of 1,024 bases, w = 1,024, 4.90 -> 1.43 ms a call on 512
+// diagonals.
 #include <algorithm>
 
 #include "xt_kernels.cuh"
@@ -544,7 +545,8 @@ bool band_scoring(const Score& sc, int32_t match, int P) {
   return base_age(P) * (fall + match) + fall + match + 2 <= (32767 >> kKeyBits) - 1;
 }
 
-// A launch with fewer warps than this leaves schedulers idle.
+// A launch with fewer warps than this leaves schedulers idle (four on each of 152 SMs;
+// one figure for all parts, so that a pair's engine does not depend on the part).
 constexpr int64_t kBandWarps = 608;
 
 }  // namespace

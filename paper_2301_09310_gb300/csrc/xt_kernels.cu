@@ -13,12 +13,11 @@ namespace xt {
 
 // ---------------------------------------------------------------- classify
 // Validates every pair, writes the results of invalid and degenerate pairs
-// directly, and assigns the others a class and a bin by
-// query length, counted for the ordering pass.  A block takes one or
-// kOrdPer times kOrdThreads consecutive pairs and counts them in a shared-memory histogram
-// of every (class, length bin), then adds its non-zero bins to the
-// global counts: a batch's pairs fall into a few hundred bins, and one global
-// atomic per pair on those bins serialised the pass.
+// directly, and assigns the others a class and a bin by query length, counted for
+// the ordering pass.  A block takes one or kOrdPer times kOrdThreads consecutive
+// pairs and counts them in a shared-memory histogram of every (class, length bin),
+// then adds its non-zero bins to the global counts: a batch's pairs fall into a few
+// hundred bins, and one global atomic per pair on those bins serialised the pass.
 constexpr int kOrdThreads = 1024;
 // pairs per thread: one while that gives fewer blocks than two per SM (a block's
 // passes over the bins cost more than its pairs, but the blocks run at once:
@@ -103,10 +102,9 @@ __global__ void __launch_bounds__(kOrdThreads) k_classify(const Batch* __restric
 }
 
 // Exclusive scan of the bin counts in queue order: per class, from the longest
-// length down (longest work first).  One block, each thread a run of
-// kScanPer counters read and written as vectors; the scan is on every call's
-// critical path (20 us with 26,112
-// counters read one by one, 4 us so).
+// length down (longest work first).  One block, each thread a run of kScanPer
+// counters read and written as vectors; the scan is on every call's critical path
+// (20 us with 26,112 counters read one by one, 4 us so).
 constexpr int kScanThreads = 1024;
 constexpr int kScanPer = 8;
 static_assert(kClassBins % kScanPer == 0 && kNumBuckets <= kScanThreads * kScanPer,
