@@ -245,6 +245,9 @@ __global__ void __launch_bounds__(kQueueThreads)
   const unsigned gmask = (P == 32) ? 0xffffffffu : (((1u << P) - 1u) << (lane - p));
   const int32_t begin = w.seg_begin[cls * kNumJ + j_hi];
   const int32_t end = w.seg_end[cls * kNumJ + j_lo];
+  // a follow-up of a narrow band has CTAs for all pairs and may have few: those take the
+  // first CTAs, one per SM, where warps of any CTA had crowded on some schedulers
+  if ((int64_t)blockIdx.x * G >= end - begin) return;
   int2* ring;
   int stride, rmask;
   if (gring) {
