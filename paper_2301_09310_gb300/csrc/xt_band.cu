@@ -445,14 +445,16 @@ __global__ void __launch_bounds__(kBandThreads, band_blocks(K))
       if (NEAR && p == P - 1 && i >= 0) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          // (1') bounds the loss on the rows up to the last hw + 1.  A pair that loses
-          // so fast that it would come to twice that (from row 255 on half as much
-          // again) is left at once: long reads with 8% errors fail some way down their
-          // thousands of rows anyway (1,000 of them, w = 512, 28.5 -> 17.4 ms with the CTAs for what is left)
+          // (1') bounds the loss on the rows up to the last hw + 1.  A pair that is a
+          // quarter of that ahead of losing it evenly is left at once: long reads with
+          // 8% errors fail some way down their thousands of rows anyway (1,000 of them,
+          // w = 512, 28.5 -> 17.4 ms with the CTAs for what is left).  A few errors close
+          // together are no reason: one pair left of a batch costs the group engine's
+          // whole pass (1,000 of 3,800 bases with 2% errors 19.3 ms where one and a half
+          // times the even rate from row 255 on was, 8.4 ms so)
           const int32_t rows = ql[h] - hw - 1, seen = i - 7;  // (was_best is of eight rows ago)
           const float lost = h0[h] + match * seen - was_best[h];
-          const bool fast = i >= 127 && i < rows &&
-                            lost * rows > (i < 255 ? 2.0f : 1.5f) * (alpha - beta + beta * (hw + 1)) * seen;
+          const bool fast = i < rows && lost * rows > (alpha - beta + beta * (hw + 1)) * (seen + 0.25f * rows);
           if (act[h] && (fast || !near_row_ok(i, ql[h], h0[h], match, hw, was_best[h], sc))) leave(h);
           was_best[h] = half(best2, h);
         }
