@@ -230,9 +230,10 @@ xt_status xt_ctx_set_schedule(xt_ctx* ctx, int P, int R);
  * Launch accounting and DP timing (measurement aid).  With timing enabled,
  * every extension call records CUDA event pairs on its stream around its DP
  * (extension) kernels: around the pass that settles pairs on their diagonal
- * before the pairs are classified, and around the kernels after.  xt_ctx_stats waits for the pending events, sums their
- * durations into dp_ms, reports the number of calls and kernel launches since
- * the previous xt_ctx_stats, and resets those counters.
+ * before the pairs are classified, and around the kernels after.  xt_ctx_stats
+ * waits for the pending events, sums their durations into dp_ms, reports the
+ * number of calls and kernel launches since the previous xt_ctx_stats, and
+ * resets those counters.
  */
 typedef struct {
   int32_t calls;        /* extension calls since the last query */

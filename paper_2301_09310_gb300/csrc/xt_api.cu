@@ -622,11 +622,10 @@ void plan_counts(xt_ctx* ctx, const Score& sc, int32_t (*cnt)[kNumJ], int32_t ho
       // NARROW pairs would take, for those it leaves
       const bool narrow_first = cls == CLS_BAND && !band_ok;
       const BucketSched* const ts = tuned(ctx, sc.w, jj);
-      // queries of up to 510 bases, half a wave of lanes or more (a third, of up to 126
-      // bases where a warp is taken), under bands that take
-      // the band engine a whole warp a pair or are three times as wide as the bucket's
-      // queries: lanes, in 32 bits, sweep the columns there are, the band engine all
-      // diagonals (300k reads, match 5, on bands / on lanes: 100 bases, w = 200 3.62 /
+      // queries of up to 510 bases, half a wave of lanes or more (a third for queries of
+      // up to 126 bases where the band takes a warp), under bands that take the band
+      // engine a whole warp a pair or are three times as wide as the bucket's queries:
+      // lanes, in 32 bits, sweep the columns there are, the band engine all diagonals (300k reads, match 5, on bands / on lanes: 100 bases, w = 200 3.62 /
       // 2.15 ms, w = 400 8.70 / 2.51; 150 bases, w = 200 6.45 / 7.3, w = 400 14.2 / 7.3)
       const int64_t diagonals = 2 * (int64_t)sc.w + 1;
       const int32_t some = kLaneSlots / (diagonals > 512 && jj <= kGroupMaxJ ? 3 : 2);
