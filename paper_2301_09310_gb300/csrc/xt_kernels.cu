@@ -246,8 +246,10 @@ __global__ void __launch_bounds__(kQueueThreads)
   const int32_t begin = w.seg_begin[cls * kNumJ + j_hi];
   const int32_t end = w.seg_end[cls * kNumJ + j_lo];
   // a follow-up of a narrow band has CTAs for all pairs and may have few: those take the
-  // first CTAs, one per SM, where warps of any CTA had crowded on some schedulers
-  if ((int64_t)blockIdx.x * G >= end - begin) return;
+  // first CTAs, one per SM, where warps of any CTA had crowded on some schedulers (beside
+  // other launches the pairs of a whole bucket are better spread over all CTAs: 3,865
+  // reads of 150 bases 240 us a call, 325 on the first ones)
+  if (cls == CLS_BAND && (int64_t)blockIdx.x * G >= end - begin) return;
   int2* ring;
   int stride, rmask;
   if (gring) {
